@@ -65,7 +65,9 @@ typedef enum {
 } smx_status;
 
 /* Arithmetic of the Newton-Schulz bulk phase (Eq. 13 iteration).
- *  SMX_FP64   : FP64 on the CUDA cores ("plain" form).
+ *  SMX_FP64   : 64-bit arithmetic ("plain" form): products by error-free slices of eight bits on
+ *               the tensor cores (the sums are exact, the result as accurate as FP64
+ *               multiply-adds), 64-bit integers between them.
  *  SMX_FP16X3 : tcgen05 tensor cores, FP16 operands split as hi + lo with three
  *               products (hi*hi + hi*lo + lo*hi) per step and FP32 accumulation
  *               in tensor memory; about 22 significant bits per operand.
@@ -203,7 +205,7 @@ smx_status smx_set_electron_count(smx_ctx* ctx, double n_e, int32_t max_steps, d
 
 /* Arithmetic of the Newton-Schulz iteration (Eq. 13; Section 3's low-precision
  * units).  fp64_final_iters (0..4): when bulk != SMX_FP64, that many plain
- * Newton-Schulz steps in FP64 (CUDA cores) follow the bulk phase's stopping
+ * Newton-Schulz steps in 64-bit arithmetic follow the bulk phase's stopping
  * rule, on its last iterate, before the owner columns are scattered (the
  * density matrix only; ignored for SMX_FP64).  Note that they restore
  * X^2 = I but not the occupied subspace a single-pass bulk phase has rotated
@@ -425,17 +427,15 @@ smx_status smx_get_submatrix_info(smx_ctx* ctx, int32_t* dims, int32_t* iters, d
  * not enter the driver's allocator (cudaMalloc/cudaFree can synchronise the
  * device).
  * Computes D = 1/2 (I - sign(H - mu I)) of one dense symmetric H by FP64
- * Newton-Schulz iteration with a Gershgorin scaling (Eq. 13 and Eq. 14 with
- * S = I on a single dense matrix; one CTA; same arithmetic as the FP64 form
- * of smx_build_density).
+ * Newton-Schulz iteration (Eq. 13 and Eq. 14 with S = I on a single dense
+ * matrix; one CTA; the same iteration as the FP64 form of smx_build_density).
  *  h_dev       : device double[n*n], row-major, symmetric (read only).
  *  n           : 1 <= n <= 256; larger n returns SMX_ERR_ARG.
  *  mu          : finite chemical potential.
  *  d_dev       : device double[n*n], row-major, receives D (caller-owned).
  *  cuda_stream : stream to run on (NULL = legacy default stream).
- * Work matrices live in one fixed __device__ array of 3*256*256 + 4 doubles
- * (about 1.5 MiB) that every GPU which loads the library keeps until the
- * process exits.  The first call on a device (and the first after a device
+ * Work matrices live in one fixed __device__ array of about 2.8 MiB that every
+ * GPU which loads the library keeps until the process exits.  The first call on a device (and the first after a device
  * reset) looks up that array's device address (cudaGetSymbolAddress), so
  * make the first call on each device before any stream capture.  All calls
  * share the array and it keeps the last call's contents (every call

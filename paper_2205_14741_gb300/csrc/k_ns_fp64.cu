@@ -1,228 +1,628 @@
-// Newton-Schulz sign iteration in FP64 on the CUDA cores (the plain form).
+// Newton-Schulz sign iteration in 64-bit arithmetic (the plain form), and the function forms.
 //
 // Eq. 13 defines sign(A) = A (A^2)^(-1/2).  The iteration
-//     X_{k+1} = 1/2 X_k (3 I - X_k^2),   X_0 = (T_j - mu I) / b_j,
-// converges to sign(T_j - mu I) when every eigenvalue of X_0 lies in
-// (-sqrt 3, 0) u (0, sqrt 3); b_j >= spectral radius guarantees |lambda| <= 1.
-// Each step is two products: Y = 3/2 I - 1/2 X X (which also yields the
-// residual ||X^2 - I||_F) and X' = X Y.  Stopping rule: after the step whose
-// residual is <= tau (the next residual is ~0.75 tau^2).
+//     X_{k+1} = 1/2 X_k (3 I - X_k^2) = X_k + 1/2 X_k W_k,   W_k = I - X_k^2,
+// converges to sign(T_j - mu I) when every eigenvalue of X_0 (a multiple of T_j - mu I) lies in
+// (-sqrt 3, 0) u (0, sqrt 3).  Each step is two symmetric products; the first also yields the
+// residual ||X^2 - I||_F.  Stopping rule: after the step whose residual is <= tau (the next
+// residual is ~0.75 tau^2).
 //
-// One CTA per submatrix; FP64 throughput on this part is about 1.2 TFLOP/s
-// for the whole GPU, so the kernel is bound by the FP64 pipes and a plain
-// shared-memory tiled product with 4x4 register blocking suffices.
+// The products run on the tensor cores by error-free slices (smx_slices.cuh), and everything
+// between them is 64-bit integer arithmetic in units of 2^-62: GB300's FP64 units take about 16
+// cycles per warp instruction, so one FP64 operation per matrix entry costs as much as a quarter of
+// a product (n = 158).  One persistent CTA per SM takes submatrices largest first and keeps an
+// iterate, one product and the operands' digits in a slot of global memory that stays in L2.
 #include "smx_finish.cuh"
 #include "smx_kernels.h"
+#include "smx_slices.cuh"
 
 namespace smx {
 
 namespace {
 
-constexpr int kTile = 64;
-constexpr int kKc = 16;
+// The matrices of one submatrix in its CTA's slot: k x k integers (units of 2^-62) and digit planes.
+struct SliceJob {
+    int n, k;  // dimension, and rounded up to 32 (rows and columns past n are zero)
+    int64_t* M[kFp64Mats];
+    uint8_t* P[kFp64Planes];
+};
 
-// C = A B (n x n, row-major, leading dimension ld).  mode 1 writes
-// dg I + cf A B (3/2 I - 1/2 A B by default) and returns this thread's share of
-// ||A B - I||_F^2; mode 2 writes oscale * A B.
-__device__ double gemm_fp64(const double* __restrict__ A, const double* __restrict__ B, double* __restrict__ C, int n,
-                            int ld, int mode, double (*As)[kTile + 1], double (*Bs)[kTile + 1], double oscale = 1.0,
-                            double cf = -0.5, double dg = 1.5) {
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    double r2 = 0.0;
-    for (int r0 = 0; r0 < n; r0 += kTile) {
-        for (int c0 = 0; c0 < n; c0 += kTile) {
-            double acc[4][4];
+// Scalars that one thread forms in FP64 for the CTA.
+struct SliceScalars {
+    int job, next;
+    int e;
+    int bad;
+    int stop;          // the schedule's factor allows this step to be the last
+    uint64_t f1, f2;   // the step's factor a and a^2 (fixed_factor), 0 for a plain step
+    double lsch;       // lower end of the interval the scaled schedule assumes (1: plain steps)
+    unsigned long long u[kSliceWarps];
+    double d[kSliceWarps];
+};
+
+__device__ __forceinline__ void slice_job(SliceJob& jb, uint8_t* slot, int n, int kmax, int mats) {
+    jb.n = n;
+    jb.k = (n + 31) & ~31;
+    const int64_t mb = static_cast<int64_t>(kmax) * kmax * 8;
+    for (int i = 0; i < kFp64Mats; ++i) jb.M[i] = reinterpret_cast<int64_t*>(slot + i * mb);
+    for (int i = 0; i < kFp64Planes; ++i) jb.P[i] = slot + mats * mb + i * slice_bytes(kmax);
+}
+
+__device__ __forceinline__ unsigned long long cta_max_u64(unsigned long long v, SliceScalars* ss) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-            for (int k0 = 0; k0 < n; k0 += kKc) {
-                for (int e = tid; e < kTile * kKc; e += 256) {
-                    const int rr = e / kKc, kk = e - rr * kKc;
-                    const int row = r0 + rr, col = k0 + kk;
-                    As[kk][rr] = (row < n && col < n) ? A[static_cast<int64_t>(row) * ld + col] : 0.0;
-                }
-                for (int e = tid; e < kTile * kKc; e += 256) {
-                    const int kk = e / kTile, cc = e - kk * kTile;
-                    const int row = k0 + kk, col = c0 + cc;
-                    Bs[kk][cc] = (row < n && col < n) ? B[static_cast<int64_t>(row) * ld + col] : 0.0;
-                }
-                __syncthreads();
-#pragma unroll
-                for (int kk = 0; kk < kKc; ++kk) {
-                    double a[4], b[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-                }
-                __syncthreads();
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int row = r0 + ty * 4 + i;
-                if (row >= n) continue;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int col = c0 + tx * 4 + j;
-                    if (col >= n) continue;
-                    const double v = acc[i][j];
-                    if (mode == 1) {
-                        const double dlt = (row == col) ? 1.0 : 0.0;
-                        C[static_cast<int64_t>(row) * ld + col] = dg * dlt + cf * v;
-                        r2 += (v - dlt) * (v - dlt);
-                    } else {
-                        C[static_cast<int64_t>(row) * ld + col] = oscale * v;
-                    }
-                }
-            }
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = w > v ? w : v;
     }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) ss->u[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0;
+    for (int w = 0; w < kSliceWarps; ++w) v = ss->u[w] > v ? ss->u[w] : v;
+    return v;
+}
+
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__device__ __forceinline__ uint64_t abs_fixed(int64_t x) { return static_cast<uint64_t>(x < 0 ? -x : x); }
+
+// What the following products keep: the weights up to 8 or 9, and the chunks of one accumulation.
+__device__ __forceinline__ void set_accumulation(SliceShared* sh, int weights, int kpart) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sh->weights = weights;
+        sh->kpart = kpart;
+    }
+    __syncthreads();
+}
+
+// The bits of entries (r, c .. c + 7) of a symmetric matrix of doubles (read along its rows), zero past n.
+__device__ __forceinline__ void load_bits(const double* __restrict__ src, int ld, int n, int r, int c, int64_t (&v)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = r < n && c + i < n ? __double_as_longlong(src[static_cast<int64_t>(c + i) * ld + r]) : 0;
+}
+
+// The elementwise passes between products (each a function of its own, so that its registers are
+// its own: what the callers keep across it lies on the stack, not what its loop works on).
+
+// The symmetric n x n matrix src - mu I, times f 2^-e, into M and the planes (see to_fixed).
+__device__ __noinline__ bool pass_source(const double* __restrict__ src, int ld, double mu, int e, uint64_t f, int64_t* M, uint8_t* planes, int n,
+                                         int k) {
+    bool bad = false;
+    slice_pass<1>(k, k, planes, [&](int r, int c, int64_t (&v)[1][8]) { load_bits(src, ld, n, r, c, v[0]); },
+                  [&](int r, int c, const int64_t (&v)[1][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i) {
+                          double x = __longlong_as_double(v[0][i]);
+                          if (mu != 0.0 && r == c + i && r < n) x -= mu;
+                          q[i] = to_fixed(x, e, f, bad);
+                      }
+                      st8(M, k, r, c, q);
+                  });
+    return bad;
+}
+
+// W = I - f S 2^up (f = 0: 1) to its digits; returns this thread's share of ||I - S 2^up||_F^2 in units of 2^-76.
+__device__ __noinline__ float pass_residual(const int64_t* S, uint8_t* planes, int n, int k, int up, uint64_t f) {
+    float r2 = 0.0f;
+    slice_pass<1>(k, k, planes, [&](int r, int c, int64_t (&v)[1][8]) { ld8(S, k, r, c, v[0]); },
+                  [&](int r, int c, const int64_t (&v)[1][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i) {
+                          const int64_t one = r == c + i && r < n ? kFixedOne : 0, s = v[0][i] << up;
+                          const float d = fixed_float(one - s);
+                          r2 = fmaf(d, d, r2);
+                          q[i] = one - (f ? fixed_mul(s, f) : s);
+                      }
+                  });
     return r2;
 }
 
-// The sign iteration of the Eq. 12 block matrix [[0, A], [I, 0]] written per block (the
-// coupled Newton-Schulz iteration): T = 3/2 I - 1/2 Z Y, Y <- Y T, Z <- T Z from Y = A (in Yb,
-// eigenvalues in (0, 1]) and Z = I (set here); Y -> A^1/2, Z -> A^-1/2.  The residual
-// ||Z Y - I||_F comes with the first product; the stopping rule is the sign iteration's.  On
-// return Yb and Zb point to the final iterates; the four n x n buffers rotate.  Returns the
-// number of steps.
-__device__ int coupled_ns(double*& Yb, double*& Zb, double*& Tb, double*& Nb, int n, int ld, int max_iter, double tau,
-                          double (*As)[kTile + 1], double (*Bs)[kTile + 1], double* scratch, bool& conv, bool& bad) {
-    for (int r = threadIdx.x / 32; r < n; r += 8)
-        for (int c = threadIdx.x & 31; c < n; c += 32) Zb[static_cast<int64_t>(r) * ld + c] = r == c ? 1.0 : 0.0;
+// X <- f (X + 1/2 S) (f = 0: 1), and its digits.
+__device__ __noinline__ void pass_update(int64_t* X, const int64_t* S, uint8_t* planes, int k, uint64_t f) {
+    slice_pass<2>(k, k, planes,
+                  [&](int r, int c, int64_t (&v)[2][8]) {
+                      ld8(X, k, r, c, v[0]);
+                      ld8(S, k, r, c, v[1]);
+                  },
+                  [&](int r, int c, const int64_t (&v)[2][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i) {
+                          q[i] = v[0][i] + (v[1][i] >> 1);
+                          if (f) q[i] = fixed_mul(q[i], f);
+                      }
+                      st8(X, k, r, c, q);
+                  });
+}
+
+// Z <- 3/2 I - 1/2 (Y - 1/2 S)
+__device__ __noinline__ void pass_first_root(const int64_t* Y, const int64_t* S, int64_t* Z, int n, int k) {
+    slice_pass<2>(k, k, nullptr,
+                  [&](int r, int c, int64_t (&v)[2][8]) {
+                      ld8(Y, k, r, c, v[0]);
+                      ld8(S, k, r, c, v[1]);
+                  },
+                  [&](int r, int c, const int64_t (&v)[2][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i)
+                          q[i] = (r == c + i && r < n ? kFixedOne + (kFixedOne >> 1) : 0) - ((v[0][i] - (v[1][i] >> 1)) >> 1);
+                      st8(Z, k, r, c, q);
+                  });
+}
+
+// diag I +- f S 2^shift (f = 0: 1) to its digits, and to out when given.
+__device__ __noinline__ void pass_affine(const int64_t* S, int64_t* out, uint8_t* planes, int n, int k, int64_t diag, bool minus, int shift,
+                                         uint64_t f) {
+    slice_pass<1>(k, k, planes, [&](int r, int c, int64_t (&v)[1][8]) { ld8(S, k, r, c, v[0]); },
+                  [&](int r, int c, const int64_t (&v)[1][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i) {
+                          // (modulo 2^64: 2 E of the Fermi form may be 2, one unit past the range, before I - 2 E)
+                          int64_t x = shift >= 0 ? static_cast<int64_t>(static_cast<uint64_t>(v[0][i]) << shift) : v[0][i] >> min(-shift, 63);
+                          if (f) x = fixed_mul(x, f);
+                          const uint64_t d = r == c + i && r < n ? static_cast<uint64_t>(diag) : 0u;
+                          q[i] = static_cast<int64_t>(minus ? d - static_cast<uint64_t>(x) : d + static_cast<uint64_t>(x));
+                      }
+                      if (out) st8(out, k, r, c, q);
+                  });
+}
+
+// T <- (a T + b S) 2^up (a = 0: 1), and its digits.
+__device__ __noinline__ void pass_mix(int64_t* T, const int64_t* S, uint8_t* planes, int k, uint64_t a, uint64_t b, int up) {
+    slice_pass<2>(k, k, planes,
+                  [&](int r, int c, int64_t (&v)[2][8]) {
+                      ld8(T, k, r, c, v[0]);
+                      ld8(S, k, r, c, v[1]);
+                  },
+                  [&](int r, int c, const int64_t (&v)[2][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i) q[i] = ((a ? fixed_mul(v[0][i], a) : v[0][i]) + fixed_mul(v[1][i], b)) << up;
+                      st8(T, k, r, c, q);
+                  });
+}
+
+// Digits of the transpose of columns c0 .. c0 + m - 1 of the k-row matrix A - B (B null: A; B's columns from
+// 0), halved or shifted right: rows of an operand of `rows` x k.
+__device__ __noinline__ void pass_transposed(const int64_t* A, const int64_t* B, int c0, int m, uint8_t* planes, int rows, int k, int shift) {
+    slice_pass<1>(rows, k, planes, [&](int r, int c, int64_t (&v)[1][8]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            v[0][i] = r < m ? (A[mat_at(k, c + i, c0 + r)] - (B ? B[mat_at(k, c + i, r)] : 0)) >> shift : 0;
+    }, [](int, int, const int64_t (&v)[1][8], int64_t (&q)[8]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) q[i] = v[0][i];
+    });
+}
+
+// The symmetric source matrix A = src - mu I (n x n, leading dimension ld) in fixed point, A 2^-e, into M and
+// the planes P.  The power of two brings the largest 2-norm of a row into (1/2, 1] (so that the
+// products are exact and use all digits); without_scale keeps e = 0.  bound: no entry is larger (0:
+// not known).  Returns e; a value that is not finite sets ss->bad.
+__device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, double mu, double bound, const SliceJob& jb, int64_t* M, uint8_t* P,
+                          bool without_scale, SliceShared* sh, SliceScalars* ss) {
+    const int n = jb.n, k = jb.k, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto entry = [&](int r, int c) -> double {
+        const double v = src[static_cast<int64_t>(r) * ld + c];
+        return r == c && mu != 0.0 ? v - mu : v;
+    };
+    int e = 0;
+    if (threadIdx.x == 0) ss->bad = 0;
+    if (!without_scale) {
+        uint32_t top = static_cast<uint32_t>(__double2hiint(bound)) & 0x7fffffffu;
+        if (top == 0) {  // high words order like the magnitudes
+            for (int r = warp; r < n; r += kSliceWarps)
+#pragma unroll 4
+                for (int c = lane; c < n; c += 32) top = max(top, static_cast<uint32_t>(__double2hiint(entry(r, c))) & 0x7fffffffu);
+            top = static_cast<uint32_t>(cta_max_u64(top, ss));
+        }
+        const int ex = static_cast<int>(top >> 20);
+        if (ex == 0x7ff) {
+            __syncthreads();
+            if (threadIdx.x == 0) ss->bad = 1;
+            __syncthreads();
+            return 0;
+        }
+        const int e0 = ex - 1022;  // |A| < 2^e0
+        auto scaled = [&](double v) -> float {  // v 2^-e0, 0 below 2^-122
+            const int hi = __double2hiint(v), ef = ((hi >> 20) & 0x7ff) - e0;
+            return ef > 900 ? d2f_rn(__hiloint2double((hi & 0x800fffff) | (ef << 20), __double2loint(v))) : 0.0f;
+        };
+        float worst = 0.0f;
+        for (int r = 2 * warp; r < n; r += 2 * kSliceWarps) {
+            const int r1 = min(r + 1, n - 1);
+            float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll 4
+            for (int c = lane; c < n; c += 32) {
+                const float x = scaled(entry(r, c)), y = scaled(entry(r1, c));
+                a0 = fmaf(x, x, a0);
+                a1 = fmaf(y, y, a1);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+                a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+            }
+            worst = fmaxf(worst, fmaxf(a0, a1));
+        }
+        worst = cta_max(worst, sh);
+        e = e0 + (worst > 0.0f ? static_cast<int>(ceilf(0.5f * log2f(worst * 1.001f))) : 0);
+    }
     __syncthreads();
-    int done = 0;
+    const bool bad = pass_source(src, ld, mu, e, 0, M, P, n, k);
+    if (bad) ss->bad = 1;
+    __syncthreads();
+    return e;
+}
+
+// The learned bound of a submatrix for sign_steps: the initial scaling b_j of X0 = A / b_j, the
+// predicted smallest |eigenvalue| of A / b_j (negative: none) and the fallback counter.
+struct SignModel {
+    double b, dhat;
+    int* fallbacks;
+};
+// What the first product gives: the largest row sum of |X0^2| and the factor c of the first step.
+struct SignBound {
+    double rmax, c;
+};
+
+// For the symmetric non-negative-bounded Y = S: the largest row sum of |Y| (every thread), and the smaller
+// max_r (|Y| w)_r / w_r of two power steps from the row sums (thread 0; 0 without any).
+__device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceShared* sh, SliceScalars* ss, double& row_max, double& best) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned long long* wv = reinterpret_cast<unsigned long long*>(sh->smem);  // row sums, then weights
+    unsigned long long* av = wv + k;
+    // row sums of |Y| in units of 2^-50
+    unsigned long long m = 0;
+    for (int r = 2 * warp; r < n; r += 2 * kSliceWarps) {  // Y is symmetric: two columns at a time
+        const longlong2* y = reinterpret_cast<const longlong2*>(S) + static_cast<int64_t>(r >> 1) * k;
+        unsigned long long a0 = 0, a1 = 0;
+#pragma unroll 4
+        for (int c = lane; c < k; c += 32) {
+            const longlong2 v = y[c];
+            a0 += abs_fixed(v.x) >> 12;
+            a1 += abs_fixed(v.y) >> 12;
+        }
+        a0 = warp_sum_u64(a0);
+        a1 = warp_sum_u64(a1);
+        if (lane == 0) {
+            wv[r] = a0;
+            wv[r + 1] = a1;
+        }
+        m = max(m, max(a0, a1));
+    }
+    m = cta_max_u64(m, ss);
+    row_max = static_cast<double>(m) * 0x1p-50;
+    best = 0.0;  // of the power steps (every row's quotient; 0: none)
+    for (int pass = 0; pass < 2 && m > 0; ++pass) {
+        // weights: any multiple of w serves; the largest into [2^62, 2^63), at least one unit
+        const int up = __clzll(static_cast<long long>(m)) - 1;
+        for (int r = tid; r < k; r += kSliceThreads) {
+            const unsigned long long w = r < n ? wv[r] : 0ull;
+            wv[r] = max(up >= 0 ? w << up : w >> -up, 1ull);
+        }
+        __syncthreads();
+        m = 0;
+        for (int r = 2 * warp; r < n; r += 2 * kSliceWarps) {
+            const longlong2* y = reinterpret_cast<const longlong2*>(S) + static_cast<int64_t>(r >> 1) * k;
+            unsigned long long a0 = 0, a1 = 0;  // (|Y| w)_r, w in units of 2^-63, in units of 2^-51
+#pragma unroll 4
+            for (int c = lane; c < k; c += 32) {  // (zero past n)
+                const longlong2 v = y[c];
+                const unsigned long long w = wv[c] << 1;
+                a0 += __umul64hi(abs_fixed(v.x) << 1, w) >> 12;
+                a1 += __umul64hi(abs_fixed(v.y) << 1, w) >> 12;
+            }
+            a0 = warp_sum_u64(a0);
+            a1 = warp_sum_u64(a1);
+            if (lane == 0) {
+                av[r] = a0;
+                av[r + 1] = a1;
+            }
+            m = max(m, max(a0, a1));
+        }
+        m = cta_max_u64(m, ss);
+        double q = 0.0;
+        if (32 * warp < n) {  // FP64 divisions only on the warps that hold rows
+            for (int r = tid; r < n; r += kSliceThreads) q = fmax(q, static_cast<double>(av[r]) / static_cast<double>(wv[r]));
+            q = warp_max(q);
+        }
+        __syncthreads();
+        if (lane == 0) ss->d[warp] = q;
+        for (int r = tid; r < n; r += kSliceThreads) wv[r] = av[r];
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < kSliceWarps; ++w)
+                if (ss->d[w] > q) q = ss->d[w];
+            q *= 0x1p12;
+            best = pass == 0 ? q : fmin(best, q);
+        }
+    }
+    __syncthreads();
+    fence_proxy_async_smem();  // the stages are the copies' again
+}
+
+// Newton-Schulz steps on X = M[0] (digits in P[0]; A = X 2^e) until the residual is <= tau (returns
+// the number of steps; conv, bad).  plain_steps > 0: exactly that many plain steps.  M[1] takes the
+// products, P[1] the digits of W.
+//
+// The first product bounds the spectrum (as in the tensor-core kernel): with Y = X0^2, rho(X0)^2 =
+// rho(Y) <= rho(|Y|) <= max_r (|Y| w)_r / w_r for any positive w (Collatz-Wielandt): w = 1 (the
+// largest row sum) and two power steps of |Y| from it, in integers; the iteration continues from
+// c X0, c = 1.2 / s.  A scaled step X' = p(a X), p(x) = x (3 - x^2) / 2, is a (X + 1/2 X W), W =
+// I - a^2 X^2.
+__device__ int sign_steps(SliceShared* sh, const SliceJob& jb, int e, int max_iter, float tau, int plain_steps, const SignModel* model,
+                          SignBound* bound_out, SliceScalars* ss, bool& conv, bool& bad) {
+    const int n = jb.n, k = jb.k, tid = threadIdx.x;
+    int64_t *X = jb.M[0], *S = jb.M[1];
     conv = bad = false;
-    for (int it = 0; it < max_iter; ++it) {
-        double r2 = gemm_fp64(Zb, Yb, Tb, n, ld, 1, As, Bs);  // T = 3/2 I - 1/2 Z Y
-        r2 = block_sum(r2, scratch);
-        gemm_fp64(Yb, Tb, Nb, n, ld, 2, As, Bs);  // Y' = Y T
+    int done = 0;
+    if (tid == 0) ss->lsch = 1.0;
+    const int limit = plain_steps > 0 ? plain_steps : max_iter;
+    for (int it = 0; it < limit; ++it) {
+        slice_product(sh, jb.P[0], jb.P[0], k, k, S, true);
+        if (*static_cast<volatile int*>(&sh->abort)) break;
+        if (it == 0 && plain_steps == 0) {
+            double row_max, best;
+            first_bound(S, n, k, sh, ss, row_max, best);
+            if (tid == 0) {
+                // s >= rho(X0); the model's rules are stated for A / b_j = X0 / phi
+                const double rmax = row_max;
+                const double smax = sqrt(fmin(best, rmax) * (1.0 + 1e-12));
+                double c = smax > 0.0 ? 1.2 / smax : 1.0, lsch = 1.0;
+                if (model && smax > 0.0) {  // same rule as the tensor-core kernel
+                    const double phi = ldexp(model->b, -e), s1 = smax / phi;
+                    double scale = 1.2 / s1;
+                    const bool gap = model->dhat > 0.0;
+                    if (gap ? model->dhat <= s1 : s1 <= 1.7) {
+                        if (gap) {  // the scaled schedule from l0 = dhat / s
+                            const double l0 = model->dhat / s1, a0 = ns_scale(l0);
+                            scale = a0 / s1;
+                            lsch = ns_next_lower(a0, l0);
+                        } else {
+                            scale = fmax(1.0, scale);
+                        }
+                    } else {
+                        atomicAdd(model->fallbacks, 1);
+                    }
+                    c = scale / phi;
+                }
+                bound_out->rmax = rmax;
+                bound_out->c = c;
+                ss->lsch = lsch;
+                ss->f1 = fixed_factor(c);
+                ss->f2 = fixed_factor(c * c);
+                ss->stop = 0;
+            }
+        } else if (tid == 0) {
+            const double l = ss->lsch;
+            ss->f1 = ss->f2 = 0;
+            ss->stop = 1;
+            if (l < 1.0) {  // the scaled schedule
+                const double f = ns_scale(l);
+                ss->lsch = ns_next_lower(f, l);
+                ss->f1 = fixed_factor(f);
+                ss->f2 = fixed_factor(f * f);
+                ss->stop = f - 1.0 <= 2e-6;
+            }
+        }
         __syncthreads();
-        gemm_fp64(Tb, Zb, Yb, n, ld, 2, As, Bs);  // Z' = T Z into Y's buffer
-        __syncthreads();
-        double* old_z = Zb;
-        Zb = Yb;
-        Yb = Nb;
-        Nb = old_z;
+        const uint64_t f1 = ss->f1, f2 = ss->f2;
+        // W = I - a^2 X^2 to its digits; the residual ||I - X^2||_F
+        float r2 = pass_residual(S, jb.P[1], n, k, 0, f2);
+        r2 = cta_sum(r2 * 0x1p-76f, sh);
+        slice_product(sh, jb.P[0], jb.P[1], k, k, S, true);
+        if (*static_cast<volatile int*>(&sh->abort)) break;
         done = it + 1;
-        if (!isfinite(r2)) { bad = true; break; }
-        if (it > 0 && sqrt(r2) <= tau) { conv = true; break; }
+        bad = !isfinite(r2);
+        bool last = bad || done == limit;
+        if (plain_steps == 0 && it > 0 && sqrtf(r2) <= tau) {
+            // stop after this step unless it was a scaled step whose factor moves converged
+            // eigenvalues off 1 (p(a) ~ 1 - 1.5 (a - 1)^2): then plain steps from here
+            if (ss->stop) {
+                conv = last = true;
+            } else {
+                __syncthreads();
+                if (tid == 0) ss->lsch = 1.0;
+            }
+        }
+        pass_update(X, S, last ? nullptr : jb.P[0], k, f1);
+        if (last) break;
     }
     return done;
 }
 
-// The finite-temperature Fermi function F = (I + exp(beta A))^-1 = 1/2 (I - tanh(beta A / 2)) of
-// a symmetric A, from X = A / g (g >= the spectral radius of A), in products only:
-//   B = (beta g / 2) X / 2^k with k such that ||B|| <= 1/16;
+// Largest 2-norm of a column of M, squared.
+__device__ __noinline__ float column_norm2(const SliceJob& jb, const int64_t* M, SliceShared* sh) {
+    const int n = jb.n, k = jb.k, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float worst = 0.0f;
+    for (int c = 2 * warp; c < n; c += 2 * kSliceWarps) {
+        const longlong2* m = reinterpret_cast<const longlong2*>(M) + static_cast<int64_t>(c >> 1) * k;
+        float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll 4
+        for (int r = lane; r < k; r += 32) {
+            const longlong2 v = m[r];
+            const float x = static_cast<float>(static_cast<int>(v.x >> 32)), y = static_cast<float>(static_cast<int>(v.y >> 32));
+            a0 = fmaf(x, x, a0);
+            a1 = fmaf(y, y, a1);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+            a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+        }
+        worst = fmaxf(worst, fmaxf(a0, a1));
+    }
+    return cta_max(worst, sh) * 0x1p-60f;
+}
+
+// The sign iteration of the Eq. 12 block matrix [[0, A], [I, 0]] written per block (the coupled
+// Newton-Schulz iteration): R = I - Z Y, Y <- Y + 1/2 Y R, Z <- Z + 1/2 R Z from Y = A / b (eigenvalues in
+// (0, 1]) and Z = I; Y -> (A / b)^1/2, Z -> (A / b)^-1/2.  The residual ||Z Y - I||_F comes with the
+// first product; the stopping rule is the sign iteration's.  src is A (leading dimension ld), b >= its
+// largest eigenvalue.  Y ends in M[0] (digits P[0]), Z in M[1] (digits P[1]) in units of 2^(ez - 62); M[2]
+// takes the products, P[2] the digits of R.  Every matrix is a polynomial of A, so the products are
+// symmetric.  The first step needs one product (Z = I), the last only that of the wanted root.
+// Y and R have 2-norms of at most 1; Z's rows are kept below 1 by its exponent (a step multiplies its
+// 2-norm by at most 1.5).  ||R||_F^2 > 1.5 n or a vanishing Z means that A is not positive definite.
+__device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* __restrict__ src, int ld, double b, int max_iter, float tau,
+                             bool want_y, bool want_z, int& ez, SliceScalars* ss, bool& conv, bool& bad) {
+    const int n = jb.n, k = jb.k;
+    int64_t *Y = jb.M[0], *Z = jb.M[1], *S = jb.M[2];
+    conv = bad = false;
+    ez = 0;
+    int done = 0;
+    // 1 / b as a 64-bit fraction in [1/2, 1) times a power of two
+    const double inv = 1.0 / b;
+    const uint64_t ib = static_cast<uint64_t>(__double_as_longlong(inv));
+    const uint64_t f = ((ib & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
+    const int e = 1022 - static_cast<int>((ib >> 52) & 0x7ff);
+    bool off = !(b > 0.0) || !isfinite(inv) || inv == 0.0;
+    off |= pass_source(src, ld, 0.0, e, f, Y, jb.P[0], n, k);
+    if (__syncthreads_or(off)) {
+        bad = true;
+        return 0;
+    }
+    for (int it = 0; it < max_iter; ++it) {
+        if (it > 0) {
+            slice_product(sh, jb.P[1], jb.P[0], k, k, S, true);  // Z Y
+            if (*static_cast<volatile int*>(&sh->abort)) break;
+        }
+        float r2 = pass_residual(it > 0 ? S : Y, jb.P[2], n, k, ez, 0);
+        r2 = cta_sum(r2 * 0x1p-76f, sh);
+        done = it + 1;
+        if (!isfinite(r2) || r2 > 1.5f * static_cast<float>(n) || ez > 40) {
+            bad = true;
+            break;
+        }
+        conv = it > 0 && sqrtf(r2) <= tau;
+        if (!conv || want_y) {
+            slice_product(sh, jb.P[0], jb.P[2], k, k, S, true);  // Y R
+            if (*static_cast<volatile int*>(&sh->abort)) break;
+            pass_update(Y, S, jb.P[0], k, 0);
+        }
+        if (!conv || want_z) {
+            if (it > 0) {
+                slice_product(sh, jb.P[2], jb.P[1], k, k, S, true);  // R Z
+                if (*static_cast<volatile int*>(&sh->abort)) break;
+            }
+            // Z' = Z + 1/2 R Z; from Z = I: I + 1/2 R = 3/2 I - 1/2 Y0, where Y now holds Y0 + 1/2 Y0 R and S = Y0 R
+            if (it > 0) pass_update(Z, S, nullptr, k, 0);
+            else pass_first_root(Y, S, Z, n, k);
+            const int shift = column_norm2(jb, Z, sh) > 1.0f ? 1 : 0;
+            ez += shift;
+            pass_affine(Z, shift ? Z : nullptr, jb.P[1], n, k, 0, false, -shift, 0);
+        }
+        if (conv) break;
+    }
+    return done;
+}
+
+// The finite-temperature Fermi function F = (I + exp(beta A))^-1 = 1/2 (I - tanh(beta A / 2)) of a
+// symmetric A (src, leading dimension ld; g >= its spectral radius), in products only:
+//   B = beta A / 2^(m + 1) with m such that ||B|| <= 1/16;
 //   T = tanh(B) by its odd Taylor series to degree 11 (the next term is below 1e-18 there);
-//   k doublings tanh(2x) = 2 tanh(x) / (1 + tanh(x)^2): T <- 2 T (I + T^2)^-1, the inverse by
-//   Newton-Schulz V <- V + V (I - M V) from V = 4/3 I - 4/9 M (the first step from 2/3 I in
-//   closed form; M = I + T^2 has its eigenvalues in [1, 2], so the residual I - M V starts
-//   below 1/9 and squares every step) until ||I - M V||_F <= 1e-15 sqrt(n);
+//   m doublings tanh(2x) = 2 tanh(x) / (1 + tanh(x)^2): with E = T^2 (eigenvalues in [0, 1]) and
+//   Q = I - 2 E the linear approximation V0 = 2/3 I + 2/9 Q of (I + E)^-1 leaves the residual
+//   I - (I + E) V0 = Q^2 / 9 = K, so T' = 2 T V0 (I + K) (I + K^2) (I + K^4) (I + K^8) (I + K^16)
+//   to 1e-30: twelve products a doubling;
 //   F = 1/2 (I - T).
-// A doubling at most doubles an error in T, so k doublings cost about 2^k rounding errors
-// (k = 11 at beta g = 150).  Five n x n buffers (X first); returns the one holding F and counts
-// the products in nprod.
-__device__ double* fermi_tanh(double* X, double* B1, double* B2, double* B3, double* B4, int n, int ld, double beta_g,
-                              double (*As)[kTile + 1], double (*Bs)[kTile + 1], double* scratch, int& nprod, bool& bad) {
-    int k = 0;
-    double sc = 0.5 * beta_g;
-    while (sc > 1.0 / 16.0 && k < 60) {
-        sc *= 0.5;
-        ++k;
-    }
-    // M <- alpha M + d I
-    auto axpy_diag = [&](double* M, double alpha, double d) {
-        for (int r = threadIdx.x / 32; r < n; r += 8)
-            for (int c = threadIdx.x & 31; c < n; c += 32) {
-                double& v = M[static_cast<int64_t>(r) * ld + c];
-                v = alpha * v + (r == c ? d : 0.0);
-            }
-        __syncthreads();
-    };
-    auto prod = [&](const double* A, const double* B, double* C) {
-        gemm_fp64(A, B, C, n, ld, 2, As, Bs);
-        __syncthreads();
-        ++nprod;
-    };
-    nprod = 0;
+// A doubling at most doubles an error in T (m = 11 at beta g = 150).  T is kept as T 2^t with the
+// largest t for which its norm bound min(1, 2^doublings / 16) stays below 1.  The result's T 2^t is in
+// M[0] (units of 2^-62), t in ss->e; M[1] takes the products.  Returns the number of products.
+__device__ int fermi_tanh(SliceShared* sh, const SliceJob& jb, const double* __restrict__ src, int ld, double g, double beta, SliceScalars* ss,
+                          bool& bad) {
+    const int n = jb.n, k = jb.k;
+    int64_t *T = jb.M[0], *S = jb.M[1];
+    uint8_t *PT = jb.P[0], *PK = jb.P[1], *PP = jb.P[2];
     bad = false;
-    // T = tanh(B): X <- B in place, Y = B^2, Horner in Y, T = B p(B^2)
-    axpy_diag(X, sc, 0.0);
-    double* Y = B1;
-    double* P = B2;
-    double* Q = B3;
-    prod(X, X, Y);
-    const double c[6] = {1.0, -1.0 / 3.0, 2.0 / 15.0, -17.0 / 315.0, 62.0 / 2835.0, -1382.0 / 155925.0};
-    for (int r = threadIdx.x / 32; r < n; r += 8)
-        for (int cc = threadIdx.x & 31; cc < n; cc += 32) {
-            const int64_t o = static_cast<int64_t>(r) * ld + cc;
-            P[o] = c[5] * Y[o] + (r == cc ? c[4] : 0.0);
+    if (threadIdx.x == 0) ss->e = 0;
+    int m = 0;
+    double sc = 0.5 * beta * g;
+    while (sc > 1.0 / 16.0 && m < 60) {
+        sc *= 0.5;
+        ++m;
+    }
+    // B 2^s with ||B 2^s|| <= 1: s = the exponent room of sc
+    int s2 = 0;
+    if (sc > 0.0)
+        while (sc < 0.5 && s2 < 60) {
+            sc *= 2.0;
+            ++s2;
         }
-    __syncthreads();
+    // A (beta / 2^(m + 1)) 2^s2 = A sc / g
+    const double fac = sc / g;
+    const uint64_t ib = static_cast<uint64_t>(__double_as_longlong(fac));
+    const uint64_t f = ((ib & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
+    const int e = 1022 - static_cast<int>((ib >> 52) & 0x7ff);
+    const bool zero = !(fac > 0.0);
+    bool off = !isfinite(fac);
+    if (!zero && !off) off = pass_source(src, ld, 0.0, e, f, T, PT, n, k);
+    if (__syncthreads_or(off)) {
+        bad = true;
+        return 0;
+    }
+    if (zero) return 0;  // T = 0
+    int nprod = 0;
+    // wide: with the digit pairs of weight 9 (an error in T may double at every doubling; the products of
+    // K enter it with factors of 1/9 and less)
+    auto prod = [&](const uint8_t* a, const uint8_t* b, bool wide) {
+        set_accumulation(sh, wide ? 8 : 7, wide ? 160 / 16 : kSliceK / 16);
+        slice_product(sh, a, b, k, k, S, true);
+        ++nprod;
+        return *static_cast<volatile int*>(&sh->abort) == 0;
+    };
+    const double cs[6] = {1.0, -1.0 / 3.0, 2.0 / 15.0, -17.0 / 315.0, 62.0 / 2835.0, -1382.0 / 155925.0};
+    auto fixed = [](double v) { return static_cast<int64_t>(v * 0x1p62); };
+    // Y = B^2 (digits of Y 2^(2 s2)); P = c4 + c5 Y, then P <- c_i + P Y
+    if (!prod(PT, PT, true)) return nprod;
+    const int down = 2 * s2;
+    const uint64_t c5 = fixed_factor(-cs[5]);
+    const int64_t c4 = fixed(cs[4]);
+    pass_affine(S, nullptr, PP, n, k, c4, true, -down, c5);
+    pass_affine(S, nullptr, PK, n, k, 0, false, 0, 0);
     for (int i = 3; i >= 0; --i) {
-        prod(P, Y, Q);
-        axpy_diag(Q, 1.0, c[i]);
-        double* t = P; P = Q; Q = t;
+        if (!prod(PP, PK, true)) return nprod;
+        const int64_t ci = fixed(cs[i]);
+        pass_affine(S, nullptr, PP, n, k, ci, false, -down, 0);
     }
-    prod(X, P, Q);
-    double* T = Q;
-    double* fr[4] = {X, Y, P, B4};  // free buffers
-    for (int d = 0; d < k && !bad; ++d) {
-        double *M = fr[0], *V = fr[1], *R = fr[2], *Vn = fr[3];
-        prod(T, T, M);  // M = I + T^2
-        axpy_diag(M, 1.0, 1.0);
-        for (int r = threadIdx.x / 32; r < n; r += 8)
-            for (int cc = threadIdx.x & 31; cc < n; cc += 32) {
-                const int64_t o = static_cast<int64_t>(r) * ld + cc;
-                V[o] = (r == cc ? 4.0 / 3.0 : 0.0) - 4.0 / 9.0 * M[o];
-            }
-        __syncthreads();
-        for (int m = 0; m < 12; ++m) {
-            prod(M, V, R);  // R = I - M V
-            double r2 = 0.0;
-            for (int r = threadIdx.x / 32; r < n; r += 8)
-                for (int cc = threadIdx.x & 31; cc < n; cc += 32) {
-                    const int64_t o = static_cast<int64_t>(r) * ld + cc;
-                    const double e = (r == cc ? 1.0 : 0.0) - R[o];
-                    R[o] = e;
-                    r2 += e * e;
-                }
-            r2 = block_sum(r2, scratch);
-            if (!isfinite(r2)) { bad = true; break; }
-            if (sqrt(r2) <= 1e-15 * sqrt(static_cast<double>(n))) break;
-            prod(V, R, Vn);  // V <- V + V R
-            for (int r = threadIdx.x / 32; r < n; r += 8)
-                for (int cc = threadIdx.x & 31; cc < n; cc += 32) {
-                    const int64_t o = static_cast<int64_t>(r) * ld + cc;
-                    Vn[o] += V[o];
-                }
-            __syncthreads();
-            double* t = V; V = Vn; Vn = t;
+    if (!prod(PT, PP, true)) return nprod;
+    pass_affine(S, T, PT, n, k, 0, false, 0, 0);
+    int t = s2;
+    const uint64_t f23 = fixed_factor(2.0 / 3.0), f29 = fixed_factor(2.0 / 9.0);
+    for (int d = 0; d < m; ++d) {
+        // E = T^2 (S holds E 2^(2 t)), Q = I - 2 E
+        if (!prod(PT, PT, true)) return nprod;
+        const int dn = 2 * t;
+        pass_affine(S, nullptr, PK, n, k, kFixedOne, true, 1 - dn, 0);
+        // U = T V0 (times 2 when T 2^t has no exponent room left; else 2 T V0 has one less)
+        if (!prod(PT, PK, true)) return nprod;
+        const int up = t > 0 ? 0 : 1;
+        t = t > 0 ? t - 1 : 0;
+        pass_mix(T, S, PT, k, f23, f29, up);
+        // K = Q^2 / 9 (digits of 9^j K^j: powers of Q^2), U <- U + U K^j for j = 1, 2, 4, 8, 16
+        double w = 1.0 / 9.0;
+        for (int j = 0; j < 5; ++j) {
+            if (!prod(PK, PK, false)) return nprod;
+            pass_affine(S, nullptr, PK, n, k, 0, false, 0, 0);
+            if (!prod(PT, PK, false)) return nprod;
+            pass_mix(T, S, PT, k, 0, fixed_factor(w), 0);
+            w *= w;
         }
-        prod(T, V, R);  // T <- 2 T V
-        axpy_diag(R, 2.0, 0.0);
-        double* oldT = T;
-        T = R;
-        fr[0] = oldT;
-        fr[1] = M;
-        fr[2] = V;
-        fr[3] = Vn;
     }
-    axpy_diag(T, -0.5, 0.5);  // F = 1/2 (I - T)
-    return T;
+    __syncthreads();
+    if (threadIdx.x == 0) ss->e = t;
+    __syncthreads();
+    return nprod;
 }
 
 // Gershgorin interval (lo, hi) of an n x n matrix held row by row.
 __device__ double2 gershgorin_interval(const double* M, int n, int ld, double* scratch) {
     const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
     double lo = INFINITY, hi = -INFINITY;
-    for (int r = warp; r < n; r += 8) {
+    for (int r = warp; r < n; r += kSliceWarps) {
         double acc = 0.0;
         for (int c = lane; c < n; c += 32) acc += c == r ? 0.0 : fabs(M[static_cast<int64_t>(r) * ld + c]);
         acc = warp_sum(acc);
@@ -230,387 +630,305 @@ __device__ double2 gershgorin_interval(const double* M, int n, int ld, double* s
         lo = fmin(lo, d - acc);
         hi = fmax(hi, d + acc);
     }
-    lo = -warp_max(-lo);
-    hi = warp_max(hi);
     if (lane == 0) {
         scratch[warp] = lo;
-        scratch[8 + warp] = hi;
+        scratch[32 + warp] = hi;
     }
     __syncthreads();
     double2 out = make_double2(INFINITY, -INFINITY);
-    for (int w = 0; w < 8; ++w) {
+    for (int w = 0; w < kSliceWarps; ++w) {
         out.x = fmin(out.x, scratch[w]);
-        out.y = fmax(out.y, scratch[8 + w]);
+        out.y = fmax(out.y, scratch[32 + w]);
     }
     __syncthreads();
     return out;
 }
 
-// C[i][q] = sum_k A[i][k] Bt[q][k] for i < n, q < m: a product with a thin right factor given
-// by its rows (Bt = the transposed factor, m rows of length n, leading dimension ldb), C with
-// leading dimension m.  mode 1 writes Bt[q][i] - C[i][q] instead; scale multiplies the result.
-// A warp per row i, eight columns q at a time.
-__device__ void thin_product(const double* __restrict__ A, int lda, const double* __restrict__ Bt, int ldb, int n, int m,
-                             double* __restrict__ C, int mode, double scale) {
-    const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-    for (int i = warp; i < n; i += 8) {
-        const double* ai = A + static_cast<int64_t>(i) * lda;
-        for (int q0 = 0; q0 < m; q0 += 8) {
-            double acc[8];
-#pragma unroll
-            for (int t = 0; t < 8; ++t) acc[t] = 0.0;
-            for (int k = lane; k < n; k += 32) {
-                const double x = ai[k];
-#pragma unroll
-                for (int t = 0; t < 8; ++t)
-                    if (q0 + t < m) acc[t] = fma(x, Bt[static_cast<int64_t>(q0 + t) * ldb + k], acc[t]);
-            }
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const double v = warp_sum(acc[t]);
-                if (lane == 0 && q0 + t < m) {
-                    const double r = mode == 1 ? Bt[static_cast<int64_t>(q0 + t) * ldb + i] - v : v;
-                    C[static_cast<int64_t>(i) * m + q0 + t] = scale * r;
-                }
-            }
+// The CTA's next submatrix (largest first; every thread gets its place in the order), claimed one
+// ahead: while it is worked on, the source of the one after it comes into L2.
+__device__ __forceinline__ int claim_job(int* counter, SliceScalars* ss, SubDesc* cur, bool first, int n_subs, const int32_t* order, const SubDesc* subs,
+                                         const double* src) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        ss->job = first ? atomicAdd(counter, 1) : ss->next;
+        if (ss->job < n_subs) *cur = subs[order[ss->job]];
+        const int nx = atomicAdd(counter, 1);
+        ss->next = nx;
+        if (nx < n_subs) {
+            const SubDesc& s = subs[order[nx]];
+            const uint64_t bytes = static_cast<uint64_t>(s.n) * s.ld * sizeof(double);
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + s.t_off),
+                         "r"(static_cast<uint32_t>(bytes < (8u << 20) ? bytes : (8u << 20)) & ~15u)
+                         : "memory");
         }
     }
     __syncthreads();
+    return ss->job;
+}
+
+// The last CTA to run out of work resets the job counter for the next launch.
+__device__ __forceinline__ void release_jobs(int* counter, unsigned int* ticket) {
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(ticket, 1u) == gridDim.x - 1) {
+            *counter = 0;
+            *ticket = 0u;
+        }
+    }
+}
+
+__device__ __forceinline__ uint8_t* slice_stages() {
+    extern __shared__ uint8_t slice_smem_raw[];
+    return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(slice_smem_raw) + 1023) & ~uintptr_t(1023));
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(256) k_ns_fp64(NsFp64Args a) {
-    __shared__ double As[kKc][kTile + 1];
-    __shared__ double Bs[kKc][kTile + 1];
-    __shared__ double scratch[32];
-    extern __shared__ int ls_smem[];
-    if (a.skip && *a.skip) return;
-    const SubDesc s = a.subs[blockIdx.x];
-    const int n = s.n, ld = s.ld;
-    double* X = a.T + s.t_off;
-    double* Y = a.W1 + s.t_off;
-    double* Z = a.W2 + s.t_off;
-    if (a.Mc) {
-        // non-orthogonal form: the sign iteration runs on M_j - mu I with M_j = L_j A_H L_j
-        // (L_j = A_S^-1/2, from the setup kernel); its Gershgorin bound starts the iteration
-        const double* M = a.Mc + s.t_off;
-        const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-        double rmax = 0.0;
-        for (int r = warp; r < n; r += 8) {
-            double acc = 0.0;
-            for (int c = lane; c < n; c += 32) {
-                const double v = M[static_cast<int64_t>(r) * ld + c] - (r == c ? a.mu : 0.0);
-                X[static_cast<int64_t>(r) * ld + c] = v;
-                acc += fabs(v);
-            }
-            rmax = fmax(rmax, warp_sum(acc));
-        }
-        rmax = warp_max(rmax);
-        if (lane == 0) scratch[warp] = rmax;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double b = 0.0;
-            for (int w = 0; w < 8; ++w) b = fmax(b, scratch[w]);
-            b = b > 0.0 ? b : 1.0;
-            a.bound[blockIdx.x] = b;
-            a.gersh[blockIdx.x] = b;
-        }
-        __syncthreads();
-    }
-    if (a.finish_iters > 0) {
-        // FP64 finishing steps after a low-precision bulk phase: X (in T) is that phase's last
-        // iterate; plain Newton-Schulz steps in FP64, then the scatter of the owner columns
-        bool bad = false;
-        for (int it = 0; it < a.finish_iters; ++it) {
-            double r2 = gemm_fp64(X, X, Y, n, ld, 1, As, Bs);  // Y = 3/2 I - 1/2 X^2
-            r2 = block_sum(r2, scratch);
-            gemm_fp64(X, Y, Z, n, ld, 2, As, Bs);
-            __syncthreads();
-            double* tmp = X; X = Z; Z = tmp;
-            if (!isfinite(r2)) bad = true;
-        }
-        if (threadIdx.x == 0) {
-            a.iters[s.col] += a.finish_iters;
-            atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * a.finish_iters);
-            if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
-        }
-        const double* Xf = X;
-        auto xrow = [&](int q, int i) -> double { return Xf[static_cast<int64_t>(s.own + q) * ld + i]; };
-        finish_column(s, a.pv, a.H, a.D, a.partial, xrow, ls_smem, scratch);
-        return;
-    }
-    const double inv_b = 1.0 / a.bound[blockIdx.x];
-    // learned bound: the predicted smallest |eigenvalue| of X0 = (T_j - mu I) / b_j (negative:
-    // no prediction), and the lower end the scaled schedule assumes (1 = plain steps)
-    const double dhat = a.pred ? a.pred[2 * blockIdx.x + 1] * a.gersh[blockIdx.x] * inv_b : -1.0;
-    double lsch = 1.0, acur = 1.0;
-    for (int r = threadIdx.x / 32; r < n; r += 8)
-        for (int c = threadIdx.x & 31; c < n; c += 32) X[static_cast<int64_t>(r) * ld + c] *= inv_b;
-    __syncthreads();
+// FORM: the sign iteration, the coupled iteration of the roots or the Fermi function (one kernel each:
+// together their live values would not fit the registers).
+enum { kFormSign, kFormRoots, kFormFermi };
 
-    int done = 0;
-    bool conv = false, bad = false;
-    if (a.function == kFnFermi) {
-        // the Fermi function of A = T_j - mu I (now A / b in X, b its Gershgorin bound)
-        int nprod = 0;
-        bool bad = false;
-        const double* F = fermi_tanh(X, Y, Z, a.W3 + s.t_off, a.W4 + s.t_off, n, ld,
-                                     a.beta * a.bound[blockIdx.x], As, Bs, scratch, nprod, bad);
-        if (threadIdx.x == 0) {
-            a.iters[s.col] = nprod;
-            atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * nprod);
-            if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
+template <int FORM>
+__global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_constant__ NsFp64Args a) {
+    __shared__ SliceShared shared;
+    __shared__ SliceScalars ss;
+    __shared__ SignBound sb;
+    __shared__ SubDesc s;
+    __shared__ SliceJob jb;
+    __shared__ double scratch[64];
+    if (a.skip && *a.skip) return;
+    SliceShared* const sh = &shared;
+    int* ls_smem = reinterpret_cast<int*>(slice_stages());  // local block starts, between products only
+    slices_begin(sh, slice_stages(), a.status);
+    uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x) * a.slot_bytes;
+    for (bool first = true;; first = false) {
+        const int job = claim_job(a.work_counter, &ss, &s, first, a.n_subs, a.order, a.subs, a.Mc ? a.Mc : a.T);
+        if (job >= a.n_subs || sh->abort) break;
+        const int j = s.col;
+        if (threadIdx.x == 0) slice_job(jb, slot, s.n, a.kmax, a.mats);
+        __syncthreads();
+        const int n = s.n, k = jb.k;
+        const double* T = a.T + s.t_off;
+        bool conv = false, bad = false;
+        int done = 0;
+        if constexpr (FORM == kFormFermi) {
+            done = fermi_tanh(sh, jb, T, s.ld, a.bound[j], a.beta, &ss, bad);
+            if (sh->abort) break;
+            if (threadIdx.x == 0) {
+                a.iters[j] = done;
+                atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
+                if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
+            }
+            const int64_t* F = jb.M[0];
+            const double fs = ldexp(1.0, -ss.e);
+            auto frow = [&](int q, int i) -> double { return fs * from_fixed(F[mat_at(k, i, s.own + q)]); };
+            finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch);  // 1/2 (I - T)
+            fence_proxy_async_smem();
+            continue;
+        } else if constexpr (FORM == kFormRoots) {
+            // f = A^-1/2, A^1/2 or A^-1 for a symmetric positive definite A = T_j - mu I
+            int ez = 0;
+            const double b = a.bound[j];
+            done = coupled_steps(sh, jb, T, s.ld, b, a.max_iter, static_cast<float>(a.tau), a.function == kFnSqrt, a.function != kFnSqrt, ez,
+                                 &ss, conv, bad);
+            if (sh->abort) break;
+            if (threadIdx.x == 0) {
+                a.iters[j] = done;
+                atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
+                if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
+                else if (!conv) atomicCAS(a.status, kOk, kErrNoconv);
+            }
+            // A^-1/2 = Z / sqrt(b), A^1/2 = sqrt(b) Y, A^-1 = Z Z / b (symmetric: row own + q is
+            // column own + q)
+            const int64_t* F = a.function == kFnSqrt ? jb.M[0] : jb.M[1];
+            double fs = a.function == kFnSqrt ? sqrt(b) : ldexp(1.0 / sqrt(b), ez);
+            if (a.function == kFnInv) {
+                slice_product(sh, jb.P[1], jb.P[1], k, k, jb.M[2], true);
+                if (sh->abort) break;
+                F = jb.M[2];
+                fs = ldexp(1.0 / b, 2 * ez);
+            }
+            auto frow = [&](int q, int i) -> double { return fs * from_fixed(F[mat_at(k, i, s.own + q)]); };
+            finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch, false);
+            fence_proxy_async_smem();
+            continue;
+        } else {
+        // the sign iteration: on T_j - mu I, on M_j - mu I (non-orthogonal form: M_j = L_j A_H L_j from the
+        // setup kernel), or FP64 finishing steps on a bulk phase's last iterate
+        const double* src = a.Mc ? a.Mc + s.t_off : T;
+        if (a.Mc) {  // its Gershgorin bound
+            const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+            double rmax = 0.0;
+            for (int r = warp; r < n; r += kSliceWarps) {
+                double acc = 0.0;
+                for (int c = lane; c < n; c += 32) acc += fabs(src[static_cast<int64_t>(r) * s.ld + c] - (r == c ? a.mu : 0.0));
+                rmax = fmax(rmax, warp_sum(acc));
+            }
+            if (lane == 0) scratch[warp] = rmax;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                double b = 0.0;
+                for (int w = 0; w < kSliceWarps; ++w) b = fmax(b, scratch[w]);
+                a.gersh[j] = b > 0.0 ? b : 1.0;
+            }
+            __syncthreads();
         }
-        auto frow = [&](int q, int i) -> double { return F[static_cast<int64_t>(s.own + q) * ld + i]; };
-        finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch, false);
-        return;
-    }
-    if (a.function != kFnDensity) {
-        // f = A^-1/2 or A^1/2 for a symmetric positive definite A = T_j - mu I (now A/b in X)
-        double* Yb = X;
-        double* Zb = Y;
-        double* Tb = Z;
-        double* Nb = a.W3 + s.t_off;
-        done = coupled_ns(Yb, Zb, Tb, Nb, n, ld, a.max_iter, a.tau, As, Bs, scratch, conv, bad);
+        const bool finish = a.finish_iters > 0;
+        SignModel model{a.bound[j], a.pred ? static_cast<double>(a.pred[2 * j + 1]) * a.gersh[j] / a.bound[j] : -1.0, a.fallbacks};
+        const int e = load_fixed(src, s.ld, a.Mc ? a.mu : 0.0, a.gersh[j], jb, jb.M[0], jb.P[0], finish, sh, &ss);
+        bad = ss.bad != 0;
+        // with the learned bound W reaches a norm of 2, with a bulk phase's iterate X one of about 1.2
+        set_accumulation(sh, 7, a.use_model || finish ? 160 / 16 : kSliceK / 16);
+        if (!bad)
+            done = sign_steps(sh, jb, e, a.max_iter, static_cast<float>(a.tau), a.finish_iters, a.use_model ? &model : nullptr, &sb, &ss, conv,
+                              bad);
+        if (sh->abort) break;
         if (threadIdx.x == 0) {
-            a.iters[s.col] = done;
+            if (finish) {
+                a.iters[j] += done;
+            } else {
+                a.iters[j] = done;
+                if (!bad || done > 0) {
+                    // feature of the next snapshot: the Gershgorin bound of A^2, over G; and the
+                    // effective bound of c X0
+                    a.sq_ratio[j] = static_cast<float>(ldexp(sqrt(sb.rmax), e) / a.gersh[j]);
+                    a.bound[j] = ldexp(1.0 / sb.c, e);
+                }
+            }
             atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
+            if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
+            else if (!conv && !finish) atomicCAS(a.status, kOk, kErrNoconv);
+        }
+        const int64_t* X = jb.M[0];
+        if (a.Mc) {
+            // P_j[:, own] = 1/2 L (I - X) L[:, own] = 1/2 L (W - X W), W = L[:, own] (rows own..
+            // of the symmetric L): Eq. 14 with sign(A_S^-1 A_H - mu I) = L sign(M - mu I) L^-1
+            // and A_S^-1 = L L.  Two products with the owner columns only: the digits of X in P[0], of L in
+            // P[1], of W^T and then of 1/2 (W - X W)^T in P[2]; the products in M[1].
+            set_accumulation(sh, 8, 160 / 16);
+            pass_affine(X, nullptr, jb.P[0], n, k, 0, false, 0, 0);
+            int64_t *L = jb.M[0], *U = jb.M[1];
+            const int el = load_fixed(a.Lc + s.t_off, s.ld, 0.0, 0.0, jb, L, jb.P[1], false, sh, &ss);
+            const int w = s.bown <= 16 ? 16 : (s.bown + 31) & ~31;
+            pass_transposed(L, nullptr, s.own, s.bown, jb.P[2], w, k, 0);
+            slice_product(sh, jb.P[0], jb.P[2], k, w, U, false);
+            if (sh->abort) break;
+            pass_transposed(L, U, s.own, s.bown, jb.P[2], w, k, 1);
+            slice_product(sh, jb.P[1], jb.P[2], k, w, U, false);
+            if (sh->abort) break;
+            const double fs = ldexp(1.0, 2 * el);
+            auto prow = [&](int q, int i) -> double { return fs * from_fixed(U[mat_at(k, i, q)]); };
+            finish_column(s, a.pv, a.H, a.D, a.partial, prow, ls_smem, scratch, false, a.Sv);
+            fence_proxy_async_smem();
+            continue;
+        }
+        auto xrow = [&](int q, int i) -> double { return from_fixed(X[mat_at(k, i, s.own + q)]); };
+        finish_column(s, a.pv, a.H, a.D, a.partial, xrow, ls_smem, scratch);
+        fence_proxy_async_smem();
+        }
+    }
+    slices_end(sh);
+    release_jobs(a.work_counter, a.ticket);
+}
+
+// Setup of the non-orthogonal form for one (H, S) pair: from A_S (in Lc) and A_H (in Mc), both
+// gathered without shift, L = A_S^-1/2 by the coupled iteration (into Lc) and M = L A_H L, exactly
+// symmetric (into Mc), and the Gershgorin interval of M.
+__global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid_constant__ NonorthSetupArgs a) {
+    __shared__ SliceShared shared;
+    __shared__ SliceScalars ss;
+    __shared__ SubDesc s;
+    __shared__ SliceJob jb;
+    __shared__ double scratch[64];
+    SliceShared* const sh = &shared;
+    slices_begin(sh, slice_stages(), a.status);
+    uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x) * a.slot_bytes;
+    for (bool first = true;; first = false) {
+        const int job = claim_job(a.work_counter, &ss, &s, first, a.n_subs, a.order, a.subs, a.Lc);
+        if (job >= a.n_subs || sh->abort) break;
+        const int j = s.col;
+        if (threadIdx.x == 0) slice_job(jb, slot, s.n, a.kmax, a.mats);
+        __syncthreads();
+        const int n = s.n, k = jb.k;
+        set_accumulation(sh, 7, kSliceK / 16);
+        double *Lc = a.Lc + s.t_off, *Mc = a.Mc + s.t_off;
+        const double b = a.bound_s[j];
+        bool conv = false, bad = false;
+        int ez = 0;
+        const int done = coupled_steps(sh, jb, Lc, s.ld, b, a.max_iter, static_cast<float>(a.tau), false, true, ez, &ss, conv, bad);
+        if (sh->abort) break;
+        if (threadIdx.x == 0) {
+            a.iters[j] = done;
             if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
             else if (!conv) atomicCAS(a.status, kOk, kErrNoconv);
         }
-        if (a.function == kFnInv) {
-            // A^-1 = (A^-1/2)^2 = Z Z / b: its owner columns Z Z[:, own] / b (Z symmetric, so
-            // the thin factor is given by rows own ..), into the free buffer T
-            thin_product(Zb, ld, Zb + static_cast<int64_t>(s.own) * ld, ld, n, s.bown, Tb, 0,
-                         1.0 / a.bound[blockIdx.x]);
-            const double* U = Tb;
-            auto irow = [&](int q, int i) -> double { return U[static_cast<int64_t>(i) * s.bown + q]; };
-            finish_column(s, a.pv, a.H, a.D, a.partial, irow, ls_smem, scratch, false);
-            return;
+        if (bad) {  // no L: the bracket is not used, the status tells
+            if (threadIdx.x == 0) a.lohi[2 * j] = a.lohi[2 * j + 1] = 0.0;
+            continue;
         }
-        // A^-1/2 = Z / sqrt(b), A^1/2 = sqrt(b) Y (both symmetric: row own + q is column own + q)
-        const double* F = a.function == kFnInvSqrt ? Zb : Yb;
-        const double fs = a.function == kFnInvSqrt ? 1.0 / sqrt(a.bound[blockIdx.x]) : sqrt(a.bound[blockIdx.x]);
-        auto frow = [&](int q, int i) -> double { return fs * F[static_cast<int64_t>(s.own + q) * ld + i]; };
-        finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch, false);
-        return;
-    }
-    for (int it = 0; it < a.max_iter; ++it) {
-        double r2 = 1.0, oscale = 1.0;
-        if (it == 0) {
-            // a-posteriori scaling (as in the tensor-core kernel): with Y = X0^2,
-            // rho(X0)^2 = rho(Y) <= rho(|Y|) <= max_r (|Y| w)_r / w_r for any
-            // positive w (Collatz-Wielandt): w = 1 (the max row sum) and two
-            // power steps of |Y| from it; continue from X0' = (1.2/s) X0
-            gemm_fp64(X, X, Y, n, ld, 2, As, Bs);
-            __syncthreads();
-            double* wv = Z;  // the output buffer of this iteration is free until the second product
-            double* wn = Z + n;
-            const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-            auto block_max2 = [&](double x, double y) -> double2 {
-                x = warp_max(x);
-                y = warp_max(y);
-                if (lane == 0) {
-                    scratch[warp] = x;
-                    scratch[8 + warp] = y;
-                }
-                __syncthreads();
-                double2 m = make_double2(0.0, 0.0);
-                for (int w = 0; w < 8; ++w) {
-                    m.x = fmax(m.x, scratch[w]);
-                    m.y = fmax(m.y, scratch[8 + w]);
-                }
-                __syncthreads();
-                return m;
-            };
-            double rmax = 0.0;
-            for (int r = warp; r < n; r += 8) {
-                double acc = 0.0;
-                for (int c = lane; c < n; c += 32) acc += fabs(Y[static_cast<int64_t>(r) * ld + c]);
-                acc = warp_sum(acc);
-                if (lane == 0) wv[r] = acc;
-                rmax = fmax(rmax, acc);
-            }
-            rmax = block_max2(rmax, 0.0).x;
-            double best = rmax, wtop = rmax;
-            for (int pass = 0; pass < 2 && best > 0.0; ++pass) {
-                for (int c = threadIdx.x; c < n; c += blockDim.x) wv[c] = fmax(wv[c], 1e-30 * wtop);
-                __syncthreads();
-                double q = 0.0, wm = 0.0;
-                for (int r = warp; r < n; r += 8) {
-                    double acc = 0.0;
-                    for (int c = lane; c < n; c += 32) acc = fma(fabs(Y[static_cast<int64_t>(r) * ld + c]), wv[c], acc);
-                    acc = warp_sum(acc);
-                    if (lane == 0) wn[r] = acc;
-                    q = fmax(q, acc / wv[r]);
-                    wm = fmax(wm, acc);
-                }
-                const double2 m2 = block_max2(q, wm);
-                best = fmin(best, m2.x);
-                if (!(m2.y > 0.0)) break;
-                for (int c = threadIdx.x; c < n; c += blockDim.x) wv[c] = wn[c] / m2.y;
-                wtop = 1.0;
-            }
-            const double smax = sqrt(best * (1.0 + 1e-12));
-            double scale = smax > 0.0 ? 1.2 / smax : 1.0;
-            if (a.use_model && smax > 0.0) {  // same rule as the tensor-core kernel
-                const bool gap = dhat > 0.0;
-                if (gap ? dhat <= smax : smax <= 1.7) {
-                    if (gap) {  // the scaled schedule from l0 = dhat / s
-                        const double l0 = dhat / smax;
-                        const double a0 = ns_scale(l0);
-                        scale = a0 / smax;
-                        lsch = ns_next_lower(a0, l0);
-                    } else {
-                        scale = fmax(1.0, scale);
-                    }
-                } else if (threadIdx.x == 0) {
-                    atomicAdd(a.fallbacks, 1);
-                }
-            }
-            const double sc2 = scale * scale;
-            for (int r = threadIdx.x / 32; r < n; r += 8)
-                for (int c = threadIdx.x & 31; c < n; c += 32) {
-                    double& y = Y[static_cast<int64_t>(r) * ld + c];
-                    y = (r == c ? 1.5 : 0.0) - 0.5 * sc2 * y;
-                }
+        // A_H 2^-eh with rows of at most 1; Q = A_H L, then M = L Q = L A_H L: the right factor's digits
+        // are those of Q^T, whose rows are Q's columns
+        const int64_t* Z = jb.M[1];
+        const int eh = load_fixed(Mc, s.ld, 0.0, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
+        if (ss.bad) {
             if (threadIdx.x == 0) {
-                // feature of the next snapshot: the Gershgorin bound of A^2, over G
-                a.sq_ratio[blockIdx.x] = static_cast<float>(sqrt(rmax) * a.bound[blockIdx.x] / a.gersh[blockIdx.x]);
-                a.bound[blockIdx.x] = a.bound[blockIdx.x] / scale;
+                atomicCAS(a.status, kOk, kErrNonfinite);
+                a.lohi[2 * j] = a.lohi[2 * j + 1] = 0.0;
             }
-            __syncthreads();
-            oscale = scale;
-        } else {
-            // Y = a (3/2 I - a^2/2 X^2) on the scaled schedule (a = 1: a plain step)
-            double cf = -0.5, dg = 1.5;
-            acur = 1.0;
-            if (lsch < 1.0) {
-                const double f = ns_scale(lsch);
-                cf = -0.5 * f * f * f;
-                dg = 1.5 * f;
-                lsch = ns_next_lower(f, lsch);
-                acur = f;
-            }
-            r2 = gemm_fp64(X, X, Y, n, ld, 1, As, Bs, 1.0, cf, dg);
-            r2 = block_sum(r2, scratch);
+            continue;
         }
-        gemm_fp64(X, Y, Z, n, ld, 2, As, Bs, oscale);
+        set_accumulation(sh, 8, 160 / 16);
+        slice_product(sh, jb.P[0], jb.P[1], k, k, jb.M[2], false);
+        if (sh->abort) break;
+        // columns of A_H L may be longer than 1 (the 2-norm of A_H exceeds that of its rows)
+        const float cn = column_norm2(jb, jb.M[2], sh);
+        const int ep = cn > 1.0f ? static_cast<int>(ceilf(0.5f * log2f(cn * 1.001f))) : 0;
+        pass_transposed(jb.M[2], nullptr, 0, k, jb.P[2], k, k, ep);
+        slice_product(sh, jb.P[1], jb.P[2], k, k, jb.M[2], true);
+        if (sh->abort) break;
+        const double ls = ldexp(1.0 / sqrt(b), ez - 62);  // A_S^-1/2 = Z / sqrt(b)
+        const double ms = ldexp(1.0 / b, 2 * ez + eh + ep - 62);
+        for (int r = threadIdx.x / 32; r < n; r += kSliceWarps)
+            for (int c = threadIdx.x & 31; c < n; c += 32) {  // symmetric: row r is column r
+                const int64_t o = mat_at(k, c, r), d = static_cast<int64_t>(r) * s.ld + c;
+                Lc[d] = ls * static_cast<double>(Z[o]);
+                Mc[d] = ms * static_cast<double>(jb.M[2][o]);
+            }
         __syncthreads();
-        double* tmp = X; X = Z; Z = tmp;
-        done = it + 1;
-        if (!isfinite(r2)) { bad = true; break; }
-        if (it > 0 && sqrt(r2) <= a.tau) {
-            // stop after this step unless it was a scaled step whose factor moves converged
-            // eigenvalues off 1 (p(a) ~ 1 - 1.5 (a - 1)^2): then plain steps from here
-            if (acur - 1.0 <= 2e-6) { conv = true; break; }
-            lsch = 1.0;
+        const double2 g = gershgorin_interval(Mc, n, s.ld, scratch);
+        if (threadIdx.x == 0) {
+            a.lohi[2 * j] = g.x;
+            a.lohi[2 * j + 1] = g.y;
         }
     }
-    if (threadIdx.x == 0) {
-        a.iters[s.col] = done;
-        atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
-        if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
-        else if (!conv) atomicCAS(a.status, kOk, kErrNoconv);
-    }
-    const double* Xf = X;
-    if (a.Mc) {
-        // P_j[:, own] = 1/2 L (I - X) L[:, own] = 1/2 L (W - X W), W = L[:, own] (rows own..
-        // of the symmetric L): Eq. 14 with sign(A_S^-1 A_H - mu I) = L sign(M - mu I) L^-1
-        // and A_S^-1 = L L.  Two thin products into the free buffers Y (U) and Z (P_own).
-        const double* L = a.Lc + s.t_off;
-        double* U = Y;
-        double* Pown = Z;
-        thin_product(Xf, ld, L + static_cast<int64_t>(s.own) * ld, ld, n, s.bown, U, 1, 1.0);
-        // second factor given by rows: U^T (bown x n) is U read with stride bown
-        const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-        for (int i = warp; i < n; i += 8) {
-            const double* li = L + static_cast<int64_t>(i) * ld;
-            for (int q0 = 0; q0 < s.bown; q0 += 8) {
-                double acc[8];
-#pragma unroll
-                for (int t = 0; t < 8; ++t) acc[t] = 0.0;
-                for (int k = lane; k < n; k += 32) {
-                    const double x = li[k];
-#pragma unroll
-                    for (int t = 0; t < 8; ++t)
-                        if (q0 + t < s.bown) acc[t] = fma(x, U[static_cast<int64_t>(k) * s.bown + q0 + t], acc[t]);
-                }
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const double v = warp_sum(acc[t]);
-                    if (lane == 0 && q0 + t < s.bown) Pown[static_cast<int64_t>(i) * s.bown + q0 + t] = 0.5 * v;
-                }
-            }
-        }
-        __syncthreads();
-        auto prow = [&](int q, int i) -> double { return Pown[static_cast<int64_t>(i) * s.bown + q]; };
-        finish_column(s, a.pv, a.H, a.D, a.partial, prow, ls_smem, scratch, false, a.Sv);
-        return;
-    }
-    auto xrow = [&](int q, int i) -> double { return Xf[static_cast<int64_t>(s.own + q) * ld + i]; };
-    finish_column(s, a.pv, a.H, a.D, a.partial, xrow, ls_smem, scratch);
+    slices_end(sh);
+    release_jobs(a.work_counter, a.ticket);
 }
 
-// Setup of the non-orthogonal form for one (H, S) pair, a CTA per submatrix: from A_S (in Lc)
-// and A_H (in Mc), both gathered without shift, L = A_S^-1/2 by the coupled iteration (into
-// Lc) and M = L A_H L, symmetrised (into Mc), and the Gershgorin interval of M.
-__global__ void __launch_bounds__(256) k_nonorth_setup(NonorthSetupArgs a) {
-    __shared__ double As[kKc][kTile + 1];
-    __shared__ double Bs[kKc][kTile + 1];
-    __shared__ double scratch[32];
-    const SubDesc s = a.subs[blockIdx.x];
-    const int n = s.n, ld = s.ld;
-    double* Lc = a.Lc + s.t_off;
-    double* Mc = a.Mc + s.t_off;
-    double* Yb = a.T + s.t_off;
-    double* Zb = a.W1 + s.t_off;
-    double* Tb = a.W2 + s.t_off;
-    double* Nb = a.W3 + s.t_off;
-    const double b = a.bound_s[blockIdx.x];
-    const double inv_b = b > 0.0 ? 1.0 / b : 0.0;
-    for (int r = threadIdx.x / 32; r < n; r += 8)
-        for (int c = threadIdx.x & 31; c < n; c += 32)
-            Yb[static_cast<int64_t>(r) * ld + c] = Lc[static_cast<int64_t>(r) * ld + c] * inv_b;
-    __syncthreads();
-    bool conv = false, bad = false;
-    const int done = coupled_ns(Yb, Zb, Tb, Nb, n, ld, a.max_iter, a.tau, As, Bs, scratch, conv, bad);
-    if (threadIdx.x == 0) {
-        a.iters[s.col] = done;
-        if (bad || !(b > 0.0)) atomicCAS(a.status, kOk, kErrNonfinite);
-        else if (!conv) atomicCAS(a.status, kOk, kErrNoconv);
-    }
-    const double ls = b > 0.0 ? 1.0 / sqrt(b) : 0.0;  // A_S^-1/2 = Z / sqrt(b)
-    for (int r = threadIdx.x / 32; r < n; r += 8)
-        for (int c = threadIdx.x & 31; c < n; c += 32)
-            Lc[static_cast<int64_t>(r) * ld + c] = ls * Zb[static_cast<int64_t>(r) * ld + c];
-    __syncthreads();
-    gemm_fp64(Mc, Lc, Tb, n, ld, 2, As, Bs);  // A_H L
-    __syncthreads();
-    gemm_fp64(Lc, Tb, Nb, n, ld, 2, As, Bs);  // L A_H L
-    __syncthreads();
-    for (int r = threadIdx.x / 32; r < n; r += 8)
-        for (int c = threadIdx.x & 31; c < n; c += 32)
-            Mc[static_cast<int64_t>(r) * ld + c] =
-                0.5 * (Nb[static_cast<int64_t>(r) * ld + c] + Nb[static_cast<int64_t>(c) * ld + r]);
-    __syncthreads();
-    const double2 g = gershgorin_interval(Mc, n, ld, scratch);
-    if (threadIdx.x == 0) {
-        a.lohi[2 * blockIdx.x] = g.x;
-        a.lohi[2 * blockIdx.x + 1] = g.y;
-    }
+size_t fp64_slot_bytes(int max_n, int mats, int planes) {
+    const int64_t k = (static_cast<int64_t>(max_n) + 31) & ~int64_t(31);
+    return static_cast<size_t>(mats * k * k * 8 + planes * slice_bytes(k));
 }
 
-cudaError_t launch_ns_fp64(const NsFp64Args& a, int max_nblk, cudaStream_t st) {
-    const size_t smem = sizeof(int) * (static_cast<size_t>(max_nblk) + 1);
-    k_ns_fp64<<<a.n_subs, 256, smem, st>>>(a);
+template <class K, class A>
+static cudaError_t launch_form(K kernel, const A& a, int slots, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSliceSmem));
+    if (e != cudaSuccess) return e;
+    kernel<<<slots, kSliceThreads, kSliceSmem, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, cudaStream_t st) {
-    k_nonorth_setup<<<a.n_subs, 256, 0, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_nblk, cudaStream_t st) {
+    if (sizeof(int) * (static_cast<size_t>(max_nblk) + 1) > kSliceSmem - 1024) return cudaErrorInvalidValue;
+    switch (a.function) {
+        case kFnDensity: return launch_form(k_ns_fp64<kFormSign>, a, slots, st);
+        case kFnFermi: return launch_form(k_ns_fp64<kFormFermi>, a, slots, st);
+        default: return launch_form(k_ns_fp64<kFormRoots>, a, slots, st);
+    }
+}
+
+cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, cudaStream_t st) {
+    return launch_form(k_nonorth_setup, a, slots, st);
 }
 
 }  // namespace smx
@@ -642,63 +960,44 @@ constexpr int64_t kNoAllocMat = int64_t(kNoAllocMaxN) * kNoAllocMaxN;
 constexpr int kNoAllocMaxDevices = 64;
 }  // namespace
 
-// X, Y, Z work matrices (n x n each, leading dimension n) followed by a small
-// header: [0] status, [1] iterations.  3 * 256^2 + 4 doubles, about 1.5 MiB.
-static __device__ __align__(256) double g_noalloc_scratch[3 * kNoAllocMat + 4];
+// The slot of one CTA (two matrices of 64-bit integers and the digits of two operands) for n = 256,
+// followed by a small header: [0] status, [1] iterations.  About 2.8 MiB.
+constexpr int64_t kNoAllocBytes = 2 * kNoAllocMat * 8 + 2 * slice_bytes(kNoAllocMaxN);
+static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes + 32];
 
-// One CTA: D = 1/2 (I - sign(H - mu I)) of a dense symmetric H by the FP64
-// Newton-Schulz iteration of k_ns_fp64, with the Gershgorin bound for X0.
-__global__ void __launch_bounds__(256) k_dense_density_noalloc(const double* __restrict__ H, int n, double mu,
-                                                               double* __restrict__ Dout, double* scratch,
-                                                               double tau, int max_iter) {
-    __shared__ double As[kKc][kTile + 1];
-    __shared__ double Bs[kKc][kTile + 1];
-    __shared__ double red[32];
-    double* X = scratch;
-    double* Y = scratch + kNoAllocMat;
-    double* Z = scratch + 2 * kNoAllocMat;
-    int* hdr = reinterpret_cast<int*>(scratch + 3 * kNoAllocMat);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// One CTA: D = 1/2 (I - sign(H - mu I)) of a dense symmetric H by the iteration of k_ns_fp64.
+__global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(const double* __restrict__ H, int n, double mu,
+                                                                            double* __restrict__ Dout, uint8_t* scratch,
+                                                                            float tau, int max_iter) {
+    __shared__ SliceShared shared;
+    __shared__ SliceScalars ss;
+    __shared__ SignBound sb;
+    int* hdr = reinterpret_cast<int*>(scratch + kNoAllocBytes);
+    if (threadIdx.x == 0) hdr[0] = kOk;
+    SliceShared* const sh = &shared;
+    slices_begin(sh, slice_stages(), hdr);
     // every call overwrites the work matrices in full; nothing is carried over
-
-    // Gershgorin bound b = max_r sum_c |H_rc - mu delta_rc| (>= spectral radius)
-    double m = 0.0;
-    for (int r = warp; r < n; r += 8) {
-        double acc = 0.0;
-        for (int c = lane; c < n; c += 32) acc += fabs(H[static_cast<int64_t>(r) * n + c] - (r == c ? mu : 0.0));
-        m = fmax(m, warp_sum(acc));
-    }
-    if (lane == 0) red[warp] = m;
+    __shared__ SliceJob jb;
+    if (threadIdx.x == 0) slice_job(jb, scratch, n, kNoAllocMaxN, 2);
     __syncthreads();
-    double b = 0.0;
-    for (int w = 0; w < 8; ++w) b = fmax(b, red[w]);
-    if (b == 0.0) b = 1.0;
-    __syncthreads();
-    const double inv_b = 1.0 / b;
-    for (int64_t e = threadIdx.x; e < static_cast<int64_t>(n) * n; e += blockDim.x) {
-        const int r = static_cast<int>(e / n), c = static_cast<int>(e - static_cast<int64_t>(r) * n);
-        X[e] = (H[e] - (r == c ? mu : 0.0)) * inv_b;
-    }
-    __syncthreads();
-
+    const int e = load_fixed(H, n, mu, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
+    bool conv = false, bad = ss.bad != 0;
     int done = 0;
-    bool conv = false, bad = false;
-    for (int it = 0; it < max_iter; ++it) {
-        double r2 = gemm_fp64(X, X, Y, n, n, 1, As, Bs);
-        r2 = block_sum(r2, red);
-        gemm_fp64(X, Y, Z, n, n, 2, As, Bs);
-        __syncthreads();
-        double* t = X; X = Z; Z = t;
-        done = it + 1;
-        if (!isfinite(r2)) { bad = true; break; }
-        if (sqrt(r2) <= tau) { conv = true; break; }
+    if (!bad) done = sign_steps(sh, jb, e, max_iter, tau, 0, nullptr, &sb, &ss, conv, bad);
+    const bool aborted = *static_cast<volatile int*>(&sh->abort) != 0;
+    if (!aborted) {
+        const int64_t* X = jb.M[0];
+        for (int r = threadIdx.x >> 5; r < n; r += kSliceWarps)
+            for (int c = threadIdx.x & 31; c < n; c += 32) {  // 1/2 (I - X) in units of 2^-63: up to 2^63
+                const int64_t x = X[mat_at(jb.k, c, r)], one = r == c ? kFixedOne : 0;
+                const bool negative = x > one;
+                const uint64_t d = static_cast<uint64_t>(one) - static_cast<uint64_t>(x);
+                Dout[static_cast<int64_t>(r) * n + c] = fixed_to_double(negative ? 0 - d : d, negative, -63);
+            }
     }
-    for (int64_t e = threadIdx.x; e < static_cast<int64_t>(n) * n; e += blockDim.x) {
-        const int r = static_cast<int>(e / n), c = static_cast<int>(e - static_cast<int64_t>(r) * n);
-        Dout[e] = 0.5 * ((r == c ? 1.0 : 0.0) - X[e]);
-    }
+    slices_end(sh);
     if (threadIdx.x == 0) {
-        hdr[0] = bad ? kErrNonfinite : (conv ? kOk : kErrNoconv);
+        if (!aborted) hdr[0] = bad ? kErrNonfinite : (conv ? kOk : kErrNoconv);
         hdr[1] = done;
     }
 }
@@ -708,7 +1007,7 @@ __global__ void __launch_bounds__(256) k_dense_density_noalloc(const double* __r
 namespace {
 std::mutex g_noalloc_mutex;
 // per device: the array's device address and the context it was looked up in
-double* g_noalloc_ptr[smx::kNoAllocMaxDevices] = {};
+uint8_t* g_noalloc_ptr[smx::kNoAllocMaxDevices] = {};
 CUcontext g_noalloc_ctx[smx::kNoAllocMaxDevices] = {};
 
 // The current driver context, through the runtime's driver entry point (no link to libcuda).
@@ -735,7 +1034,7 @@ extern "C" smx_status smx_dense_density_noalloc(const double* h_dev, int32_t n, 
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return SMX_ERR_CUDA;
     if (dev < 0 || dev >= smx::kNoAllocMaxDevices) return SMX_ERR_UNSUPPORTED;
-    double* scratch = nullptr;
+    uint8_t* scratch = nullptr;
     {
         // set-up once per device, with that device current: the host-side name
         // of a __device__ array is not a device address, so look the address up.
@@ -746,16 +1045,19 @@ extern "C" smx_status smx_dense_density_noalloc(const double* h_dev, int32_t n, 
         if (!g_noalloc_ptr[dev] || g_noalloc_ctx[dev] != cur) {
             void* p = nullptr;
             if (cudaGetSymbolAddress(&p, smx::g_noalloc_scratch) != cudaSuccess || !p) return SMX_ERR_CUDA;
-            g_noalloc_ptr[dev] = static_cast<double*>(p);
+            if (cudaFuncSetAttribute(smx::k_dense_density_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(smx::kSliceSmem)) != cudaSuccess)
+                return SMX_ERR_CUDA;
+            g_noalloc_ptr[dev] = static_cast<uint8_t*>(p);
             g_noalloc_ctx[dev] = cur;
         }
         scratch = g_noalloc_ptr[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    smx::k_dense_density_noalloc<<<1, 256, 0, st>>>(h_dev, n, mu, d_dev, scratch, 1e-7, 100);
+    smx::k_dense_density_noalloc<<<1, smx::kSliceThreads, smx::kSliceSmem, st>>>(h_dev, n, mu, d_dev, scratch, 1e-7f, 100);
     if (cudaGetLastError() != cudaSuccess) return SMX_ERR_CUDA;
     int hdr[2] = {0, 0};
-    if (cudaMemcpyAsync(hdr, scratch + 3 * smx::kNoAllocMat, sizeof(hdr), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if (cudaMemcpyAsync(hdr, scratch + smx::kNoAllocBytes, sizeof(hdr), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return SMX_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return SMX_ERR_CUDA;
     return static_cast<smx_status>(hdr[0]);

@@ -101,7 +101,7 @@ struct smx_ctx {
     DevBuf d_sc;                      // DevScalars: status, flags, bracket, trace and energy
     DevScalars* h_sc = nullptr;       // pinned copy, filled by fetch()
     DevBuf d_fcol_ptr, d_frow_idx, d_fvoff, d_lstart, d_subs, d_order, d_maps, d_map_off;
-    DevBuf d_T, d_W1, d_W2, d_W3, d_W4, d_ws, d_D, d_xown;
+    DevBuf d_T, d_W1, d_ws, d_ws64, d_D, d_xown;
     DevBuf d_bound, d_iters, d_partial, d_work_n3;
     uint8_t* h_keep_pinned = nullptr;
 
@@ -520,6 +520,13 @@ static smx_status gather_chunk(smx_ctx* c, int j0, int m, double mu, const Gathe
 
 static smx_status read_status(smx_ctx* c);
 
+// Slots of the 64-bit kernels for m submatrices: one per persistent CTA (at most one per SM).
+static smx_status prepare_fp64_slots(smx_ctx* c, int m, int mats, int planes, int* slots, size_t* slot_bytes) {
+    *slots = std::max(1, std::min(c->num_sms, m));
+    *slot_bytes = fp64_slot_bytes(c->max_n, mats, planes);
+    return ensure(c->d_ws64, *slot_bytes * static_cast<size_t>(*slots));
+}
+
 // Setup of the non-orthogonal form for the current (H, S) and filtered pattern:
 // A_S and A_H gathered without shift, L_j = A_S^-1/2 and M_j = L_j A_H L_j kept
 // for every block column, and the bisection bracket from the Gershgorin
@@ -528,15 +535,14 @@ static smx_status nonorth_setup(smx_ctx* c) {
     if (c->chunk_start.size() != 2) return SMX_ERR_UNSUPPORTED;  // L_j and M_j of every column stay resident
     cudaStream_t st = c->stream;
     const size_t tb = static_cast<size_t>(c->t_elems) * sizeof(double);
-    SMX_TRY(ensure(c->d_T, tb));
-    SMX_TRY(ensure(c->d_W1, tb));
-    SMX_TRY(ensure(c->d_W2, tb));
-    SMX_TRY(ensure(c->d_W3, tb));
     SMX_TRY(ensure(c->d_Lc, tb));
     SMX_TRY(ensure(c->d_Mc, tb));
     SMX_TRY(ensure(c->d_nlohi, sizeof(double) * 2 * c->B));
     SMX_TRY(ensure(c->d_setup_iters, sizeof(int32_t) * c->B));
     const int j0 = c->chunk_start[0], m = c->chunk_start[1] - j0;
+    int slots = 0;
+    size_t slot_bytes = 0;
+    SMX_TRY(prepare_fp64_slots(c, m, kFp64Mats, kFp64Planes, &slots, &slot_bytes));
     const PatternView pv = pattern_view(c);
     SubDesc* subs = dp<SubDesc>(c->d_subs) + j0;
     GatherExtras ex;
@@ -545,24 +551,27 @@ static smx_status nonorth_setup(smx_ctx* c) {
     SMX_CUDA(launch_gather_bound(subs, m, c->max_nblk, c->max_n, c->bmax, c->bsize_uniform, pv, dp<double>(c->d_H), 0.0, dp<double>(c->d_Mc),
                                  dp<double>(c->d_gersh) + j0, ex, st));
     NonorthSetupArgs a;
-    a.subs = subs;
+    a.subs = dp<SubDesc>(c->d_subs);  // indexed by block column through the order slice
+    a.order = dp<int32_t>(c->d_order) + j0;
     a.n_subs = m;
+    a.work_counter = &scalars(c)->ns_counter;
+    a.ticket = &scalars(c)->fp64_done;
+    a.ws = dp<uint8_t>(c->d_ws64);
+    a.slot_bytes = static_cast<int64_t>(slot_bytes);
+    a.kmax = static_cast<int>(round_up(c->max_n, 32));
+    a.mats = kFp64Mats;
     a.Lc = dp<double>(c->d_Lc);
     a.Mc = dp<double>(c->d_Mc);
-    a.T = dp<double>(c->d_T);
-    a.W1 = dp<double>(c->d_W1);
-    a.W2 = dp<double>(c->d_W2);
-    a.W3 = dp<double>(c->d_W3);
-    a.bound_s = dp<double>(c->d_bound) + j0;
+    a.bound_s = dp<double>(c->d_bound);
     a.tau = tau_for(SMX_FP64);
     a.max_iter = 100;
     a.iters = dp<int32_t>(c->d_setup_iters);
     a.lohi = dp<double>(c->d_nlohi);
     a.status = &scalars(c)->status;
-    SMX_CUDA(launch_nonorth_setup(a, st));
+    SMX_CUDA(launch_nonorth_setup(a, slots, st));
     c->kernel_launches += 3;
     std::vector<double> lohi(2 * static_cast<size_t>(m));
-    SMX_CUDA(cudaMemcpyAsync(lohi.data(), c->d_nlohi.p, sizeof(double) * lohi.size(), cudaMemcpyDeviceToHost, st));
+    SMX_CUDA(cudaMemcpyAsync(lohi.data(), dp<double>(c->d_nlohi) + 2 * j0, sizeof(double) * lohi.size(), cudaMemcpyDeviceToHost, st));
     const smx_status ds = read_status(c);  // synchronises
     if (ds != SMX_OK) return ds;
     double lo = lohi[0], hi = lohi[1];
@@ -595,23 +604,49 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
     const bool model = c->model_on && c->function == SMX_FN_DENSITY && !c->have_S;  // other forms start from G_j
     SMX_CUDA(cudaEventRecord(c->ev0, st));
     const PatternView pv = pattern_view(c);
-    if (c->precision == SMX_FP64) {
-        const size_t tb = static_cast<size_t>(c->t_elems) * sizeof(double);
-        SMX_TRY(ensure(c->d_T, tb));
-        SMX_TRY(ensure(c->d_W1, tb));
-        SMX_TRY(ensure(c->d_W2, tb));
-        if (c->function != SMX_FN_DENSITY) SMX_TRY(ensure(c->d_W3, tb));
-        if (c->function == SMX_FN_FERMI) SMX_TRY(ensure(c->d_W4, tb));
-    } else {
+    const bool finish = c->precision != SMX_FP64 && c->fp64_final > 0 && c->function == SMX_FN_DENSITY;
+    // matrices and digit planes of a 64-bit slot: the sign iteration two of each (the non-orthogonal
+    // form three operands), the function forms three of each
+    const int mats = c->function == SMX_FN_DENSITY ? 2 : kFp64Mats;
+    const int planes = c->function == SMX_FN_DENSITY && !c->have_S ? 2 : kFp64Planes;
+    int max_m = 0, slots = 0;
+    for (size_t k = 0; k + 1 < c->chunk_start.size(); ++k) max_m = std::max(max_m, c->chunk_start[k + 1] - c->chunk_start[k]);
+    size_t slot_bytes = 0;
+    if (c->precision == SMX_FP64 || finish) SMX_TRY(prepare_fp64_slots(c, max_m, mats, planes, &slots, &slot_bytes));
+    if (c->precision != SMX_FP64) {
         SMX_TRY(prepare_tc_workspace(c));
         SMX_TRY(ensure(c->d_xown, static_cast<size_t>(c->x_elems) * sizeof(float)));
-        if (c->fp64_final > 0) {  // the bulk phase's last iterate in FP64, and two work buffers
-            const size_t tb = static_cast<size_t>(c->t_elems) * sizeof(double);
-            SMX_TRY(ensure(c->d_W1, tb));
-            SMX_TRY(ensure(c->d_W2, tb));
-            SMX_TRY(ensure(c->d_W3, tb));
-        }
+        if (finish)  // the bulk phase's last iterate in FP64
+            SMX_TRY(ensure(c->d_W1, static_cast<size_t>(c->t_elems) * sizeof(double)));
     }
+    // what every launch of the 64-bit kernel in this build has in common
+    auto fp64_args = [&](int j0, int m) {
+        NsFp64Args a;
+        a.subs = dp<SubDesc>(c->d_subs);  // indexed by block column through the order slice
+        a.order = dp<int32_t>(c->d_order) + j0;
+        a.n_subs = m;
+        a.work_counter = &sc->ns_counter;
+        a.ticket = &sc->fp64_done;
+        a.ws = dp<uint8_t>(c->d_ws64);
+        a.slot_bytes = static_cast<int64_t>(slot_bytes);
+        a.kmax = static_cast<int>(round_up(c->max_n, 32));
+        a.mats = mats;
+        a.function = c->function;
+        a.bound = dp<double>(c->d_bound);
+        a.tau = tau_for(SMX_FP64);
+        a.iters = dp<int32_t>(c->d_iters);
+        a.work_n3 = dp<unsigned long long>(c->d_work_n3);
+        a.gersh = dp<double>(c->d_gersh);
+        a.sq_ratio = dp<float>(c->d_sq_ratio);
+        a.fallbacks = &sc->fallbacks;
+        a.status = &sc->status;
+        a.pv = pv;
+        a.H = dp<double>(c->d_H);
+        a.D = dp<double>(c->d_D);
+        a.partial = dp<double2>(c->d_partial);
+        a.skip = skip;
+        return a;
+    };
     SubDesc* subs = dp<SubDesc>(c->d_subs);
     // one pass of a3-a7 per chunk of block columns (the staging of T_j is reused)
     for (size_t k = 0; k + 1 < c->chunk_start.size(); ++k) {
@@ -630,32 +665,12 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
         cudaEvent_t ns0, ns1;
         SMX_TRY(ns_event_pair(c, &ns0, &ns1));
         if (c->precision == SMX_FP64) {
-            NsFp64Args a;
-            a.subs = subs + j0;
-            a.n_subs = m;
+            NsFp64Args a = fp64_args(j0, m);
             a.T = dp<double>(c->d_T);
-            a.W1 = dp<double>(c->d_W1);
-            a.W2 = dp<double>(c->d_W2);
-            a.W3 = c->function != SMX_FN_DENSITY ? dp<double>(c->d_W3) : nullptr;
-            a.W4 = c->function == SMX_FN_FERMI ? dp<double>(c->d_W4) : nullptr;
             a.beta = c->beta;
-            a.function = c->function;
-            a.bound = dp<double>(c->d_bound) + j0;
-            a.tau = tau_for(SMX_FP64);
             a.max_iter = 100;
-            a.iters = dp<int32_t>(c->d_iters);
-            a.work_n3 = dp<unsigned long long>(c->d_work_n3);
-            a.gersh = dp<double>(c->d_gersh) + j0;
-            a.sq_ratio = dp<float>(c->d_sq_ratio) + j0;
             a.use_model = model ? 1 : 0;
-            if (model && c->model_gap) a.pred = dp<float>(c->d_pred) + 2 * j0;
-            a.skip = skip;
-            a.fallbacks = &sc->fallbacks;
-            a.status = &sc->status;
-            a.pv = pv;
-            a.H = dp<double>(c->d_H);
-            a.D = dp<double>(c->d_D);
-            a.partial = dp<double2>(c->d_partial);
+            if (model && c->model_gap) a.pred = dp<float>(c->d_pred);
             if (c->have_S) {
                 a.Mc = dp<double>(c->d_Mc);
                 a.Lc = dp<double>(c->d_Lc);
@@ -663,7 +678,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
                 a.mu = mu;
             }
             SMX_CUDA(cudaEventRecord(ns0, st));
-            SMX_CUDA(launch_ns_fp64(a, c->max_nblk, st));
+            SMX_CUDA(launch_ns_fp64(a, std::min(slots, m), c->max_nblk, st));
             SMX_CUDA(cudaEventRecord(ns1, st));
         } else {
             NsTcArgs a;
@@ -693,7 +708,6 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
             a.D = dp<double>(c->d_D);
             a.partial = dp<double2>(c->d_partial);
             a.xown = dp<float>(c->d_xown);
-            const bool finish = c->fp64_final > 0 && c->function == SMX_FN_DENSITY;
             if (finish) a.xfull = dp<double>(c->d_W1);
             SMX_CUDA(cudaEventRecord(ns0, st));
             SMX_CUDA(launch_ns_tc(a, c->precision, c->tmap, c->max_nblk, st));
@@ -701,31 +715,12 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
                 // FP64 finishing steps on the bulk phase's last iterate, then the scatter (the
                 // tensor-core scatter, which also resets the job counter, is not run)
                 SMX_CUDA(cudaMemsetAsync(&sc->ns_counter, 0, sizeof(int), st));
-                NsFp64Args f;
-                f.subs = subs + j0;
-                f.n_subs = m;
+                NsFp64Args f = fp64_args(j0, m);
                 f.T = dp<double>(c->d_W1);
-                f.W1 = dp<double>(c->d_W2);
-                f.W2 = dp<double>(c->d_W3);
-                f.W3 = nullptr;
-                f.function = SMX_FN_DENSITY;
-                f.bound = dp<double>(c->d_bound) + j0;
-                f.tau = tau_for(SMX_FP64);
                 f.max_iter = c->fp64_final;
-                f.iters = dp<int32_t>(c->d_iters);
-                f.work_n3 = dp<unsigned long long>(c->d_work_n3);
-                f.gersh = dp<double>(c->d_gersh) + j0;
-                f.sq_ratio = dp<float>(c->d_sq_ratio) + j0;
                 f.use_model = 0;
-                f.fallbacks = &sc->fallbacks;
-                f.status = &sc->status;
-                f.pv = pv;
-                f.H = dp<double>(c->d_H);
-                f.D = dp<double>(c->d_D);
-                f.partial = dp<double2>(c->d_partial);
                 f.finish_iters = c->fp64_final;
-                f.skip = skip;
-                SMX_CUDA(launch_ns_fp64(f, c->max_nblk, st));
+                SMX_CUDA(launch_ns_fp64(f, std::min(slots, m), c->max_nblk, st));
                 c->kernel_launches += 1;
             }
             SMX_CUDA(cudaEventRecord(ns1, st));
@@ -738,7 +733,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
         c->kernel_launches += 1;
         c->ns_launches += 1;
     }
-    if (c->precision == SMX_FP64 || (c->fp64_final > 0 && c->function == SMX_FN_DENSITY)) {
+    if (c->precision == SMX_FP64 || finish) {
         // the tensor-core scatter sums the partials itself
         SMX_CUDA(launch_reduce(dp<double2>(c->d_partial), B, sc, st, skip));
         c->kernel_launches += 1;
@@ -1488,7 +1483,7 @@ void smx_destroy(smx_ctx* c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     DevBuf* bufs[] = {&c->d_H, &c->d_H32, &c->d_voff, &c->d_row_idx, &c->d_col_ptr, &c->d_bs, &c->d_keep_prev, &c->d_sc, &c->d_keep, &c->d_fcol_ptr,
                       &c->d_frow_idx, &c->d_fvoff, &c->d_lstart, &c->d_subs, &c->d_order, &c->d_T, &c->d_W1,
-                      &c->d_W2, &c->d_W3, &c->d_W4, &c->d_ws, &c->d_D, &c->d_xown, &c->d_bound, &c->d_iters, &c->d_partial,
+                      &c->d_ws, &c->d_ws64, &c->d_maps, &c->d_map_off, &c->d_pairs, &c->d_D, &c->d_xown, &c->d_bound, &c->d_iters, &c->d_partial,
                       &c->d_work_n3,
                       &c->d_params, &c->d_mst, &c->d_vst, &c->d_partial_mlp, &c->d_feat, &c->d_pred, &c->d_labels,
                       &c->d_gersh, &c->d_prev_ratio, &c->d_sq_ratio, &c->d_loss, &c->d_sx, &c->d_st,

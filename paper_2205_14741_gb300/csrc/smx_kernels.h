@@ -19,8 +19,8 @@ struct DevScalars {
     int status;            // first error recorded by a kernel (kOk = 0)
     int changed;           // the keep flags differ from the current filtered pattern
     int fallbacks;         // learned-bound fallbacks since the last reset
-    int ns_counter;        // job counter of the tensor-core Newton-Schulz kernel (reset by the scatter)
-    unsigned int filter_done, scatter_done;  // last-block tickets (each reset by its last block)
+    int ns_counter;        // job counter of the Newton-Schulz kernels (reset by the scatter or the FP64 kernel's last CTA)
+    unsigned int filter_done, scatter_done, fp64_done;  // last-block tickets (each reset by its last block)
     unsigned long long nlo_enc, hi_enc;      // filter: running bracket as order-preserving images (reset by its last block)
     int bis_done;          // device-side bisection: stopped (the later builds are skipped)
     int bis_steps;         // ... builds evaluated
@@ -84,21 +84,30 @@ cudaError_t launch_symmetrize(const SymPair* pairs, int n_pairs, const uint8_t* 
 // poll_limit polls (records kErrTimeout in *status; *polls_out, if set, the polls made).
 cudaError_t launch_wait_selftest(int* status, uint32_t poll_limit, int* polls_out, cudaStream_t st);
 
-// a5/a6 (FP64 plain form) + a7: Newton-Schulz in FP64, then scatter.
+// a5/a6 (FP64 plain form) + a7: Newton-Schulz in 64-bit arithmetic, then scatter.
 // Matrix function of a build (values of smx_function): 0 = the density matrix
 // 1/2 (I - sign(A)), 1 = A^-1/2, 2 = A^1/2 (A = T_j - mu I symmetric positive definite).
 enum : int { kFnDensity = 0, kFnInvSqrt = 1, kFnSqrt = 2, kFnInv = 3, kFnFermi = 4 };
 
+// A CTA of the 64-bit kernels works in a slot of global memory: up to three k x k matrices of 64-bit
+// integers and the digits of up to three operands (smx_slices.cuh).
+constexpr int kFp64Mats = 3, kFp64Planes = 3;
+// Bytes of a slot for submatrices of up to max_n rows.
+size_t fp64_slot_bytes(int max_n, int mats, int planes);
+
 struct NsFp64Args {
     const SubDesc* subs;
+    const int32_t* order;  // processing order (largest first)
     int n_subs;
-    double* T;   // FP64 staging buffer (overwritten: X0 = T / b)
-    double* W1;  // FP64 work buffers laid out like T
-    double* W2;
-    double* W3;  // a third one for the function forms (coupled iteration), else unused
-    double* W4 = nullptr;  // a fourth one for the Fermi function
-    int function;  // kFnDensity, kFnInvSqrt or kFnSqrt
-    double* bound;  // in: initial bound b_j; out: effective bound after the a-posteriori rescale
+    int* work_counter;     // job counter and last-CTA ticket, zero at launch (the kernel leaves them so)
+    unsigned int* ticket;
+    const double* T;       // FP64 staging of T_j - mu I (finishing steps: the bulk phase's last iterate)
+    uint8_t* ws;           // slots
+    int64_t slot_bytes;
+    int kmax;              // largest dimension rounded up to 32
+    int mats;              // matrices per slot (the digit planes follow them)
+    int function;          // kFnDensity .. kFnFermi
+    double* bound;         // in: initial bound b_j; out: effective bound after the a-posteriori rescale
     double tau;
     int max_iter;
     int32_t* iters;
@@ -119,37 +128,39 @@ struct NsFp64Args {
     const double* Lc = nullptr;  // L_j = A_S^-1/2, laid out like T
     const double* Sv = nullptr;  // S in the input value layout
     double mu = 0.0;
-    // learned bound: predictions of this chunk ([2 i + 1] = delta_hat / G for the i-th
-    // submatrix); see NsTcArgs::pred
+    // learned bound: predictions per block column ([2 j + 1] = delta_hat / G_j); see NsTcArgs::pred
     const float* pred = nullptr;
     // FP64 finishing steps after a low-precision bulk phase (> 0): T holds the bulk phase's last
-    // iterate X (not T_j - mu I); exactly this many plain steps in FP64, then the scatter; the
-    // steps are added to iters
+    // iterate X (not T_j - mu I); exactly this many plain steps, then the scatter; the steps are
+    // added to iters
     int finish_iters = 0;
     const int* skip = nullptr;  // when set and non-zero at launch, the kernel does nothing
     double beta = 0.0;          // kFnFermi: the inverse temperature (in inverse units of H)
 };
-cudaError_t launch_ns_fp64(const NsFp64Args& a, int max_nblk, cudaStream_t st);
+cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_nblk, cudaStream_t st);
 
 // Setup of the non-orthogonal form, once per (H, S): L_j = A_S^-1/2 (coupled iteration) and
-// M_j = L_j A_H L_j with its Gershgorin interval, a CTA per submatrix.
+// M_j = L_j A_H L_j with its Gershgorin interval.
 struct NonorthSetupArgs {
     const SubDesc* subs;
+    const int32_t* order;
     int n_subs;
+    int* work_counter;
+    unsigned int* ticket;
+    uint8_t* ws;
+    int64_t slot_bytes;
+    int kmax;
+    int mats;
     double* Lc;             // in: A_S = S[R_j, R_j]; out: L_j
-    double* Mc;             // in: A_H = H[R_j, R_j]; out: M_j (symmetrised)
-    double* T;              // work buffers laid out like Lc
-    double* W1;
-    double* W2;
-    double* W3;
+    double* Mc;             // in: A_H = H[R_j, R_j]; out: M_j (symmetric)
     const double* bound_s;  // Gershgorin bound of A_S (>= its largest eigenvalue)
     double tau;
     int max_iter;
     int32_t* iters;         // out: steps of the coupled iteration per block column
-    double* lohi;           // out: [2 * n_subs] Gershgorin interval of M_j
+    double* lohi;           // out: [2 * B] Gershgorin interval of M_j
     int* status;
 };
-cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, cudaStream_t st);
+cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, cudaStream_t st);
 
 // a5 (tcgen05 tensor cores) + a7.
 struct NsTcArgs {
