@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         // row tile mt: N tiles of up to NT columns from column 128 mt
         auto ntiles_of = [&](int mt) { return (kpad - 128 * mt + NT - 1) / NT; };
         if (warp == 0) {
-            if (lane == 0) {
+            if (elect_one()) {
                 for (int mt = 0; mt < mtiles && !*abortp; ++mt)
                     for (int nt = 0; nt < ntiles_of(mt) && !*abortp; ++nt) {
                         const int n0 = 128 * mt + NT * nt, nn = min(NT, kpad - n0);
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             }
             __syncwarp();
         } else if (warp == 1) {
-            if (lane == 0) {
+            if (elect_one()) {
                 for (int mt = 0; mt < mtiles && !*abortp; ++mt)
                     for (int nt = 0; nt < ntiles_of(mt) && !*abortp; ++nt) {
                         const int nn = min(NT, kpad - 128 * mt - NT * nt);
@@ -1085,7 +1085,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     // on the scaled schedule 3/a^2 and -a^3/2
                     float alpha = -0.5f, shift = 3.0f;
                     if (it > 0) next_step(shift, alpha);
-                    if (warp == 1 && lane == 0) {
+                    if (warp == 1 && elect_one()) {
                         tc_fence_after();
                         issue_xx(0, TA);
                         tc_commit(&mma_bar);
@@ -1107,7 +1107,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     if (lane == 0) resid_s2[warp] = r2;
                     tc_fence_before();
                     __syncthreads();
-                    if (warp == 1 && lane == 0) {
+                    if (warp == 1 && elect_one()) {
                         tc_fence_after();
                         issue_yx(TA, TB);
                         tc_commit(&mma_bar);
@@ -1149,7 +1149,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                 for (int it = 0; it < a.max_iter; ++it) {
                     float alpha = -0.5f, shift = 3.0f;
                     if (it > 0) next_step(shift, alpha);
-                    if (it == 0 && warp == 1 && lane == 0) {  // later iterations: issued at the end of the previous one
+                    if (it == 0 && warp == 1 && elect_one()) {  // later iterations: issued at the end of the previous one
                         tc_fence_after();
                         issue_xx(0, TA);
                         tc_commit(&mma_bar);
@@ -1176,7 +1176,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     fence_proxy_async_smem();  // Bz rows 0 .. 127 (read by Q_c's products)
                     tc_fence_before();
                     __syncthreads();
-                    if (warp == 1 && lane == 0) {
+                    if (warp == 1 && elect_one()) {
                         tc_fence_after();
                         issue_yx(TA, TC);
                         tc_commit(&mma_bar);
@@ -1189,7 +1189,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     tc_fence_before();
                     __syncthreads();
                     if (*abortp) break;
-                    if (warp == 1 && lane == 0) {
+                    if (warp == 1 && elect_one()) {
                         tc_fence_after();
                         issue_cyx(TB);
                         tc_commit(&mma_bar2);
@@ -1208,13 +1208,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     // X_0 in TC are final) while rows 128 .. are written; issued by warp 10, which
                     // has no rows or chunks in the two passes below, so its wait for the MMA queue
                     // delays no pass
-                    if (!last && warp == 10 && lane == 0) issue_yx_k(TC, TA, 0, 8);
+                    if (!last && warp == 10 && elect_one()) issue_yx_k(TC, TA, 0, 8);
                     drain_t(TC);
                     drain_corner(TB, alpha);
                     fence_proxy_async_smem();
                     tc_fence_before();
                     __syncthreads();
-                    if (!last && warp == 10 && lane == 0) {
+                    if (!last && warp == 10 && elect_one()) {
                         tc_fence_after();
                         issue_yx_k(TC, TA, 8, ksteps);  // K rows 128 ..
                         tc_commit(&mma_bar);
@@ -1414,7 +1414,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         for (int it = m_consumed_s; it < p_issued_s; ++it)
             mbar_wait_plain(&full_bar[it % S], (it / S) & 1, 1u << 20);
     }
-    if (*abortp && warp == 1 && lane == 0) {
+    if (*abortp && warp == 1 && elect_one()) {
         tc_commit(&drain_bar);
         mbar_wait_plain(&drain_bar, 0, 1u << 20);
     }
