@@ -24,6 +24,8 @@ namespace {
 constexpr int kF = kModelFeatures, kH = kModelHidden, kO = 2;
 
 constexpr int kChunk = 64;  // samples per gradient block
+constexpr int kGradThreads = 1024;
+constexpr int kHs = kH + 1;  // row stride of W2 and h2 in shared memory: a column's entries lie in different banks
 
 __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
@@ -38,41 +40,75 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 // ---------------------------------------------------------------------------
 namespace {
 
-// number of eigenvalues below x of the symmetric tridiagonal (a, b), b[0] unused
-__device__ int sturm_count(const double* a, const double* b, int k, double x) {
-    int cnt = 0;
-    double q = 1.0;
-    for (int i = 0; i < k; ++i) {
-        const double bb = i ? b[i] * b[i] : 0.0;
-        q = (a[i] - x) - (i ? bb / q : 0.0);
-        if (q == 0.0) q = -1e-300;
-        if (q < 0.0) ++cnt;
-    }
-    return cnt;
-}
-
-// i-th smallest eigenvalue (0-based) of the tridiagonal by bisection
-__device__ double tridiag_eig(const double* a, const double* b, int k, int i) {
+// The i-th smallest eigenvalue (0-based) of the symmetric tridiagonal with diagonal a and off-diagonal
+// b (b[0] unused), k <= kMaxLanczos, by one warp: each round counts the eigenvalues below 32 points of the
+// current interval, a point per lane, and keeps the part that holds the i-th.  FP64 instructions take
+// about 16 cycles per warp here however many lanes are active, so a round costs what one step of a
+// bisection would and gains log2(33) bits instead of one: 11 rounds for 2^-55 of the starting interval.
+// The count is the number of sign changes in the sequence of leading determinants p_j = (a_j - x) p_{j-1} -
+// b_j^2 p_{j-2} (no division: three FP64 instructions a step), the matrix scaled by a power of two to
+// norm 1 (entries a_j, -b_j^2 in `scaled`, the warp's own k of them) and the sequence rescaled before it
+// can underflow.
+__device__ double tridiag_eig(const double* a, const double* b, int k, int i, double2* scaled) {
+    const int lane = threadIdx.x & 31;
     double lo = 1e300, hi = -1e300;
-    for (int j = 0; j < k; ++j) {
+    for (int j = lane; j < k; j += 32) {
         const double r = (j ? fabs(b[j]) : 0.0) + (j + 1 < k ? fabs(b[j + 1]) : 0.0);
         lo = fmin(lo, a[j] - r);
         hi = fmax(hi, a[j] + r);
     }
-    for (int it = 0; it < 100; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        if (sturm_count(a, b, k, mid) > i) hi = mid; else lo = mid;
+    lo = -warp_max(-lo);
+    hi = warp_max(hi);
+    const int e = ilogb(fmax(fmax(fabs(lo), fabs(hi)), 1e-300)) + 1;
+    const double sc = ldexp(1.0, -e);
+    lo *= sc;
+    hi *= sc;
+    for (int j = lane; j < k; j += 32) {
+        const double bj = j ? b[j] * sc : 0.0;
+        scaled[j] = make_double2(a[j] * sc, -(bj * bj));
     }
-    return 0.5 * (lo + hi);
+    __syncwarp();
+    for (int round = 0; round < 11 && hi > lo; ++round) {
+        const double x = lo + (hi - lo) * (static_cast<double>(lane + 1) * (1.0 / 33.0));
+        double p1 = 1.0, p0 = 0.0;  // p_{j-1}, p_{j-2}
+        int cnt = 0;
+        for (int j = 0; j < k; ++j) {
+            const double2 ab = scaled[j];
+            double p = fma(ab.x - x, p1, ab.y * p0);
+            const int s1 = __double2hiint(p1) >> 31;
+            // an exact zero counts as a sign change
+            if (__double2loint(p) == 0 && (__double2hiint(p) & 0x7fffffff) == 0) p = s1 ? 1e-300 : -1e-300;
+            cnt += (__double2hiint(p) >> 31) != s1;
+            p0 = p1;
+            p1 = p;
+            if ((j & 3) == 3) {  // both small: up by 2^600 (an exponent added on the integer units)
+                const int ex = max((__double2hiint(p0) >> 20) & 0x7ff, (__double2hiint(p1) >> 20) & 0x7ff);
+                if (ex < 400) {
+                    p0 *= 0x1p600;
+                    p1 *= 0x1p600;
+                }
+            }
+        }
+        const unsigned above = __ballot_sync(0xffffffffu, cnt > i);  // the points right of the eigenvalue
+        const int first = above ? __ffs(above) - 1 : 32;
+        const double xl = __shfl_sync(0xffffffffu, x, first > 0 ? first - 1 : 0), xr = __shfl_sync(0xffffffffu, x, first & 31);
+        if (first > 0) lo = xl;
+        if (first < 32) hi = xr;
+    }
+    return ldexp(0.5 * (lo + hi), e);
 }
 
 }  // namespace
 
-template <class R>
+// STAGED: the submatrix is kept in shared memory (as FP32) for the up to 192 matrix-vector products
+// that read it (144 at 48 steps): from L2 they took longer than anything but the eigenvalue searches.
+template <class R, bool STAGED>
 __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ subs, const R* __restrict__ T, int ksteps,
                                                  float* __restrict__ labels) {
-    extern __shared__ float lz[];  // 4 vectors of max_n
+    extern __shared__ float lz[];  // 4 vectors of n, then (STAGED) the submatrix
     __shared__ double alpha[kMaxLanczos], beta[kMaxLanczos + 1];
+    __shared__ double2 scaled[2][kMaxLanczos];
+    __shared__ double eig[2];
     __shared__ float red[8];
     __shared__ float gmax_s;
     const SubDesc s = subs[blockIdx.x];
@@ -82,6 +118,17 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
     float* w = lz + n;
     float* vp = lz + 2 * n;
     float* u = lz + 3 * n;
+    float* ts = lz + 4 * n;
+    if constexpr (STAGED) {
+        for (int r = warp; r < n; r += 8)
+#pragma unroll 4
+            for (int c = lane; c < n; c += 32) ts[r * n + c] = static_cast<float>(t[static_cast<int64_t>(r) * s.ld + c]);
+        __syncthreads();
+    }
+    auto entry = [&](int r, int c) -> float {
+        if constexpr (STAGED) return ts[r * n + c];
+        else return static_cast<float>(t[static_cast<int64_t>(r) * s.ld + c]);
+    };
 
     auto block_sum_f = [&](float x) -> float {
         x = warp_sum_f(x);
@@ -93,13 +140,23 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
         __syncthreads();
         return r;
     };
-    // y = A x (a warp per row)
+    // y = A x (a warp per row, four rows at a time)
     auto matvec = [&](const float* x, float* y) {
-        for (int r = warp; r < n; r += 8) {
-            float acc = 0.f;
-            for (int c = lane; c < n; c += 32) acc = fmaf(static_cast<float>(t[static_cast<int64_t>(r) * s.ld + c]), x[c], acc);
-            acc = warp_sum_f(acc);
-            if (lane == 0) y[r] = acc;
+        for (int r = warp; r < n; r += 32) {
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int c = lane; c < n; c += 32) {
+                const float xc = x[c];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (r + 8 * i < n) acc[i] = fmaf(entry(r + 8 * i, c), xc, acc[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] = warp_sum_f(acc[i]);
+            if (lane == 0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (r + 8 * i < n) y[r + 8 * i] = acc[i];
+            }
         }
         __syncthreads();
     };
@@ -108,7 +165,7 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
         float g = 0.f;
         for (int r = warp; r < n; r += 8) {
             float acc = 0.f;
-            for (int c = lane; c < n; c += 32) acc += fabsf(static_cast<float>(t[static_cast<int64_t>(r) * s.ld + c]));
+            for (int c = lane; c < n; c += 32) acc += fabsf(entry(r, c));
             g = fmaxf(g, warp_sum_f(acc));
         }
         if (lane == 0) red[warp] = g;
@@ -159,13 +216,16 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
             __syncthreads();
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            if (pass == 0) {
-                lam_lo = tridiag_eig(alpha, beta, k, 0);
-                lam_hi = tridiag_eig(alpha, beta, k, k - 1);
-            } else {
-                sq_lo = tridiag_eig(alpha, beta, k, 0);
-            }
+        if (warp < 2 - pass) {  // the two ends of A's spectrum, or the lower end of A^2's, a warp each
+            const double x = tridiag_eig(alpha, beta, k, warp == 0 ? 0 : k - 1, scaled[warp]);
+            if (lane == 0) eig[warp] = x;
+        }
+        __syncthreads();
+        if (pass == 0) {
+            lam_lo = eig[0];
+            lam_hi = eig[1];
+        } else {
+            sq_lo = eig[0];
         }
         __syncthreads();
     }
@@ -182,21 +242,28 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
 
 // Forward + backward for samples [blockIdx.x * 64, +64): per-block gradient sums
 // (sum over the block's samples, in sample order) and half the squared residual.
-__global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ X,
+// Bound by shared-memory reads; with rows of 64 words the lanes of a warp read W2 (a unit each) and h2 (a
+// sample each) from one bank, 32 cycles a read.
+__global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ X,
                                                   const float* __restrict__ Tg, int m, float* __restrict__ partial,
                                                   float* __restrict__ partial_loss) {
     extern __shared__ float sm[];
     float* p = sm;                              // kModelParams
     float* xs = p + kModelParams;               // [64][kF]
     float* h1 = xs + kChunk * kF;               // [64][64]
-    float* h2 = h1 + kChunk * kH;               // [64][64]
-    float* d1 = h2 + kChunk * kH;               // [64][64]  dL/d(pre-activation 1)
+    float* h2 = h1 + kChunk * kH;               // [64][65]
+    float* w2 = h2 + kChunk * kHs;              // [64][65]  W2
+    float* d1 = w2 + kH * kHs;                  // [64][64]  dL/d(pre-activation 1)
     float* d2 = d1 + kChunk * kH;               // [64][64]
     float* dy = d2 + kChunk * kH;               // [64][2]
     float* ls = dy + kChunk * kO;               // [64] half squared residual per sample
     const int s0 = blockIdx.x * kChunk;
     const int cnt = min(kChunk, m - s0);
-    for (int i = threadIdx.x; i < kModelParams; i += blockDim.x) p[i] = params[i];
+    for (int i = threadIdx.x; i < kModelParams; i += blockDim.x) {
+        const float x = params[i];
+        p[i] = x;
+        if (i >= kOffW2 && i < kOffB2) w2[(i - kOffW2) / kH * kHs + (i - kOffW2) % kH] = x;
+    }
     for (int i = threadIdx.x; i < kChunk * kF; i += blockDim.x) {
         const int sidx = i / kF;
         xs[i] = sidx < cnt ? X[static_cast<int64_t>(s0) * kF + i] : 0.f;
@@ -213,8 +280,8 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ para
     for (int e = threadIdx.x; e < kChunk * kH; e += blockDim.x) {
         const int sidx = e / kH, i = e - sidx * kH;
         float a = p[kOffB2 + i];
-        for (int k = 0; k < kH; ++k) a = fmaf(p[kOffW2 + i * kH + k], h1[sidx * kH + k], a);
-        h2[e] = tanhf(a);
+        for (int k = 0; k < kH; ++k) a = fmaf(w2[i * kHs + k], h1[sidx * kH + k], a);
+        h2[sidx * kHs + i] = tanhf(a);
     }
     __syncthreads();
     if (threadIdx.x < kChunk) {
@@ -222,7 +289,7 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ para
         float l = 0.f;
         for (int o = 0; o < kO; ++o) {
             float y = p[kOffB3 + o];
-            for (int k = 0; k < kH; ++k) y = fmaf(p[kOffW3 + o * kH + k], h2[sidx * kH + k], y);
+            for (int k = 0; k < kH; ++k) y = fmaf(p[kOffW3 + o * kH + k], h2[sidx * kHs + k], y);
             const float r = sidx < cnt ? y - Tg[2 * static_cast<int64_t>(s0 + sidx) + o] : 0.f;
             dy[sidx * kO + o] = r;
             l = fmaf(r, r, l);
@@ -239,13 +306,14 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ para
     for (int e = threadIdx.x; e < kChunk * kH; e += blockDim.x) {
         const int sidx = e / kH, i = e - sidx * kH;
         const float g = dy[sidx * kO] * p[kOffW3 + i] + dy[sidx * kO + 1] * p[kOffW3 + kH + i];
-        d2[e] = g * (1.f - h2[e] * h2[e]);
+        const float h = h2[sidx * kHs + i];
+        d2[e] = g * (1.f - h * h);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < kChunk * kH; e += blockDim.x) {
         const int sidx = e / kH, k = e - sidx * kH;
         float g = 0.f;
-        for (int i = 0; i < kH; ++i) g = fmaf(d2[sidx * kH + i], p[kOffW2 + i * kH + k], g);
+        for (int i = 0; i < kH; ++i) g = fmaf(d2[sidx * kH + i], w2[i * kHs + k], g);
         d1[e] = g * (1.f - h1[e] * h1[e]);
     }
     __syncthreads();
@@ -267,7 +335,7 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ para
             for (int sidx = 0; sidx < kChunk; ++sidx) g += d2[sidx * kH + i];
         } else if (q < kOffB3) {
             const int o = (q - kOffW3) / kH, k = (q - kOffW3) - o * kH;
-            for (int sidx = 0; sidx < kChunk; ++sidx) g = fmaf(dy[sidx * kO + o], h2[sidx * kH + k], g);
+            for (int sidx = 0; sidx < kChunk; ++sidx) g = fmaf(dy[sidx * kO + o], h2[sidx * kHs + k], g);
         } else {
             const int o = q - kOffB3;
             for (int sidx = 0; sidx < kChunk; ++sidx) g += dy[sidx * kO + o];
@@ -291,6 +359,7 @@ __global__ void k_mlp_reduce_adam(const float* __restrict__ partial, const float
     }
     if (q >= kModelParams) return;
     float g = 0.f;
+#pragma unroll 8
     for (int b = 0; b < nblocks; ++b) g += partial[static_cast<int64_t>(b) * kModelParams + q];
     g *= inv_m;
     if (grad_out) grad_out[q] = g;
@@ -309,19 +378,23 @@ __global__ void k_mlp_reduce_adam(const float* __restrict__ partial, const float
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+template <class R>
+static cudaError_t launch_lanczos_type(const SubDesc* subs, int n_subs, int max_n, const R* T, int ksteps, float* labels, cudaStream_t st) {
+    const size_t vectors = sizeof(float) * 4 * static_cast<size_t>(max_n), staged = vectors + sizeof(float) * static_cast<size_t>(max_n) * max_n;
+    // up to n = 238 the submatrix fits shared memory (two CTAs per SM up to n = 165)
+    const bool fits = staged <= 225u * 1024u;
+    const size_t smem = fits ? staged : vectors;
+    auto kernel = fits ? k_lanczos<R, true> : k_lanczos<R, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    kernel<<<n_subs, 256, smem, st>>>(subs, T, ksteps, labels);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_lanczos(const SubDesc* subs, int n_subs, int max_n, const void* T, bool fp32, int ksteps,
                            float* labels, cudaStream_t st) {
-    const size_t smem = sizeof(float) * 4 * static_cast<size_t>(max_n);
-    if (fp32) {
-        cudaError_t e = cudaFuncSetAttribute(k_lanczos<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-        k_lanczos<float><<<n_subs, 256, smem, st>>>(subs, static_cast<const float*>(T), ksteps, labels);
-    } else {
-        cudaError_t e = cudaFuncSetAttribute(k_lanczos<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-        k_lanczos<double><<<n_subs, 256, smem, st>>>(subs, static_cast<const double*>(T), ksteps, labels);
-    }
-    return cudaGetLastError();
+    if (fp32) return launch_lanczos_type(subs, n_subs, max_n, static_cast<const float*>(T), ksteps, labels, st);
+    return launch_lanczos_type(subs, n_subs, max_n, static_cast<const double*>(T), ksteps, labels, st);
 }
 
 size_t mlp_partial_floats(int m) { return static_cast<size_t>((m + kChunk - 1) / kChunk) * (kModelParams + 1); }
@@ -332,10 +405,10 @@ cudaError_t launch_mlp_step(const float* params_in, const float* X, const float*
     if (m <= 0) return cudaErrorInvalidValue;
     const int nb = (m + kChunk - 1) / kChunk;
     float* partial_loss = partial + static_cast<size_t>(nb) * kModelParams;
-    const size_t smem = sizeof(float) * (kModelParams + kChunk * kF + 4 * kChunk * kH + kChunk * kO + kChunk);
+    const size_t smem = sizeof(float) * (kModelParams + kChunk * kF + 3 * kChunk * kH + kChunk * kHs + kH * kHs + kChunk * kO + kChunk);
     cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    k_mlp_grad<<<nb, 256, smem, st>>>(params_in, X, Tg, m, partial, partial_loss);
+    k_mlp_grad<<<nb, kGradThreads, smem, st>>>(params_in, X, Tg, m, partial, partial_loss);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_mlp_reduce_adam<<<(kModelParams + 255) / 256, 256, 0, st>>>(partial, partial_loss, nb, m, params, mst, vst, t, lr,
