@@ -24,7 +24,7 @@ namespace {
 constexpr int kF = kModelFeatures, kH = kModelHidden, kO = 2;
 
 constexpr int kChunk = 64;  // samples per gradient block
-constexpr int kGradThreads = 1024;
+constexpr int kGradThreads = 1024;  // kH units x kChunk / 4 samples
 constexpr int kHs = kH + 1;  // row stride of W2 and h2 in shared memory: a column's entries lie in different banks
 
 __device__ __forceinline__ float warp_sum_f(float v) {
@@ -102,8 +102,12 @@ __device__ double tridiag_eig(const double* a, const double* b, int k, int i, do
 
 // STAGED: the submatrix is kept in shared memory (as FP32) for the up to 192 matrix-vector products
 // that read it (144 at 48 steps): from L2 they took longer than anything but the eigenvalue searches.
+// All 32 warps multiply (a row each, up to eight at a time); the vectors' sums stay with the first
+// eight warps, whose order fixes their rounding.
+constexpr int kLanczosThreads = 1024, kLanczosVec = 256;
+
 template <class R, bool STAGED>
-__global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ subs, const R* __restrict__ T, int ksteps,
+__global__ void __launch_bounds__(kLanczosThreads) k_lanczos(const SubDesc* __restrict__ subs, const R* __restrict__ T, int ksteps,
                                                  float* __restrict__ labels) {
     extern __shared__ float lz[];  // 4 vectors of n, then (STAGED) the submatrix
     __shared__ double alpha[kMaxLanczos], beta[kMaxLanczos + 1];
@@ -120,7 +124,7 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
     float* u = lz + 3 * n;
     float* ts = lz + 4 * n;
     if constexpr (STAGED) {
-        for (int r = warp; r < n; r += 8)
+        for (int r = warp; r < n; r += kLanczosThreads / 32)
 #pragma unroll 4
             for (int c = lane; c < n; c += 32) ts[r * n + c] = static_cast<float>(t[static_cast<int64_t>(r) * s.ld + c]);
         __syncthreads();
@@ -131,65 +135,67 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
     };
 
     auto block_sum_f = [&](float x) -> float {
-        x = warp_sum_f(x);
-        __syncthreads();
-        if (lane == 0) red[warp] = x;
+        if (warp < 8) x = warp_sum_f(x);
+        if (warp < 8 && lane == 0) red[warp] = x;
         __syncthreads();
         float r = 0.f;
         for (int i = 0; i < 8; ++i) r += red[i];
         __syncthreads();
         return r;
     };
-    // y = A x (a warp per row, four rows at a time)
+    // y = A x
     auto matvec = [&](const float* x, float* y) {
-        for (int r = warp; r < n; r += 32) {
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        constexpr int kW = kLanczosThreads / 32, kRows = 8;
+        for (int r0 = warp; r0 < n; r0 += kW * kRows) {
+            float acc[kRows];
+            int row[kRows];  // (rows past n repeat row r0, not stored)
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                acc[i] = 0.f;
+                row[i] = r0 + kW * i < n ? r0 + kW * i : r0;
+            }
             for (int c = lane; c < n; c += 32) {
                 const float xc = x[c];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (r + 8 * i < n) acc[i] = fmaf(entry(r + 8 * i, c), xc, acc[i]);
+                for (int i = 0; i < kRows; ++i) acc[i] = fmaf(entry(row[i], c), xc, acc[i]);
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i] = warp_sum_f(acc[i]);
+            for (int i = 0; i < kRows; ++i) acc[i] = warp_sum_f(acc[i]);
             if (lane == 0) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (r + 8 * i < n) y[r + 8 * i] = acc[i];
+                for (int i = 0; i < kRows; ++i)
+                    if (r0 + kW * i < n) y[r0 + kW * i] = acc[i];
             }
         }
         __syncthreads();
     };
+    const bool vec = threadIdx.x < kLanczosVec;  // this thread works on the vectors' entries threadIdx.x, + 256, ...
     // Gershgorin bound G
     {
         float g = 0.f;
-        for (int r = warp; r < n; r += 8) {
+        for (int r = warp; r < n; r += kLanczosThreads / 32) {
             float acc = 0.f;
             for (int c = lane; c < n; c += 32) acc += fabsf(entry(r, c));
             g = fmaxf(g, warp_sum_f(acc));
         }
-        if (lane == 0) red[warp] = g;
+        if (threadIdx.x == 0) gmax_s = 0.f;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            float m = 0.f;
-            for (int i = 0; i < 8; ++i) m = fmaxf(m, red[i]);
-            gmax_s = m;
-        }
+        if (lane == 0) atomicMax(reinterpret_cast<int*>(&gmax_s), __float_as_int(g));  // (non-negative floats order like integers)
         __syncthreads();
     }
     const int K = min(ksteps, min(n, kMaxLanczos));
     double lam_lo = 0.0, lam_hi = 0.0, sq_lo = 0.0;
     for (int pass = 0; pass < 2; ++pass) {  // pass 0: A, pass 1: A^2
         // deterministic start vector with all components non-zero
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) {
             v[i] = 1.0f + 0.5f * __sinf(1.7f * static_cast<float>(i) + 0.3f * pass);
             vp[i] = 0.f;
         }
         __syncthreads();
         float nv = 0.f;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) nv += v[i] * v[i];
+        for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) nv += v[i] * v[i];
         nv = sqrtf(block_sum_f(nv));
-        for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] /= nv;
+        for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) v[i] /= nv;
         __syncthreads();
         float bprev = 0.f;
         int k = 0;
@@ -197,10 +203,10 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
             if (pass == 0) matvec(v, w);
             else { matvec(v, u); matvec(u, w); }
             float al = 0.f;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) al += v[i] * w[i];
+            for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) al += v[i] * w[i];
             al = block_sum_f(al);
             float nw = 0.f;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) {
                 const float x = w[i] - al * v[i] - bprev * vp[i];
                 w[i] = x;
                 nw += x * x;
@@ -208,7 +214,7 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
             nw = sqrtf(block_sum_f(nw));
             if (threadIdx.x == 0) { alpha[k] = al; beta[k + 1] = nw; }
             if (nw <= 1e-12f * gmax_s || k + 1 == K) { ++k; break; }
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) {
                 vp[i] = v[i];
                 v[i] = w[i] / nw;
             }
@@ -247,15 +253,15 @@ __global__ void __launch_bounds__(256) k_lanczos(const SubDesc* __restrict__ sub
 __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ X,
                                                   const float* __restrict__ Tg, int m, float* __restrict__ partial,
                                                   float* __restrict__ partial_loss) {
-    extern __shared__ float sm[];
-    float* p = sm;                              // kModelParams
-    float* xs = p + kModelParams;               // [64][kF]
-    float* h1 = xs + kChunk * kF;               // [64][64]
-    float* h2 = h1 + kChunk * kH;               // [64][65]
+    extern __shared__ __align__(16) float sm[];
+    float* h1 = sm;                             // [64][64] (16-byte aligned, as d2)
+    float* d2 = h1 + kChunk * kH;               // [64][64]
+    float* d1 = d2 + kChunk * kH;               // [64][64]  dL/d(pre-activation 1)
+    float* h2 = d1 + kChunk * kH;               // [64][65]
     float* w2 = h2 + kChunk * kHs;              // [64][65]  W2
-    float* d1 = w2 + kH * kHs;                  // [64][64]  dL/d(pre-activation 1)
-    float* d2 = d1 + kChunk * kH;               // [64][64]
-    float* dy = d2 + kChunk * kH;               // [64][2]
+    float* p = w2 + kH * kHs;                   // kModelParams
+    float* xs = p + kModelParams;               // [64][kF]
+    float* dy = xs + kChunk * kF;               // [64][2]
     float* ls = dy + kChunk * kO;               // [64] half squared residual per sample
     const int s0 = blockIdx.x * kChunk;
     const int cnt = min(kChunk, m - s0);
@@ -277,11 +283,28 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
         h1[e] = tanhf(a);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < kChunk * kH; e += blockDim.x) {
-        const int sidx = e / kH, i = e - sidx * kH;
-        float a = p[kOffB2 + i];
-        for (int k = 0; k < kH; ++k) a = fmaf(w2[i * kHs + k], h1[sidx * kH + k], a);
-        h2[sidx * kHs + i] = tanhf(a);
+    // four samples a thread: a weight is read once for them, their h1 four units at a time
+    const int unit = threadIdx.x & (kH - 1), four = 4 * (threadIdx.x / kH);
+    {
+        float a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = p[kOffB2 + unit];
+#pragma unroll 4
+        for (int k = 0; k < kH; k += 4) {
+            float4 h[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) h[u] = *reinterpret_cast<const float4*>(h1 + (four + u) * kH + k);
+            const float* wr = w2 + unit * kHs + k;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a[u] = fmaf(wr[0], h[u].x, a[u]);
+                a[u] = fmaf(wr[1], h[u].y, a[u]);
+                a[u] = fmaf(wr[2], h[u].z, a[u]);
+                a[u] = fmaf(wr[3], h[u].w, a[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h2[(four + u) * kHs + unit] = tanhf(a[u]);
     }
     __syncthreads();
     if (threadIdx.x < kChunk) {
@@ -310,16 +333,47 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
         d2[e] = g * (1.f - h * h);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < kChunk * kH; e += blockDim.x) {
-        const int sidx = e / kH, k = e - sidx * kH;
-        float g = 0.f;
-        for (int i = 0; i < kH; ++i) g = fmaf(d2[sidx * kH + i], w2[i * kHs + k], g);
-        d1[e] = g * (1.f - h1[e] * h1[e]);
+    {
+        float g[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int i = 0; i < kH; i += 4) {
+            float4 d[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) d[u] = *reinterpret_cast<const float4*>(d2 + (four + u) * kH + i);
+            const float* wc = w2 + i * kHs + unit;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                g[u] = fmaf(d[u].x, wc[0], g[u]);
+                g[u] = fmaf(d[u].y, wc[kHs], g[u]);
+                g[u] = fmaf(d[u].z, wc[2 * kHs], g[u]);
+                g[u] = fmaf(d[u].w, wc[3 * kHs], g[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = (four + u) * kH + unit;
+            d1[e] = g[u] * (1.f - h1[e] * h1[e]);
+        }
     }
     __syncthreads();
     // parameter gradients, each a sum over the block's samples in order
     float* gout = partial + static_cast<int64_t>(blockIdx.x) * kModelParams;
-    for (int q = threadIdx.x; q < kModelParams; q += blockDim.x) {
+    {  // W2: rows four .. four + 3, column `unit`
+        float g[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int sidx = 0; sidx < kChunk; ++sidx) {
+            const float4 d = *reinterpret_cast<const float4*>(d2 + sidx * kH + four);
+            const float h = h1[sidx * kH + unit];
+            g[0] = fmaf(d.x, h, g[0]);
+            g[1] = fmaf(d.y, h, g[1]);
+            g[2] = fmaf(d.z, h, g[2]);
+            g[3] = fmaf(d.w, h, g[3]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) gout[kOffW2 + (four + u) * kH + unit] = g[u];
+    }
+    for (int x = threadIdx.x; x < kModelParams - kH * kH; x += blockDim.x) {  // the others
+        const int q = x < kOffW2 ? x : x + kH * kH;
         float g = 0.f;
         if (q < kOffB1) {
             const int i = q / kF, k = q - i * kF;
@@ -327,9 +381,6 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
         } else if (q < kOffW2) {
             const int i = q - kOffB1;
             for (int sidx = 0; sidx < kChunk; ++sidx) g += d1[sidx * kH + i];
-        } else if (q < kOffB2) {
-            const int i = (q - kOffW2) / kH, k = (q - kOffW2) - i * kH;
-            for (int sidx = 0; sidx < kChunk; ++sidx) g = fmaf(d2[sidx * kH + i], h1[sidx * kH + k], g);
         } else if (q < kOffW3) {
             const int i = q - kOffB2;
             for (int sidx = 0; sidx < kChunk; ++sidx) g += d2[sidx * kH + i];
@@ -381,13 +432,13 @@ __global__ void k_mlp_reduce_adam(const float* __restrict__ partial, const float
 template <class R>
 static cudaError_t launch_lanczos_type(const SubDesc* subs, int n_subs, int max_n, const R* T, int ksteps, float* labels, cudaStream_t st) {
     const size_t vectors = sizeof(float) * 4 * static_cast<size_t>(max_n), staged = vectors + sizeof(float) * static_cast<size_t>(max_n) * max_n;
-    // up to n = 238 the submatrix fits shared memory (two CTAs per SM up to n = 165)
+    // up to n = 238 the submatrix fits shared memory
     const bool fits = staged <= 225u * 1024u;
     const size_t smem = fits ? staged : vectors;
     auto kernel = fits ? k_lanczos<R, true> : k_lanczos<R, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    kernel<<<n_subs, 256, smem, st>>>(subs, T, ksteps, labels);
+    kernel<<<n_subs, kLanczosThreads, smem, st>>>(subs, T, ksteps, labels);
     return cudaGetLastError();
 }
 
