@@ -105,15 +105,17 @@ __device__ double tridiag_eig(const double* a, const double* b, int k, int i, do
 // All 32 warps multiply (a row each, up to eight at a time); the vectors' sums stay with the first
 // eight warps, whose order fixes their rounding.
 constexpr int kLanczosThreads = 1024, kLanczosVec = 256;
+// a tridiagonal in global memory: diagonal, off-diagonal (entry 0 unused, one more at the end), size, and (the
+// second one of a submatrix) the Gershgorin bound
+constexpr int kTridiag = 2 * kMaxLanczos + 3;
+static_assert(kTridiag == kLanczosTridiag, "doubles per tridiagonal");
 
 template <class R, bool STAGED>
 __global__ void __launch_bounds__(kLanczosThreads) k_lanczos(const SubDesc* __restrict__ subs, const R* __restrict__ T, int ksteps,
-                                                 float* __restrict__ labels) {
+                                                             double* __restrict__ tridiag) {
     extern __shared__ float lz[];  // 4 vectors of n, then (STAGED) the submatrix
-    __shared__ double alpha[kMaxLanczos], beta[kMaxLanczos + 1];
-    __shared__ double2 scaled[2][kMaxLanczos];
-    __shared__ double eig[2];
     __shared__ float red[8];
+    __shared__ int last_s;
     __shared__ float gmax_s;
     const SubDesc s = subs[blockIdx.x];
     const R* t = T + s.t_off;
@@ -134,18 +136,21 @@ __global__ void __launch_bounds__(kLanczosThreads) k_lanczos(const SubDesc* __re
         else return static_cast<float>(t[static_cast<int64_t>(r) * s.ld + c]);
     };
 
+    // the sum of the first eight warps' values (called by them alone; a barrier of their own)
+    auto vec_sync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
     auto block_sum_f = [&](float x) -> float {
-        if (warp < 8) x = warp_sum_f(x);
-        if (warp < 8 && lane == 0) red[warp] = x;
-        __syncthreads();
+        x = warp_sum_f(x);
+        if (lane == 0) red[warp] = x;
+        vec_sync();
         float r = 0.f;
         for (int i = 0; i < 8; ++i) r += red[i];
-        __syncthreads();
+        vec_sync();
         return r;
     };
-    // y = A x
+    // y = A x, kRows rows a warp at a time: each row's products summed over the lane's columns, then over the
+    // lanes (the pairs of a butterfly, every pair added once: after three exchanges a lane holds one row)
+    constexpr int kW = kLanczosThreads / 32, kRows = 8;
     auto matvec = [&](const float* x, float* y) {
-        constexpr int kW = kLanczosThreads / 32, kRows = 8;
         for (int r0 = warp; r0 < n; r0 += kW * kRows) {
             float acc[kRows];
             int row[kRows];  // (rows past n repeat row r0, not stored)
@@ -157,15 +162,28 @@ __global__ void __launch_bounds__(kLanczosThreads) k_lanczos(const SubDesc* __re
             for (int c = lane; c < n; c += 32) {
                 const float xc = x[c];
 #pragma unroll
-                for (int i = 0; i < kRows; ++i) acc[i] = fmaf(entry(row[i], c), xc, acc[i]);
-            }
-#pragma unroll
-            for (int i = 0; i < kRows; ++i) acc[i] = warp_sum_f(acc[i]);
-            if (lane == 0) {
-#pragma unroll
                 for (int i = 0; i < kRows; ++i)
-                    if (r0 + kW * i < n) y[r0 + kW * i] = acc[i];
+                    if (i < 4 || r0 + kW * i < n) acc[i] = fmaf(entry(row[i], c), xc, acc[i]);  // (uniform over the warp)
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const bool up = lane & 16;
+                const float send = up ? acc[i] : acc[i + 4], keep = up ? acc[i + 4] : acc[i];
+                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const bool up = lane & 8;
+                const float send = up ? acc[i] : acc[i + 2], keep = up ? acc[i + 2] : acc[i];
+                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+            }
+            const bool up = lane & 4;
+            const float send = up ? acc[0] : acc[1], keep = up ? acc[1] : acc[0];
+            float a = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+            a += __shfl_xor_sync(0xffffffffu, a, 2);
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+            const int mine = r0 + kW * (((lane & 16) ? 4 : 0) + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0));
+            if ((lane & 3) == 0 && mine < n) y[mine] = a;
         }
         __syncthreads();
     };
@@ -184,61 +202,79 @@ __global__ void __launch_bounds__(kLanczosThreads) k_lanczos(const SubDesc* __re
         __syncthreads();
     }
     const int K = min(ksteps, min(n, kMaxLanczos));
-    double lam_lo = 0.0, lam_hi = 0.0, sq_lo = 0.0;
+    double* tri = tridiag + static_cast<int64_t>(blockIdx.x) * 2 * kTridiag;  // A's tridiagonal, then A^2's
     for (int pass = 0; pass < 2; ++pass) {  // pass 0: A, pass 1: A^2
         // deterministic start vector with all components non-zero
-        for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) {
-            v[i] = 1.0f + 0.5f * __sinf(1.7f * static_cast<float>(i) + 0.3f * pass);
-            vp[i] = 0.f;
+        if (vec) {
+            float nv = 0.f;
+            for (int i = threadIdx.x; i < n; i += kLanczosVec) {
+                v[i] = 1.0f + 0.5f * __sinf(1.7f * static_cast<float>(i) + 0.3f * pass);
+                vp[i] = 0.f;
+                nv += v[i] * v[i];
+            }
+            nv = sqrtf(block_sum_f(nv));
+            for (int i = threadIdx.x; i < n; i += kLanczosVec) v[i] /= nv;
         }
-        __syncthreads();
-        float nv = 0.f;
-        for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) nv += v[i] * v[i];
-        nv = sqrtf(block_sum_f(nv));
-        for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) v[i] /= nv;
         __syncthreads();
         float bprev = 0.f;
         int k = 0;
         for (; k < K; ++k) {
             if (pass == 0) matvec(v, w);
             else { matvec(v, u); matvec(u, w); }
-            float al = 0.f;
-            for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) al += v[i] * w[i];
-            al = block_sum_f(al);
-            float nw = 0.f;
-            for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) {
-                const float x = w[i] - al * v[i] - bprev * vp[i];
-                w[i] = x;
-                nw += x * x;
+            if (vec) {  // (an entry stays with its thread)
+                float al = 0.f;
+                for (int i = threadIdx.x; i < n; i += kLanczosVec) al += v[i] * w[i];
+                al = block_sum_f(al);
+                float nw = 0.f;
+                for (int i = threadIdx.x; i < n; i += kLanczosVec) {
+                    const float x = w[i] - al * v[i] - bprev * vp[i];
+                    w[i] = x;
+                    nw += x * x;
+                }
+                nw = sqrtf(block_sum_f(nw));
+                const bool last = nw <= 1e-12f * gmax_s || k + 1 == K;
+                if (threadIdx.x == 0) {
+                    tri[k] = al;
+                    tri[kMaxLanczos + k + 1] = nw;
+                    last_s = last;
+                }
+                if (!last)
+                    for (int i = threadIdx.x; i < n; i += kLanczosVec) {
+                        vp[i] = v[i];
+                        v[i] = w[i] / nw;
+                    }
+                bprev = nw;
             }
-            nw = sqrtf(block_sum_f(nw));
-            if (threadIdx.x == 0) { alpha[k] = al; beta[k + 1] = nw; }
-            if (nw <= 1e-12f * gmax_s || k + 1 == K) { ++k; break; }
-            for (int i = vec ? threadIdx.x : n; i < n; i += kLanczosVec) {
-                vp[i] = v[i];
-                v[i] = w[i] / nw;
-            }
-            bprev = nw;
             __syncthreads();
+            if (last_s) {
+                ++k;
+                break;
+            }
         }
-        __syncthreads();
-        if (warp < 2 - pass) {  // the two ends of A's spectrum, or the lower end of A^2's, a warp each
-            const double x = tridiag_eig(alpha, beta, k, warp == 0 ? 0 : k - 1, scaled[warp]);
-            if (lane == 0) eig[warp] = x;
-        }
-        __syncthreads();
-        if (pass == 0) {
-            lam_lo = eig[0];
-            lam_hi = eig[1];
-        } else {
-            sq_lo = eig[0];
-        }
+        if (threadIdx.x == 0) tri[2 * kMaxLanczos + 1] = k;
+        tri += kTridiag;
         __syncthreads();
     }
+    if (threadIdx.x == 0) tridiag[(static_cast<int64_t>(blockIdx.x) + 1) * 2 * kTridiag - 1] = gmax_s;
+}
+
+// The labels from the two tridiagonals of each submatrix: a warp finds the smallest and largest eigenvalue
+// of A or the smallest of A^2 (three warps a submatrix, 3072 at a time in flight on 1024 submatrices:
+// inside the Lanczos kernel, a CTA per SM, the latency of the FP64 recurrence was a third of its time).
+__global__ void __launch_bounds__(96) k_lanczos_labels(const double* __restrict__ tridiag, float* __restrict__ labels) {
+    __shared__ double2 scaled[3][kMaxLanczos];
+    __shared__ double eig[3];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double* tri = tridiag + static_cast<int64_t>(blockIdx.x) * 2 * kTridiag;
+    const double* mine = tri + (warp == 2 ? kTridiag : 0);
+    const int k = static_cast<int>(mine[2 * kMaxLanczos + 1]);
+    const double x = tridiag_eig(mine, mine + kMaxLanczos, k, warp == 1 ? k - 1 : 0, scaled[warp]);
+    if (lane == 0) eig[warp] = x;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        const double G = gmax_s > 0.f ? gmax_s : 1.f;
-        labels[2 * blockIdx.x] = static_cast<float>(fmax(fabs(lam_lo), fabs(lam_hi)) / G);
-        labels[2 * blockIdx.x + 1] = static_cast<float>(sqrt(fmax(sq_lo, 0.0)) / G);
+        const double g = tri[2 * kTridiag - 1], G = g > 0.0 ? g : 1.0;
+        labels[2 * blockIdx.x] = static_cast<float>(fmax(fabs(eig[0]), fabs(eig[1])) / G);
+        labels[2 * blockIdx.x + 1] = static_cast<float>(sqrt(fmax(eig[2], 0.0)) / G);
     }
 }
 
@@ -307,21 +343,20 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
         for (int u = 0; u < 4; ++u) h2[(four + u) * kHs + unit] = tanhf(a[u]);
     }
     __syncthreads();
-    if (threadIdx.x < kChunk) {
-        const int sidx = threadIdx.x;
-        float l = 0.f;
-        for (int o = 0; o < kO; ++o) {
-            float y = p[kOffB3 + o];
-            for (int k = 0; k < kH; ++k) y = fmaf(p[kOffW3 + o * kH + k], h2[sidx * kHs + k], y);
-            const float r = sidx < cnt ? y - Tg[2 * static_cast<int64_t>(s0 + sidx) + o] : 0.f;
-            dy[sidx * kO + o] = r;
-            l = fmaf(r, r, l);
-        }
-        ls[sidx] = 0.5f * l;
+    if (threadIdx.x < kChunk * kO) {  // (a sample's outputs in neighbouring lanes)
+        const int sidx = threadIdx.x >> 1, o = threadIdx.x & 1;
+        float y = p[kOffB3 + o];
+#pragma unroll 16
+        for (int k = 0; k < kH; ++k) y = fmaf(p[kOffW3 + o * kH + k], h2[sidx * kHs + k], y);
+        const float r = sidx < cnt ? y - Tg[2 * static_cast<int64_t>(s0 + sidx) + o] : 0.f;
+        dy[sidx * kO + o] = r;
+        const float r0 = __shfl_xor_sync(0xffffffffu, r, 1);
+        if (o == 1) ls[sidx] = 0.5f * fmaf(r, r, r0 * r0);
     }
     __syncthreads();
     if (threadIdx.x == 0) {  // summed in sample order
         float l = 0.f;
+#pragma unroll 16
         for (int i = 0; i < kChunk; ++i) l += ls[i];
         partial_loss[blockIdx.x] = l;
     }
@@ -377,6 +412,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
         float g = 0.f;
         if (q < kOffB1) {
             const int i = q / kF, k = q - i * kF;
+#pragma unroll 16
             for (int sidx = 0; sidx < kChunk; ++sidx) g = fmaf(d1[sidx * kH + i], xs[sidx * kF + k], g);
         } else if (q < kOffW2) {
             const int i = q - kOffB1;
@@ -430,7 +466,8 @@ __global__ void k_mlp_reduce_adam(const float* __restrict__ partial, const float
 // launchers
 // ---------------------------------------------------------------------------
 template <class R>
-static cudaError_t launch_lanczos_type(const SubDesc* subs, int n_subs, int max_n, const R* T, int ksteps, float* labels, cudaStream_t st) {
+static cudaError_t launch_lanczos_type(const SubDesc* subs, int n_subs, int max_n, const R* T, int ksteps, double* tridiag, float* labels,
+                                       cudaStream_t st) {
     const size_t vectors = sizeof(float) * 4 * static_cast<size_t>(max_n), staged = vectors + sizeof(float) * static_cast<size_t>(max_n) * max_n;
     // up to n = 238 the submatrix fits shared memory
     const bool fits = staged <= 225u * 1024u;
@@ -438,14 +475,17 @@ static cudaError_t launch_lanczos_type(const SubDesc* subs, int n_subs, int max_
     auto kernel = fits ? k_lanczos<R, true> : k_lanczos<R, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    kernel<<<n_subs, kLanczosThreads, smem, st>>>(subs, T, ksteps, labels);
+    kernel<<<n_subs, kLanczosThreads, smem, st>>>(subs, T, ksteps, tridiag);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_lanczos_labels<<<n_subs, 96, 0, st>>>(tridiag, labels);
     return cudaGetLastError();
 }
 
 cudaError_t launch_lanczos(const SubDesc* subs, int n_subs, int max_n, const void* T, bool fp32, int ksteps,
-                           float* labels, cudaStream_t st) {
-    if (fp32) return launch_lanczos_type(subs, n_subs, max_n, static_cast<const float*>(T), ksteps, labels, st);
-    return launch_lanczos_type(subs, n_subs, max_n, static_cast<const double*>(T), ksteps, labels, st);
+                           double* tridiag, float* labels, cudaStream_t st) {
+    if (fp32) return launch_lanczos_type(subs, n_subs, max_n, static_cast<const float*>(T), ksteps, tridiag, labels, st);
+    return launch_lanczos_type(subs, n_subs, max_n, static_cast<const double*>(T), ksteps, tridiag, labels, st);
 }
 
 size_t mlp_partial_floats(int m) { return static_cast<size_t>((m + kChunk - 1) / kChunk) * (kModelParams + 1); }

@@ -146,7 +146,7 @@ struct smx_ctx {
     int adam_t = 0;
     int64_t n_samples = 0, cap_samples = 0;
     DevBuf d_params, d_mst, d_vst, d_partial_mlp, d_feat, d_pred, d_labels, d_gersh, d_prev_ratio, d_sq_ratio,
-        d_loss, d_sx, d_st, d_fit_x, d_fit_t, d_grad;
+        d_tridiag, d_loss, d_sx, d_st, d_fit_x, d_fit_t, d_grad;
 };
 
 // ---------------------------------------------------------------------------
@@ -1274,9 +1274,10 @@ static smx_status features_labels(smx_ctx* c, int32_t lanczos_steps, bool predic
         }
         SMX_TRY(gather_chunk(c, j0, m, c->mu, ex));
         if (lanczos_steps > 0) {
-            SMX_CUDA(launch_lanczos(subs + j0, m, c->max_n, c->d_T.p, f32, lanczos_steps, dp<float>(c->d_labels) + 2 * j0,
-                                    c->stream));
-            c->kernel_launches += 1;
+            SMX_TRY(ensure(c->d_tridiag, sizeof(double) * 2 * kLanczosTridiag * m));
+            SMX_CUDA(launch_lanczos(subs + j0, m, c->max_n, c->d_T.p, f32, lanczos_steps, dp<double>(c->d_tridiag),
+                                    dp<float>(c->d_labels) + 2 * j0, c->stream));
+            c->kernel_launches += 2;
         }
     }
     return SMX_OK;
@@ -1486,7 +1487,7 @@ void smx_destroy(smx_ctx* c) {
                       &c->d_ws, &c->d_ws64, &c->d_maps, &c->d_map_off, &c->d_pairs, &c->d_D, &c->d_xown, &c->d_bound, &c->d_iters, &c->d_partial,
                       &c->d_work_n3,
                       &c->d_params, &c->d_mst, &c->d_vst, &c->d_partial_mlp, &c->d_feat, &c->d_pred, &c->d_labels,
-                      &c->d_gersh, &c->d_prev_ratio, &c->d_sq_ratio, &c->d_loss, &c->d_sx, &c->d_st,
+                      &c->d_gersh, &c->d_prev_ratio, &c->d_sq_ratio, &c->d_tridiag, &c->d_loss, &c->d_sx, &c->d_st,
                       &c->d_fit_x, &c->d_fit_t, &c->d_grad, &c->d_S, &c->d_Lc, &c->d_Mc, &c->d_nlohi,
                       &c->d_setup_iters};
     for (DevBuf* b : bufs) release(*b);

@@ -227,9 +227,11 @@ constexpr int kMaxLanczos = 64;
 // under-prediction (a few percent) so that the first-product check passes
 constexpr float kModelMargin = 0.05f;
 
-// labels[2j] = rho/G, labels[2j+1] = delta/G by Lanczos on A and A^2
+// labels[2j] = rho/G, labels[2j+1] = delta/G by Lanczos on A and A^2 (two kernels); tridiag: scratch of
+// 2 kLanczosTridiag doubles per submatrix
+constexpr int kLanczosTridiag = 2 * kMaxLanczos + 3;
 cudaError_t launch_lanczos(const SubDesc* subs, int n_subs, int max_n, const void* T, bool fp32, int ksteps,
-                           float* labels, cudaStream_t st);
+                           double* tridiag, float* labels, cudaStream_t st);
 // floats of scratch one gradient/Adam step on m samples needs
 size_t mlp_partial_floats(int m);
 // gradient at params_in on (X, Tg); grad_out/loss_out optional; Adam update of params when lr > 0
