@@ -10,8 +10,11 @@
 // The products run on the tensor cores by error-free slices (smx_slices.cuh), and everything
 // between them is 64-bit integer arithmetic in units of 2^-62: GB300's FP64 units take about 16
 // cycles per warp instruction, so one FP64 operation per matrix entry costs as much as a quarter of
-// a product (n = 158).  One persistent CTA per SM takes submatrices largest first and keeps an
-// iterate, one product and the operands' digits in a slot of global memory that stays in L2.
+// a product (n = 158).  One persistent CTA per SM (or cluster of CTAs, where there are fewer
+// submatrices than SMs: launch_form) takes submatrices largest first and keeps an iterate, one product
+// and the operands' digits in a slot of global memory that stays in L2.
+#include <climits>
+
 #include "smx_finish.cuh"
 #include "smx_kernels.h"
 #include "smx_slices.cuh"
@@ -25,11 +28,12 @@ struct SliceJob {
     int n, k;  // dimension, and rounded up to 32 (rows and columns past n are zero)
     int64_t* M[kFp64Mats];
     uint8_t* P[kFp64Planes];
+    float* scratch;  // of the cluster (the first kSlotHead bytes of its slot): sums, maxima, the claimed job, maxima
 };
 
 // Scalars that one thread forms in FP64 for the CTA.
 struct SliceScalars {
-    int job, next;
+    int job;
     int e;
     int bad;
     int stop;          // the schedule's factor allows this step to be the last
@@ -46,6 +50,10 @@ __device__ __forceinline__ void slice_job(SliceJob& jb, uint8_t* slot, int n, in
     for (int i = 0; i < kFp64Mats; ++i) jb.M[i] = reinterpret_cast<int64_t*>(slot + i * mb);
     for (int i = 0; i < kFp64Planes; ++i) jb.P[i] = slot + mats * mb + i * slice_bytes(kmax);
 }
+// The first bytes of a slot serve the cluster (kSlotHead); slice_job gets what follows.
+constexpr int64_t kSlotHead = 256;
+
+__device__ __forceinline__ int64_t ld1(const int64_t* p) { return __ldcg(reinterpret_cast<const long long*>(p)); }
 
 __device__ __forceinline__ unsigned long long cta_max_u64(unsigned long long v, SliceScalars* ss) {
 #pragma unroll
@@ -190,7 +198,7 @@ __device__ __noinline__ void pass_transposed(const int64_t* A, const int64_t* B,
     slice_pass<1>(rows, k, planes, [&](int r, int c, int64_t (&v)[1][8]) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            v[0][i] = r < m ? (A[mat_at(k, c + i, c0 + r)] - (B ? B[mat_at(k, c + i, r)] : 0)) >> shift : 0;
+            v[0][i] = r < m ? (ld1(A + mat_at(k, c + i, c0 + r)) - (B ? ld1(B + mat_at(k, c + i, r)) : 0)) >> shift : 0;
     }, [](int, int, const int64_t (&v)[1][8], int64_t (&q)[8]) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) q[i] = v[0][i];
@@ -208,15 +216,16 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
         const double v = src[static_cast<int64_t>(r) * ld + c];
         return r == c && mu != 0.0 ? v - mu : v;
     };
+    const int ranks = cluster_size(), rank = cluster_rank();
     int e = 0;
     if (threadIdx.x == 0) ss->bad = 0;
     if (!without_scale) {
         uint32_t top = static_cast<uint32_t>(__double2hiint(bound)) & 0x7fffffffu;
         if (top == 0) {  // high words order like the magnitudes
-            for (int r = warp; r < n; r += kSliceWarps)
+            for (int r = warp + rank * kSliceWarps; r < n; r += ranks * kSliceWarps)
 #pragma unroll 4
                 for (int c = lane; c < n; c += 32) top = max(top, static_cast<uint32_t>(__double2hiint(entry(r, c))) & 0x7fffffffu);
-            top = static_cast<uint32_t>(cta_max_u64(top, ss));
+            top = cluster_max(static_cast<uint32_t>(cta_max_u64(top, ss)), reinterpret_cast<uint32_t*>(jb.scratch) + 24);
         }
         const int ex = static_cast<int>(top >> 20);
         if (ex == 0x7ff) {
@@ -231,7 +240,7 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
             return ef > 900 ? d2f_rn(__hiloint2double((hi & 0x800fffff) | (ef << 20), __double2loint(v))) : 0.0f;
         };
         float worst = 0.0f;
-        for (int r = 2 * warp; r < n; r += 2 * kSliceWarps) {
+        for (int r = 2 * (warp + rank * kSliceWarps); r < n; r += 2 * ranks * kSliceWarps) {
             const int r1 = min(r + 1, n - 1);
             float a0 = 0.0f, a1 = 0.0f;
 #pragma unroll 4
@@ -247,11 +256,11 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
             }
             worst = fmaxf(worst, fmaxf(a0, a1));
         }
-        worst = cta_max(worst, sh);
+        worst = __uint_as_float(cluster_max(__float_as_uint(cta_max(worst, sh)), reinterpret_cast<uint32_t*>(jb.scratch) + 8));
         e = e0 + (worst > 0.0f ? static_cast<int>(ceilf(0.5f * log2f(worst * 1.001f))) : 0);
     }
     __syncthreads();
-    const bool bad = pass_source(src, ld, mu, e, 0, M, P, n, k);
+    const bool bad = cluster_sum(pass_source(src, ld, mu, e, 0, M, P, n, k) ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f;
     if (bad) ss->bad = 1;
     __syncthreads();
     return e;
@@ -269,19 +278,38 @@ struct SignBound {
 };
 
 // For the symmetric non-negative-bounded Y = S: the largest row sum of |Y| (every thread), and the smaller
-// max_r (|Y| w)_r / w_r of two power steps from the row sums (thread 0; 0 without any).
-__device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceShared* sh, SliceScalars* ss, double& row_max, double& best) {
+// max_r (|Y| w)_r / w_r of two power steps from the row sums (thread 0; 0 without any).  The CTAs of a
+// cluster take 32 rows each in turn and exchange the sums at `exchange` (3 k values).
+__device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceShared* sh, SliceScalars* ss, unsigned long long* exchange,
+                                         double& row_max, double& best) {
+    const int ranks = cluster_size(), rank = cluster_rank();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     unsigned long long* wv = reinterpret_cast<unsigned long long*>(sh->smem);  // row sums, then weights
     unsigned long long* av = wv + k;
+    // v complete in every CTA of the cluster; the maximum (m: of the CTA's own rows)
+    auto share = [&](unsigned long long* v, unsigned long long m) {
+        if (ranks > 1) {
+            __syncthreads();
+            for (int r = tid; r < n; r += kSliceThreads)
+                if ((r >> 5) % ranks == rank) __stcg(exchange + r, v[r]);
+            phase_sync();
+            for (int r = tid; r < n; r += kSliceThreads)
+                if ((r >> 5) % ranks != rank) {
+                    v[r] = __ldcg(exchange + r);
+                    m = max(m, v[r]);
+                }
+            exchange += k;
+        }
+        return cta_max_u64(m, ss);
+    };
     // row sums of |Y| in units of 2^-50
     unsigned long long m = 0;
-    for (int r = 2 * warp; r < n; r += 2 * kSliceWarps) {  // Y is symmetric: two columns at a time
+    for (int r = 2 * (warp + rank * kSliceWarps); r < n; r += 2 * ranks * kSliceWarps) {  // Y is symmetric: two columns at a time
         const longlong2* y = reinterpret_cast<const longlong2*>(S) + static_cast<int64_t>(r >> 1) * k;
         unsigned long long a0 = 0, a1 = 0;
 #pragma unroll 4
         for (int c = lane; c < k; c += 32) {
-            const longlong2 v = y[c];
+            const longlong2 v = __ldcg(y + c);
             a0 += abs_fixed(v.x) >> 12;
             a1 += abs_fixed(v.y) >> 12;
         }
@@ -293,7 +321,7 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
         }
         m = max(m, max(a0, a1));
     }
-    m = cta_max_u64(m, ss);
+    m = share(wv, m);
     row_max = static_cast<double>(m) * 0x1p-50;
     best = 0.0;  // of the power steps (every row's quotient; 0: none)
     for (int pass = 0; pass < 2 && m > 0; ++pass) {
@@ -305,12 +333,12 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
         }
         __syncthreads();
         m = 0;
-        for (int r = 2 * warp; r < n; r += 2 * kSliceWarps) {
+        for (int r = 2 * (warp + rank * kSliceWarps); r < n; r += 2 * ranks * kSliceWarps) {
             const longlong2* y = reinterpret_cast<const longlong2*>(S) + static_cast<int64_t>(r >> 1) * k;
             unsigned long long a0 = 0, a1 = 0;  // (|Y| w)_r, w in units of 2^-63, in units of 2^-51
 #pragma unroll 4
             for (int c = lane; c < k; c += 32) {  // (zero past n)
-                const longlong2 v = y[c];
+                const longlong2 v = __ldcg(y + c);
                 const unsigned long long w = wv[c] << 1;
                 a0 += __umul64hi(abs_fixed(v.x) << 1, w) >> 12;
                 a1 += __umul64hi(abs_fixed(v.y) << 1, w) >> 12;
@@ -323,7 +351,7 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
             }
             m = max(m, max(a0, a1));
         }
-        m = cta_max_u64(m, ss);
+        m = share(av, m);
         double q = 0.0;
         if (32 * warp < n) {  // FP64 divisions only on the warps that hold rows
             for (int r = tid; r < n; r += kSliceThreads) q = fmax(q, static_cast<double>(av[r]) / static_cast<double>(wv[r]));
@@ -366,7 +394,7 @@ __device__ int sign_steps(SliceShared* sh, const SliceJob& jb, int e, int max_it
         if (*static_cast<volatile int*>(&sh->abort)) break;
         if (it == 0 && plain_steps == 0) {
             double row_max, best;
-            first_bound(S, n, k, sh, ss, row_max, best);
+            first_bound(S, n, k, sh, ss, reinterpret_cast<unsigned long long*>(jb.P[1]), row_max, best);
             if (tid == 0) {
                 // s >= rho(X0); the model's rules are stated for A / b_j = X0 / phi
                 const double rmax = row_max;
@@ -385,7 +413,7 @@ __device__ int sign_steps(SliceShared* sh, const SliceJob& jb, int e, int max_it
                             scale = fmax(1.0, scale);
                         }
                     } else {
-                        atomicAdd(model->fallbacks, 1);
+                        if (cluster_rank() == 0) atomicAdd(model->fallbacks, 1);
                     }
                     c = scale / phi;
                 }
@@ -412,7 +440,7 @@ __device__ int sign_steps(SliceShared* sh, const SliceJob& jb, int e, int max_it
         const uint64_t f1 = ss->f1, f2 = ss->f2;
         // W = I - a^2 X^2 to its digits; the residual ||I - X^2||_F
         float r2 = pass_residual(S, jb.P[1], n, k, 0, f2);
-        r2 = cta_sum(r2 * 0x1p-76f, sh);
+        r2 = cluster_sum(r2 * 0x1p-76f, sh, jb.scratch);
         slice_product(sh, jb.P[0], jb.P[1], k, k, S, true);
         if (*static_cast<volatile int*>(&sh->abort)) break;
         done = it + 1;
@@ -443,7 +471,7 @@ __device__ __noinline__ float column_norm2(const SliceJob& jb, const int64_t* M,
         float a0 = 0.0f, a1 = 0.0f;
 #pragma unroll 4
         for (int r = lane; r < k; r += 32) {
-            const longlong2 v = m[r];
+            const longlong2 v = __ldcg(m + r);
             const float x = static_cast<float>(static_cast<int>(v.x >> 32)), y = static_cast<float>(static_cast<int>(v.y >> 32));
             a0 = fmaf(x, x, a0);
             a1 = fmaf(y, y, a1);
@@ -481,7 +509,7 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
     const int e = 1022 - static_cast<int>((ib >> 52) & 0x7ff);
     bool off = !(b > 0.0) || !isfinite(inv) || inv == 0.0;
     off |= pass_source(src, ld, 0.0, e, f, Y, jb.P[0], n, k);
-    if (__syncthreads_or(off)) {
+    if (cluster_sum(off ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f) {
         bad = true;
         return 0;
     }
@@ -491,7 +519,7 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
             if (*static_cast<volatile int*>(&sh->abort)) break;
         }
         float r2 = pass_residual(it > 0 ? S : Y, jb.P[2], n, k, ez, 0);
-        r2 = cta_sum(r2 * 0x1p-76f, sh);
+        r2 = cluster_sum(r2 * 0x1p-76f, sh, jb.scratch);
         done = it + 1;
         if (!isfinite(r2) || r2 > 1.5f * static_cast<float>(n) || ez > 40) {
             bad = true;
@@ -560,7 +588,7 @@ __device__ int fermi_tanh(SliceShared* sh, const SliceJob& jb, const double* __r
     const bool zero = !(fac > 0.0);
     bool off = !isfinite(fac);
     if (!zero && !off) off = pass_source(src, ld, 0.0, e, f, T, PT, n, k);
-    if (__syncthreads_or(off)) {
+    if (cluster_sum(off ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f) {
         bad = true;
         return 0;
     }
@@ -618,6 +646,13 @@ __device__ int fermi_tanh(SliceShared* sh, const SliceJob& jb, const double* __r
     return nprod;
 }
 
+// The symmetric matrix f M as doubles, row by row.
+__device__ __noinline__ void store_scaled(const int64_t* M, int k, double f, double* __restrict__ out, int n, int ld) {
+    for (int r = cluster_rank() * kSliceWarps + (threadIdx.x >> 5); r < n; r += cluster_size() * kSliceWarps)
+        for (int c = threadIdx.x & 31; c < n; c += 32)  // row r is column r
+            out[static_cast<int64_t>(r) * ld + c] = f * static_cast<double>(ld1(M + mat_at(k, c, r)));
+}
+
 // Gershgorin interval (lo, hi) of an n x n matrix held row by row.
 __device__ double2 gershgorin_interval(const double* M, int n, int ld, double* scratch) {
     const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
@@ -644,33 +679,43 @@ __device__ double2 gershgorin_interval(const double* M, int n, int ld, double* s
     return out;
 }
 
-// The CTA's next submatrix (largest first; every thread gets its place in the order), claimed one
-// ahead: while it is worked on, the source of the one after it comes into L2.
-__device__ __forceinline__ int claim_job(int* counter, SliceScalars* ss, SubDesc* cur, bool first, int n_subs, const int32_t* order, const SubDesc* subs,
-                                         const double* src) {
+// The next submatrix of the CTA or cluster (largest first; every thread gets its place in the order): its
+// own place first, then whichever is next when it is free.  (Claimed one ahead, 256 submatrices on 152
+// SMs took 8 % longer: some SMs held two of the largest.)  Meanwhile the source of the submatrix that
+// the launch is likely to reach next comes into L2.
+__device__ __forceinline__ int claim_job(int* counter, SliceScalars* ss, SubDesc* cur, int* shared_job, bool first, int n_subs,
+                                         const int32_t* order, const SubDesc* subs, const double* src) {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        ss->job = first ? atomicAdd(counter, 1) : ss->next;
-        if (ss->job < n_subs) *cur = subs[order[ss->job]];
-        const int nx = atomicAdd(counter, 1);
-        ss->next = nx;
-        if (nx < n_subs) {
-            const SubDesc& s = subs[order[nx]];
+    const int ranks = cluster_size(), clusters = gridDim.x / ranks;
+    const bool leader = cluster_rank() == 0;
+    if (threadIdx.x == 0 && leader) {
+        const int job = first ? blockIdx.x / ranks : clusters + atomicAdd(counter, 1);
+        if (ranks > 1) __stcg(shared_job, job);
+        ss->job = job;
+        if (job + clusters < n_subs) {
+            const SubDesc& s = subs[order[job + clusters]];
             const uint64_t bytes = static_cast<uint64_t>(s.n) * s.ld * sizeof(double);
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + s.t_off),
                          "r"(static_cast<uint32_t>(bytes < (8u << 20) ? bytes : (8u << 20)) & ~15u)
                          : "memory");
         }
     }
+    if (ranks > 1) phase_sync();
+    if (threadIdx.x == 0) {
+        if (!leader) ss->job = __ldcg(shared_job);
+        if (ss->job < n_subs) *cur = subs[order[ss->job]];
+    }
     __syncthreads();
     return ss->job;
 }
 
-// The last CTA to run out of work resets the job counter for the next launch.
-__device__ __forceinline__ void release_jobs(int* counter, unsigned int* ticket) {
-    if (threadIdx.x == 0) {
+// The last cluster to run out of work resets the job counter for the next launch.
+// A leader that gave up leaves its cluster no job to find.
+__device__ __forceinline__ void release_jobs(int* counter, unsigned int* ticket, int* shared_job) {
+    if (threadIdx.x == 0 && cluster_rank() == 0) {
+        __stcg(shared_job, INT_MAX);
         __threadfence();
-        if (atomicAdd(ticket, 1u) == gridDim.x - 1) {
+        if (atomicAdd(ticket, 1u) == gridDim.x / cluster_size() - 1) {
             *counter = 0;
             *ticket = 0u;
         }
@@ -700,12 +745,16 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
     SliceShared* const sh = &shared;
     int* ls_smem = reinterpret_cast<int*>(slice_stages());  // local block starts, between products only
     slices_begin(sh, slice_stages(), a.status);
-    uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x) * a.slot_bytes;
+    uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x / cluster_size()) * a.slot_bytes;
+    const bool lead = cluster_rank() == 0;  // writes the results
     for (bool first = true;; first = false) {
-        const int job = claim_job(a.work_counter, &ss, &s, first, a.n_subs, a.order, a.subs, a.Mc ? a.Mc : a.T);
+        const int job = claim_job(a.work_counter, &ss, &s, reinterpret_cast<int*>(slot + 64), first, a.n_subs, a.order, a.subs, a.Mc ? a.Mc : a.T);
         if (job >= a.n_subs || sh->abort) break;
         const int j = s.col;
-        if (threadIdx.x == 0) slice_job(jb, slot, s.n, a.kmax, a.mats);
+        if (threadIdx.x == 0) {
+            slice_job(jb, slot + kSlotHead, s.n, a.kmax, a.mats);
+            jb.scratch = reinterpret_cast<float*>(slot);
+        }
         __syncthreads();
         const int n = s.n, k = jb.k;
         const double* T = a.T + s.t_off;
@@ -714,15 +763,15 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
         if constexpr (FORM == kFormFermi) {
             done = fermi_tanh(sh, jb, T, s.ld, a.bound[j], a.beta, &ss, bad);
             if (sh->abort) break;
-            if (threadIdx.x == 0) {
+            if (threadIdx.x == 0 && lead) {
                 a.iters[j] = done;
                 atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
                 if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
             }
             const int64_t* F = jb.M[0];
             const double fs = ldexp(1.0, -ss.e);
-            auto frow = [&](int q, int i) -> double { return fs * from_fixed(F[mat_at(k, i, s.own + q)]); };
-            finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch);  // 1/2 (I - T)
+            auto frow = [&](int q, int i) -> double { return fs * from_fixed(ld1(F + mat_at(k, i, s.own + q))); };
+            if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch);  // 1/2 (I - T)
             fence_proxy_async_smem();
             continue;
         } else if constexpr (FORM == kFormRoots) {
@@ -732,7 +781,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
             done = coupled_steps(sh, jb, T, s.ld, b, a.max_iter, static_cast<float>(a.tau), a.function == kFnSqrt, a.function != kFnSqrt, ez,
                                  &ss, conv, bad);
             if (sh->abort) break;
-            if (threadIdx.x == 0) {
+            if (threadIdx.x == 0 && lead) {
                 a.iters[j] = done;
                 atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
                 if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
@@ -748,8 +797,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
                 F = jb.M[2];
                 fs = ldexp(1.0 / b, 2 * ez);
             }
-            auto frow = [&](int q, int i) -> double { return fs * from_fixed(F[mat_at(k, i, s.own + q)]); };
-            finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch, false);
+            auto frow = [&](int q, int i) -> double { return fs * from_fixed(ld1(F + mat_at(k, i, s.own + q))); };
+            if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch, false);
             fence_proxy_async_smem();
             continue;
         } else {
@@ -769,13 +818,15 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
             if (threadIdx.x == 0) {
                 double b = 0.0;
                 for (int w = 0; w < kSliceWarps; ++w) b = fmax(b, scratch[w]);
-                a.gersh[j] = b > 0.0 ? b : 1.0;
+                scratch[32] = b > 0.0 ? b : 1.0;
+                if (lead) a.gersh[j] = scratch[32];
             }
             __syncthreads();
         }
         const bool finish = a.finish_iters > 0;
-        SignModel model{a.bound[j], a.pred ? static_cast<double>(a.pred[2 * j + 1]) * a.gersh[j] / a.bound[j] : -1.0, a.fallbacks};
-        const int e = load_fixed(src, s.ld, a.Mc ? a.mu : 0.0, a.gersh[j], jb, jb.M[0], jb.P[0], finish, sh, &ss);
+        const double gersh = a.Mc ? scratch[32] : a.gersh[j];
+        SignModel model{a.bound[j], a.pred ? static_cast<double>(a.pred[2 * j + 1]) * gersh / a.bound[j] : -1.0, a.fallbacks};
+        const int e = load_fixed(src, s.ld, a.Mc ? a.mu : 0.0, gersh, jb, jb.M[0], jb.P[0], finish, sh, &ss);
         bad = ss.bad != 0;
         // with the learned bound W reaches a norm of 2, with a bulk phase's iterate X one of about 1.2
         set_accumulation(sh, 7, a.use_model || finish ? 160 / 16 : kSliceK / 16);
@@ -783,7 +834,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
             done = sign_steps(sh, jb, e, a.max_iter, static_cast<float>(a.tau), a.finish_iters, a.use_model ? &model : nullptr, &sb, &ss, conv,
                               bad);
         if (sh->abort) break;
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && lead) {
             if (finish) {
                 a.iters[j] += done;
             } else {
@@ -791,7 +842,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
                 if (!bad || done > 0) {
                     // feature of the next snapshot: the Gershgorin bound of A^2, over G; and the
                     // effective bound of c X0
-                    a.sq_ratio[j] = static_cast<float>(ldexp(sqrt(sb.rmax), e) / a.gersh[j]);
+                    a.sq_ratio[j] = static_cast<float>(ldexp(sqrt(sb.rmax), e) / gersh);
                     a.bound[j] = ldexp(1.0 / sb.c, e);
                 }
             }
@@ -817,18 +868,18 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
             slice_product(sh, jb.P[1], jb.P[2], k, w, U, false);
             if (sh->abort) break;
             const double fs = ldexp(1.0, 2 * el);
-            auto prow = [&](int q, int i) -> double { return fs * from_fixed(U[mat_at(k, i, q)]); };
-            finish_column(s, a.pv, a.H, a.D, a.partial, prow, ls_smem, scratch, false, a.Sv);
+            auto prow = [&](int q, int i) -> double { return fs * from_fixed(ld1(U + mat_at(k, i, q))); };
+            if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, prow, ls_smem, scratch, false, a.Sv);
             fence_proxy_async_smem();
             continue;
         }
-        auto xrow = [&](int q, int i) -> double { return from_fixed(X[mat_at(k, i, s.own + q)]); };
-        finish_column(s, a.pv, a.H, a.D, a.partial, xrow, ls_smem, scratch);
+        auto xrow = [&](int q, int i) -> double { return from_fixed(ld1(X + mat_at(k, i, s.own + q))); };
+        if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, xrow, ls_smem, scratch);
         fence_proxy_async_smem();
         }
     }
     slices_end(sh);
-    release_jobs(a.work_counter, a.ticket);
+    release_jobs(a.work_counter, a.ticket, reinterpret_cast<int*>(slot + 64));
 }
 
 // Setup of the non-orthogonal form for one (H, S) pair: from A_S (in Lc) and A_H (in Mc), both
@@ -842,93 +893,138 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid
     __shared__ double scratch[64];
     SliceShared* const sh = &shared;
     slices_begin(sh, slice_stages(), a.status);
-    uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x) * a.slot_bytes;
+    uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x / cluster_size()) * a.slot_bytes;
     for (bool first = true;; first = false) {
-        const int job = claim_job(a.work_counter, &ss, &s, first, a.n_subs, a.order, a.subs, a.Lc);
+        const int job = claim_job(a.work_counter, &ss, &s, reinterpret_cast<int*>(slot + 64), first, a.n_subs, a.order, a.subs, a.Lc);
         if (job >= a.n_subs || sh->abort) break;
-        const int j = s.col;
-        if (threadIdx.x == 0) slice_job(jb, slot, s.n, a.kmax, a.mats);
+        if (threadIdx.x == 0) {
+            slice_job(jb, slot + kSlotHead, s.n, a.kmax, a.mats);
+            jb.scratch = reinterpret_cast<float*>(slot);
+        }
         __syncthreads();
-        const int n = s.n, k = jb.k;
         set_accumulation(sh, 7, kSliceK / 16);
-        double *Lc = a.Lc + s.t_off, *Mc = a.Mc + s.t_off;
-        const double b = a.bound_s[j];
         bool conv = false, bad = false;
         int ez = 0;
-        const int done = coupled_steps(sh, jb, Lc, s.ld, b, a.max_iter, static_cast<float>(a.tau), false, true, ez, &ss, conv, bad);
+        const int done = coupled_steps(sh, jb, a.Lc + s.t_off, s.ld, a.bound_s[s.col], a.max_iter, static_cast<float>(a.tau), false, true, ez, &ss, conv, bad);
         if (sh->abort) break;
-        if (threadIdx.x == 0) {
-            a.iters[j] = done;
+        if (threadIdx.x == 0 && cluster_rank() == 0) {
+            a.iters[s.col] = done;
             if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
             else if (!conv) atomicCAS(a.status, kOk, kErrNoconv);
         }
         if (bad) {  // no L: the bracket is not used, the status tells
-            if (threadIdx.x == 0) a.lohi[2 * j] = a.lohi[2 * j + 1] = 0.0;
+            if (threadIdx.x == 0 && cluster_rank() == 0) a.lohi[2 * s.col] = a.lohi[2 * s.col + 1] = 0.0;
             continue;
         }
         // A_H 2^-eh with rows of at most 1; Q = A_H L, then M = L Q = L A_H L: the right factor's digits
         // are those of Q^T, whose rows are Q's columns
-        const int64_t* Z = jb.M[1];
-        const int eh = load_fixed(Mc, s.ld, 0.0, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
+        const int eh = load_fixed(a.Mc + s.t_off, s.ld, 0.0, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
         if (ss.bad) {
-            if (threadIdx.x == 0) {
+            if (threadIdx.x == 0 && cluster_rank() == 0) {
                 atomicCAS(a.status, kOk, kErrNonfinite);
-                a.lohi[2 * j] = a.lohi[2 * j + 1] = 0.0;
+                a.lohi[2 * s.col] = a.lohi[2 * s.col + 1] = 0.0;
             }
             continue;
         }
         set_accumulation(sh, 8, 160 / 16);
-        slice_product(sh, jb.P[0], jb.P[1], k, k, jb.M[2], false);
+        slice_product(sh, jb.P[0], jb.P[1], jb.k, jb.k, jb.M[2], false);
         if (sh->abort) break;
         // columns of A_H L may be longer than 1 (the 2-norm of A_H exceeds that of its rows)
         const float cn = column_norm2(jb, jb.M[2], sh);
         const int ep = cn > 1.0f ? static_cast<int>(ceilf(0.5f * log2f(cn * 1.001f))) : 0;
-        pass_transposed(jb.M[2], nullptr, 0, k, jb.P[2], k, k, ep);
-        slice_product(sh, jb.P[1], jb.P[2], k, k, jb.M[2], true);
+        pass_transposed(jb.M[2], nullptr, 0, jb.k, jb.P[2], jb.k, jb.k, ep);
+        slice_product(sh, jb.P[1], jb.P[2], jb.k, jb.k, jb.M[2], true);
         if (sh->abort) break;
-        const double ls = ldexp(1.0 / sqrt(b), ez - 62);  // A_S^-1/2 = Z / sqrt(b)
-        const double ms = ldexp(1.0 / b, 2 * ez + eh + ep - 62);
-        for (int r = threadIdx.x / 32; r < n; r += kSliceWarps)
-            for (int c = threadIdx.x & 31; c < n; c += 32) {  // symmetric: row r is column r
-                const int64_t o = mat_at(k, c, r), d = static_cast<int64_t>(r) * s.ld + c;
-                Lc[d] = ls * static_cast<double>(Z[o]);
-                Mc[d] = ms * static_cast<double>(jb.M[2][o]);
-            }
-        __syncthreads();
-        const double2 g = gershgorin_interval(Mc, n, s.ld, scratch);
+        const double b = a.bound_s[s.col];  // A_S^-1/2 = Z / sqrt(b)
+        store_scaled(jb.M[1], jb.k, ldexp(1.0 / sqrt(b), ez - 62), a.Lc + s.t_off, s.n, s.ld);
+        store_scaled(jb.M[2], jb.k, ldexp(1.0 / b, 2 * ez + eh + ep - 62), a.Mc + s.t_off, s.n, s.ld);
+        if (cluster_size() > 1) phase_sync();
+        else __syncthreads();
+        if (cluster_rank() != 0) continue;
+        const double2 g = gershgorin_interval(a.Mc + s.t_off, s.n, s.ld, scratch);
         if (threadIdx.x == 0) {
-            a.lohi[2 * j] = g.x;
-            a.lohi[2 * j + 1] = g.y;
+            a.lohi[2 * s.col] = g.x;
+            a.lohi[2 * s.col + 1] = g.y;
         }
     }
     slices_end(sh);
-    release_jobs(a.work_counter, a.ticket);
+    release_jobs(a.work_counter, a.ticket, reinterpret_cast<int*>(slot + 64));
 }
 
 size_t fp64_slot_bytes(int max_n, int mats, int planes) {
     const int64_t k = (static_cast<int64_t>(max_n) + 31) & ~int64_t(31);
-    return static_cast<size_t>(mats * k * k * 8 + planes * slice_bytes(k));
+    return static_cast<size_t>(kSlotHead + mats * k * k * 8 + planes * slice_bytes(k));
 }
 
-template <class K, class A>
-static cudaError_t launch_form(K kernel, const A& a, int slots, cudaStream_t st) {
+// n_clusters clusters of `size` CTAs.
+template <class... P, class... A>
+static cudaError_t launch_clusters(void (*kernel)(P...), int n_clusters, int size, cudaStream_t st, const A&... args) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSliceSmem));
     if (e != cudaSuccess) return e;
-    kernel<<<slots, kSliceThreads, kSliceSmem, st>>>(a);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = static_cast<unsigned>(size);
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(n_clusters * size));
+    cfg.blockDim = dim3(kSliceThreads);
+    cfg.dynamicSmemBytes = kSliceSmem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = size > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_nblk, cudaStream_t st) {
+// CTAs that a submatrix of n rows has work for: at most one per tile of 32 columns of its symmetric products
+// (a power of two up to 8).
+static int cluster_for(int n) {
+    const int k = (n + 31) & ~31;
+    int tiles = 0;
+    for (int r = 0; r < k; r += 128) tiles += (k - r) / 32;
+    return tiles >= 8 ? 8 : tiles >= 4 ? 4 : tiles >= 2 ? 2 : 1;
+}
+
+// CTAs per submatrix: as many as find room at once for all n_subs of them, at most cluster_for(max_n);
+// with more submatrices than SMs each keeps to one (two SMs that share a submatrix also share its
+// barriers, reductions and short products, so they finish fewer of them).  Builds measured with one CTA each and
+// with clusters: 32 submatrices of n = 66 .. 120 (four each) 595 and 301 us, one of n = 192 (eight) 944 and
+// 275 us.  room[i]: clusters of 2^i CTAs the device holds at once (device_clusters).
+template <class K, class A>
+static cudaError_t launch_form(K kernel, const A& a, int slots, int max_n, const int* room, cudaStream_t st) {
+    int size = cluster_for(max_n), i = size == 8 ? 3 : size == 4 ? 2 : size == 2 ? 1 : 0;
+    while (i > 0 && a.n_subs > room[i]) --i;
+    return launch_clusters(kernel, slots, 1 << i, st, a);
+}
+
+cudaError_t device_clusters(int* room) {
+    cudaError_t e = cudaFuncSetAttribute(k_ns_fp64<kFormSign>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSliceSmem));
+    for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 1u << i;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1u << i);
+        cfg.blockDim = dim3(kSliceThreads);
+        cfg.dynamicSmemBytes = kSliceSmem;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        e = cudaOccupancyMaxActiveClusters(&room[i], k_ns_fp64<kFormSign>, &cfg);
+    }
+    return e;
+}
+
+cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_n, int max_nblk, const int* room, cudaStream_t st) {
     if (sizeof(int) * (static_cast<size_t>(max_nblk) + 1) > kSliceSmem - 1024) return cudaErrorInvalidValue;
     switch (a.function) {
-        case kFnDensity: return launch_form(k_ns_fp64<kFormSign>, a, slots, st);
-        case kFnFermi: return launch_form(k_ns_fp64<kFormFermi>, a, slots, st);
-        default: return launch_form(k_ns_fp64<kFormRoots>, a, slots, st);
+        case kFnDensity: return launch_form(k_ns_fp64<kFormSign>, a, slots, max_n, room, st);
+        case kFnFermi: return launch_form(k_ns_fp64<kFormFermi>, a, slots, max_n, room, st);
+        default: return launch_form(k_ns_fp64<kFormRoots>, a, slots, max_n, room, st);
     }
 }
 
-cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, cudaStream_t st) {
-    return launch_form(k_nonorth_setup, a, slots, st);
+cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, int max_n, const int* room, cudaStream_t st) {
+    return launch_form(k_nonorth_setup, a, slots, max_n, room, st);
 }
 
 }  // namespace smx
@@ -962,10 +1058,10 @@ constexpr int kNoAllocMaxDevices = 64;
 
 // The slot of one CTA (two matrices of 64-bit integers and the digits of two operands) for n = 256,
 // followed by a small header: [0] status, [1] iterations.  About 2.8 MiB.
-constexpr int64_t kNoAllocBytes = 2 * kNoAllocMat * 8 + 2 * slice_bytes(kNoAllocMaxN);
+constexpr int64_t kNoAllocBytes = kSlotHead + 2 * kNoAllocMat * 8 + 2 * slice_bytes(kNoAllocMaxN);
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes + 32];
 
-// One CTA: D = 1/2 (I - sign(H - mu I)) of a dense symmetric H by the iteration of k_ns_fp64.
+// One cluster: D = 1/2 (I - sign(H - mu I)) of a dense symmetric H by the iteration of k_ns_fp64.
 __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(const double* __restrict__ H, int n, double mu,
                                                                             double* __restrict__ Dout, uint8_t* scratch,
                                                                             float tau, int max_iter) {
@@ -973,12 +1069,15 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(cons
     __shared__ SliceScalars ss;
     __shared__ SignBound sb;
     int* hdr = reinterpret_cast<int*>(scratch + kNoAllocBytes);
-    if (threadIdx.x == 0) hdr[0] = kOk;
+    if (threadIdx.x == 0 && cluster_rank() == 0) hdr[0] = kOk;
     SliceShared* const sh = &shared;
     slices_begin(sh, slice_stages(), hdr);
     // every call overwrites the work matrices in full; nothing is carried over
     __shared__ SliceJob jb;
-    if (threadIdx.x == 0) slice_job(jb, scratch, n, kNoAllocMaxN, 2);
+    if (threadIdx.x == 0) {
+        slice_job(jb, scratch + kSlotHead, n, kNoAllocMaxN, 2);
+        jb.scratch = reinterpret_cast<float*>(scratch);
+    }
     __syncthreads();
     const int e = load_fixed(H, n, mu, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
     bool conv = false, bad = ss.bad != 0;
@@ -987,17 +1086,17 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(cons
     const bool aborted = *static_cast<volatile int*>(&sh->abort) != 0;
     if (!aborted) {
         const int64_t* X = jb.M[0];
-        for (int r = threadIdx.x >> 5; r < n; r += kSliceWarps)
+        for (int r = cluster_rank() * kSliceWarps + (threadIdx.x >> 5); r < n; r += cluster_size() * kSliceWarps)
             for (int c = threadIdx.x & 31; c < n; c += 32) {  // 1/2 (I - X) in units of 2^-63: up to 2^63
-                const int64_t x = X[mat_at(jb.k, c, r)], one = r == c ? kFixedOne : 0;
+                const int64_t x = ld1(X + mat_at(jb.k, c, r)), one = r == c ? kFixedOne : 0;
                 const bool negative = x > one;
                 const uint64_t d = static_cast<uint64_t>(one) - static_cast<uint64_t>(x);
                 Dout[static_cast<int64_t>(r) * n + c] = fixed_to_double(negative ? 0 - d : d, negative, -63);
             }
     }
     slices_end(sh);
-    if (threadIdx.x == 0) {
-        if (!aborted) hdr[0] = bad ? kErrNonfinite : (conv ? kOk : kErrNoconv);
+    if (threadIdx.x == 0 && cluster_rank() == 0) {
+        if (!aborted) atomicCAS(hdr, kOk, bad ? kErrNonfinite : (conv ? kOk : kErrNoconv));
         hdr[1] = done;
     }
 }
@@ -1054,8 +1153,9 @@ extern "C" smx_status smx_dense_density_noalloc(const double* h_dev, int32_t n, 
         scratch = g_noalloc_ptr[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    smx::k_dense_density_noalloc<<<1, smx::kSliceThreads, smx::kSliceSmem, st>>>(h_dev, n, mu, d_dev, scratch, 1e-7f, 100);
-    if (cudaGetLastError() != cudaSuccess) return SMX_ERR_CUDA;
+    if (smx::launch_clusters(smx::k_dense_density_noalloc, 1, smx::cluster_for(n), st, h_dev, static_cast<int>(n), mu, d_dev, scratch,
+                             1e-7f, 100) != cudaSuccess)
+        return SMX_ERR_CUDA;
     int hdr[2] = {0, 0};
     if (cudaMemcpyAsync(hdr, scratch + smx::kNoAllocBytes, sizeof(hdr), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return SMX_ERR_CUDA;

@@ -63,6 +63,7 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 struct smx_ctx {
     int device = 0;
     int num_sms = 0;
+    int clusters[4] = {0, 0, 0, 0};  // device_clusters, asked on the first 64-bit build
     cudaStream_t stream = nullptr;
 
     // input pattern
@@ -522,6 +523,7 @@ static smx_status read_status(smx_ctx* c);
 
 // Slots of the 64-bit kernels for m submatrices: one per persistent CTA (at most one per SM).
 static smx_status prepare_fp64_slots(smx_ctx* c, int m, int mats, int planes, int* slots, size_t* slot_bytes) {
+    if (!c->clusters[0]) SMX_CUDA(device_clusters(c->clusters));
     *slots = std::max(1, std::min(c->num_sms, m));
     *slot_bytes = fp64_slot_bytes(c->max_n, mats, planes);
     return ensure(c->d_ws64, *slot_bytes * static_cast<size_t>(*slots));
@@ -568,7 +570,7 @@ static smx_status nonorth_setup(smx_ctx* c) {
     a.iters = dp<int32_t>(c->d_setup_iters);
     a.lohi = dp<double>(c->d_nlohi);
     a.status = &scalars(c)->status;
-    SMX_CUDA(launch_nonorth_setup(a, slots, st));
+    SMX_CUDA(launch_nonorth_setup(a, slots, c->max_n, c->clusters, st));
     c->kernel_launches += 3;
     std::vector<double> lohi(2 * static_cast<size_t>(m));
     SMX_CUDA(cudaMemcpyAsync(lohi.data(), dp<double>(c->d_nlohi) + 2 * j0, sizeof(double) * lohi.size(), cudaMemcpyDeviceToHost, st));
@@ -678,7 +680,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
                 a.mu = mu;
             }
             SMX_CUDA(cudaEventRecord(ns0, st));
-            SMX_CUDA(launch_ns_fp64(a, std::min(slots, m), c->max_nblk, st));
+            SMX_CUDA(launch_ns_fp64(a, std::min(slots, m), c->max_n, c->max_nblk, c->clusters, st));
             SMX_CUDA(cudaEventRecord(ns1, st));
         } else {
             NsTcArgs a;
@@ -720,7 +722,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
                 f.max_iter = c->fp64_final;
                 f.use_model = 0;
                 f.finish_iters = c->fp64_final;
-                SMX_CUDA(launch_ns_fp64(f, std::min(slots, m), c->max_nblk, st));
+                SMX_CUDA(launch_ns_fp64(f, std::min(slots, m), c->max_n, c->max_nblk, c->clusters, st));
                 c->kernel_launches += 1;
             }
             SMX_CUDA(cudaEventRecord(ns1, st));

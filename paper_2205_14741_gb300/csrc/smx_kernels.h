@@ -89,7 +89,7 @@ cudaError_t launch_wait_selftest(int* status, uint32_t poll_limit, int* polls_ou
 // 1/2 (I - sign(A)), 1 = A^-1/2, 2 = A^1/2 (A = T_j - mu I symmetric positive definite).
 enum : int { kFnDensity = 0, kFnInvSqrt = 1, kFnSqrt = 2, kFnInv = 3, kFnFermi = 4 };
 
-// A CTA of the 64-bit kernels works in a slot of global memory: up to three k x k matrices of 64-bit
+// A CTA (or cluster) of the 64-bit kernels works in a slot of global memory: up to three k x k matrices of 64-bit
 // integers and the digits of up to three operands (smx_slices.cuh).
 constexpr int kFp64Mats = 3, kFp64Planes = 3;
 // Bytes of a slot for submatrices of up to max_n rows.
@@ -137,7 +137,10 @@ struct NsFp64Args {
     const int* skip = nullptr;  // when set and non-zero at launch, the kernel does nothing
     double beta = 0.0;          // kFnFermi: the inverse temperature (in inverse units of H)
 };
-cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_nblk, cudaStream_t st);
+// slots: clusters to launch; room: see device_clusters.
+cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_n, int max_nblk, const int* room, cudaStream_t st);
+// room[i]: how many clusters of 2^i CTAs of the 64-bit kernels the device holds at once, i = 0 .. 3.
+cudaError_t device_clusters(int* room);
 
 // Setup of the non-orthogonal form, once per (H, S): L_j = A_S^-1/2 (coupled iteration) and
 // M_j = L_j A_H L_j with its Gershgorin interval.
@@ -160,7 +163,7 @@ struct NonorthSetupArgs {
     double* lohi;           // out: [2 * B] Gershgorin interval of M_j
     int* status;
 };
-cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, cudaStream_t st);
+cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, int max_n, const int* room, cudaStream_t st);
 
 // a5 (tcgen05 tensor cores) + a7.
 struct NsTcArgs {

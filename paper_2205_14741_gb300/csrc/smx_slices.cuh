@@ -2,6 +2,9 @@
 // splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, with FP16 slices and
 // FP32 accumulation as in Mukunoki et al., ISC 2020).
 //
+// A cluster of CTAs may share the work of a submatrix: the tiles of a product and the units of an
+// elementwise pass go round the CTAs; whatever is decided from a reduction is decided alike by each.
+//
 // Numbers.  A matrix is held in fixed point: 64-bit integers in units of 2^-62.  An operand of a
 // product is cut into seven 8-bit digits,
 //     x = sum_{i=1..7} d_i 2^(-8 i),   |d_1| <= 256 (1 + a little), |d_i| <= 128,
@@ -63,6 +66,7 @@ struct SliceShared {
     uint32_t tmem;
     int abort;
     int kpart;       // chunks of one exact accumulation (fewer than kSliceK / 16 where an operand's rows are longer)
+    int tile;        // columns of a tile: kSliceTile, or half of it to have tiles for all CTAs of a larger cluster
     int weights;     // 7: the pairs of weights 2 .. 8; 8: of weight 9 too (kpart at most 10)
     // positions of the roles in the pipelines, continuous over the products of a CTA: chunks copied,
     // chunks multiplied, accumulations begun, accumulations read (each written by one role)
@@ -120,6 +124,35 @@ __device__ __forceinline__ int acc_steps(uint32_t v) {
     return 4 * (__float_as_int(t) - 0x4C400000) + acc_small(__float_as_uint(__fsub_rn(x, __fsub_rn(t, 50331648.0f))));
 }
 
+// The CTA's place in its cluster, and the cluster's size (1 without a cluster launch).
+__device__ __forceinline__ int cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return static_cast<int>(r);
+}
+__device__ __forceinline__ int cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return static_cast<int>(r);
+}
+
+// The end of a phase: what the cluster's threads wrote to global memory is seen by the others' loads
+// (which bypass L1: __ldcg) after it.  The cluster's barrier does not wait for threads that have exited,
+// so a CTA that gave up after a timeout holds no other one back.
+__device__ __forceinline__ void phase_sync() {
+    if (cluster_size() == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+    }
+}
+// The same where bulk copies read it.
+__device__ __forceinline__ void phase_sync_copies() {
+    fence_proxy_async_global();
+    phase_sync();
+    if (cluster_size() > 1) fence_proxy_async_global();
+}
+
 // Entries (r, c .. c + 7) of a matrix with k rows (c even).
 __device__ __forceinline__ int64_t mat_at(int k, int r, int c) {
     return ((static_cast<int64_t>(c >> 1) * k + r) << 1) + (c & 1);
@@ -128,7 +161,7 @@ __device__ __forceinline__ void ld8(const int64_t* m, int k, int r, int c, int64
     const longlong2* p = reinterpret_cast<const longlong2*>(m) + static_cast<int64_t>(c >> 1) * k + r;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const longlong2 x = p[static_cast<int64_t>(i) * k];
+        const longlong2 x = __ldcg(p + static_cast<int64_t>(i) * k);
         v[2 * i] = x.x;
         v[2 * i + 1] = x.y;
     }
@@ -146,6 +179,7 @@ __device__ void slices_begin(SliceShared* sh, uint8_t* smem, int* status) {
         sh->status = status;
         sh->kpart = kSliceK / 16;
         sh->weights = 7;
+        sh->tile = cluster_size() >= 4 ? kSliceTile / 2 : kSliceTile;
         sh->copied = sh->multiplied = sh->begun = sh->read = 0;
         for (int s = 0; s < kSliceStages; ++s) {
             mbar_init(&sh->full[s], 1);
@@ -202,7 +236,8 @@ __device__ __noinline__ void slice_product(SliceShared* sh, const uint8_t* __res
     volatile int* ab = &sh->abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mtiles = (k + 127) >> 7, chunks = k >> 4;
-    const int kpart = sh->kpart, weights = sh->weights;
+    const int kpart = sh->kpart, weights = sh->weights, tile = sh->tile;
+    const int ranks = cluster_size(), rank = cluster_rank();
     const int parts = (chunks + kpart - 1) / kpart;
     const uint32_t tmem = sh->tmem;
     if (warp == 0) {
@@ -210,9 +245,11 @@ __device__ __noinline__ void slice_product(SliceShared* sh, const uint8_t* __res
             const int64_t blk = static_cast<int64_t>(k) * 128 * kSlicePlanes * 2;  // bytes of a block of 128 rows
             uint32_t it = sh->copied;
             bool ok = true;
+            int turn = 0;
             for (int mt = 0; mt < mtiles && ok; ++mt)
-                for (int c0 = sym ? 128 * mt : 0; c0 < kb && ok; c0 += kSliceTile) {
-                    const uint32_t ra = static_cast<uint32_t>(min(128, k - 128 * mt)) * 32, w = static_cast<uint32_t>(min(kSliceTile, kb - c0)) * 32;
+                for (int c0 = sym ? 128 * mt : 0; c0 < kb && ok; c0 += tile) {
+                    if (turn++ % ranks != rank) continue;
+                    const uint32_t ra = static_cast<uint32_t>(min(128, k - 128 * mt)) * 32, w = static_cast<uint32_t>(min(tile, kb - c0)) * 32;
                     const uint32_t rb = static_cast<uint32_t>(min(128, kb - (c0 & ~127))) * 32;
                     const uint8_t* a = pa + mt * blk;
                     const uint8_t* b = pb + (c0 >> 7) * blk + (c0 & 127) * 32;
@@ -236,14 +273,16 @@ __device__ __noinline__ void slice_product(SliceShared* sh, const uint8_t* __res
         __syncwarp();
     } else if (warp == 1) {
         bool alive = true;
+        int turn = 0;
         for (int mt = 0; mt < mtiles && alive; ++mt)
-            for (int c0 = sym ? 128 * mt : 0; c0 < kb && alive; c0 += kSliceTile) {
+            for (int c0 = sym ? 128 * mt : 0; c0 < kb && alive; c0 += tile) {
+                if (turn++ % ranks != rank) continue;
                 // The products of one chunk, the same for every chunk of the tile, listed once (a lane per
                 // product): formed in the issuing loop, their descriptors would take longer than the products.
                 // A's plane i (from 1) takes B's planes 1 .. j1 = min(7, weights + 1 - i), in one or two
                 // instructions of N <= 256.  In the first chunk plane 1 opens the accumulators; that of weight
                 // 9 is opened by planes 2 and 7, on their own.
-                const int w = min(kSliceTile, kb - c0);
+                const int w = min(tile, kb - c0);
                 int count;
                 {
                     const uint32_t ra = static_cast<uint32_t>(min(128, k - 128 * mt)) * 32;
@@ -307,9 +346,11 @@ __device__ __noinline__ void slice_product(SliceShared* sh, const uint8_t* __res
         constexpr int kTurns = (kSliceTile / 4 + 2) / 3;
         uint32_t use = sh->read;
         bool alive = true;
+        int turn = 0;
         for (int mt = 0; mt < mtiles && alive; ++mt)
-            for (int c0 = sym ? 128 * mt : 0; c0 < kb && alive; c0 += kSliceTile) {
-                const int w = min(kSliceTile, kb - c0);
+            for (int c0 = sym ? 128 * mt : 0; c0 < kb && alive; c0 += tile) {
+                if (turn++ % ranks != rank) continue;
+                const int w = min(tile, kb - c0);
                 int64_t sum[kTurns][4];
                 for (int p = 0; p < parts; ++p) {
                     // one lane polls; the other warps wait at a barrier without touching shared memory, whose
@@ -385,7 +426,7 @@ __device__ __noinline__ void slice_product(SliceShared* sh, const uint8_t* __res
             }
         if (warp == 2 && lane == 0) sh->read = use;  // (every reader took its copy before the last barrier)
     }
-    __syncthreads();
+    phase_sync();
 }
 
 // Digits of eight neighbouring values of a row (units of 2^-62) to the seven planes, 16 bytes each.
@@ -422,13 +463,14 @@ __device__ __forceinline__ void store_digits(const int64_t (&q)[8], uint8_t* dst
 
 // An elementwise pass: f(r, c, v, q) turns the values v loaded by load(r, c, v) (eight from each of N
 // matrices) into the values q = (r, c .. c + 7) of an operand of rows x k (zero past the matrix); their
-// digits go to the planes (null: f alone).  Ends with the proxy fence and a barrier that the next
-// product needs.  Lane pairs take the two halves of a plane's 32-byte row, 16 rows a warp.
+// digits go to the planes (null: f alone).  Ends a phase.  Lane pairs take the two halves of a plane's
+// 32-byte row, 16 rows a warp.
 template <int N, class L, class F>
 __device__ __forceinline__ void slice_pass(int rows, int k, uint8_t* planes, L load, F f) {
+    const int first = cluster_rank() * kSliceThreads + threadIdx.x, step = cluster_size() * kSliceThreads;
     const int units = rows * (k >> 3), half = threadIdx.x & 1;
-    int r = threadIdx.x >> 1, c = 8 * half;
-    for (int u = threadIdx.x; u < units; u += kSliceThreads, r += kSliceThreads / 2) {
+    int r = first >> 1, c = 8 * half;
+    for (int u = first; u < units; u += step, r += step >> 1) {
         while (r >= rows) {
             r -= rows;
             c += 16;
@@ -443,8 +485,7 @@ __device__ __forceinline__ void slice_pass(int rows, int k, uint8_t* planes, L l
             store_digits(q, dst, static_cast<int64_t>(rb) * 32);
         }
     }
-    fence_proxy_async_global();
-    __syncthreads();
+    phase_sync_copies();
 }
 
 // ---------------------------------------------------------------------------
@@ -507,6 +548,26 @@ __device__ __forceinline__ float cta_sum(float v, SliceShared* sh) {
     float s = 0.0f;
     for (int w = 0; w < kSliceWarps; ++w) s += sh->red[w];
     return s;
+}
+// The sum over the cluster; scratch: one float per CTA in global memory.
+__device__ __noinline__ float cluster_sum(float v, SliceShared* sh, float* scratch) {
+    v = cta_sum(v, sh);
+    const int ranks = cluster_size();
+    if (ranks == 1) return v;
+    if (threadIdx.x == 0) __stcg(scratch + cluster_rank(), v);
+    phase_sync();
+    float s = 0.0f;
+    for (int r = 0; r < ranks; ++r) s += __ldcg(scratch + r);
+    return s;
+}
+// The maximum over the cluster of one value per CTA (the same for its threads); scratch as above.
+__device__ __forceinline__ uint32_t cluster_max(uint32_t v, uint32_t* scratch) {
+    const int ranks = cluster_size();
+    if (ranks == 1) return v;
+    if (threadIdx.x == 0) __stcg(scratch + cluster_rank(), v);
+    phase_sync();
+    for (int r = 0; r < ranks; ++r) v = max(v, __ldcg(scratch + r));
+    return v;
 }
 __device__ __forceinline__ float cta_max(float v, SliceShared* sh) {
 #pragma unroll

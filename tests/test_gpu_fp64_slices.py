@@ -122,3 +122,30 @@ def test_not_positive_definite_is_reported():
         c.set_mu(0.0)
         c.build_density()
         c.get_trace()
+
+
+@pytest.mark.parametrize("f", ["density", "inv", "fermi", "overlap"])
+@pytest.mark.parametrize("m,b", [(100, 2), (100, 1)])
+def test_clusters_change_no_bit(m, b, f):
+    # 100 submatrices take one SM each; column ranges of 60, 30 and 9 take clusters of two, four and eight SMs
+    # (n = 200; at n = 100 up to four).  Sums are of integers, and every SM decides from the same ones.
+    from paper_2205_14741_gb300 import SubmatrixDensity
+
+    if f == "overlap":
+        h, s = make_nonorth_pair(m, b, np.inf, 1.5, 9, sigma_s=0.02)
+    else:
+        h, s = make_mixed_block_system([b] * m, r_c=np.inf, ell=1.5, seed=4), None
+    with SubmatrixDensity.from_system(h) as c:
+        if s is not None:
+            c.set_overlap(s.values)
+        else:
+            c.set_function(f)
+            c.set_fermi_beta(12.0)
+        lam = np.linalg.eigvalsh(O.to_dense(h.block_size, h.col_ptr, h.row_idx, h.values))
+        c.set_mu(float(lam[0]) - 0.5 if f == "inv" else 0.02)
+        c.build_density()
+        full = c.get_density().reshape(m, -1)
+        for j0, j1 in ((3, 63), (40, 70), (91, 100)):
+            c.set_column_range(j0, j1)
+            c.build_density()
+            assert np.array_equal(c.get_density().reshape(m, -1)[j0:j1], full[j0:j1]), (j0, j1)
