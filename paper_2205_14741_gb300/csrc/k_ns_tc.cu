@@ -361,9 +361,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         __syncthreads();
     };
 
-    // Jobs are claimed one ahead: while a submatrix iterates, its successor's staged
-    // T_j is prefetched into L2 (the prologue then reads it from there).
-    __shared__ int next_s;
+    // A job's successor is claimed when the job nears its end (kNearEnd), and its staged T_j is then
+    // prefetched into L2 (the prologue reads it from there).  Not earlier: the jobs are ordered by size, and
+    // a CTA that claims while it still has a large one to do keeps the next largest waiting.
+    constexpr float kNearEnd = 0.25f;  // residual ||X^2 - I||_F: two or three steps are left
+    __shared__ int next_s, claimed_s;
     __shared__ float rprev_s;  // the previous step's residual (rounding-floor stop)
     // the job's scalars in FP32: 1 / b_j, the predicted smallest |eigenvalue| of
     // X0 = (T_j - mu I) / b_j (negative when there is no prediction), and b_j / G_j; with b_j
@@ -374,12 +376,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
     __shared__ double next_b_s;
     // Claims the successor of the current job: one atomic, its descriptors, a prefetch of its
     // staged T_j into L2, and its scalars (FP32 divisions: FP64 division is slow on this GPU's
-    // FP64 pipe).  Run by one thread: thread 0 for the first job, then warp 11's first lane
-    // while the job's first product is multiplied, so that no CTA barrier waits for its
-    // memory round trips; the loop head takes the results from shared memory.
+    // FP64 pipe).  Run by one thread: thread 0 for the first job and in the streamed form, warp 11's
+    // first lane while a product is multiplied in the on-chip form, so that no CTA barrier waits
+    // for its memory round trips; the loop head takes the results from shared memory.
     auto claim_next = [&]() {
         const int nx = atomicAdd(a.work_counter, 1);
         next_s = nx;
+        claimed_s = 1;
         if (nx < a.n_subs) {
             const int jj = a.order[nx];
             const SubDesc sn = a.subs[jj];
@@ -401,6 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
     for (;;) {
         if (tid == 0) {
             job_s = next_s;
+            claimed_s = 0;
             inv_b_s = next_inv_b_s;
             dhat_s = next_dhat_s;
             bg_s = next_bg_s;
@@ -486,7 +490,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             fence_proxy_async_smem();
             if (tid == 0) { conv_s = 0; bad_s = 0; plain_s = 0; rprev_s = INFINITY; }
             __syncthreads();
-            if (warp == 11 && lane == 0) claim_next();  // while the first product runs
         } else {
             const float inv_b = inv_b_s;
             const float* t = a.T + s.t_off;
@@ -526,7 +529,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             fence_proxy_async_global();
             if (tid == 0) { conv_s = 0; bad_s = 0; plain_s = 0; rprev_s = INFINITY; }
             __syncthreads();
-            if (warp == 11 && lane == 0) claim_next();  // while the first product runs
         }
 
         // The factor c of the first step X1 = p(c X0), p(x) = x (3 - x^2) / 2, from the guaranteed
@@ -1090,6 +1092,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                         issue_xx(0, TA);
                         tc_commit(&mma_bar);
                     }
+                    if (warp == 11 && lane == 0 && !claimed_s && rprev_s < kNearEnd) claim_next();
                     mma_wait();  // Z
                     if (it == 0) {
                         __syncthreads();
@@ -1156,6 +1159,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                         issue_xx_cols(1, TB, 128, idesc_w);
                         tc_commit(&mma_bar2);
                     }
+                    if (warp == 11 && lane == 0 && !claimed_s && rprev_s < kNearEnd) claim_next();
                     mma_wait();  // Z_0
                     if (it == 0) {
                         mma_wait2();  // Z_c
@@ -1347,6 +1351,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     float r2 = 0.0f;
                     for (int w = 0; w < kEpiWarps; ++w) r2 += resid_s[w];
                     check_stop(sqrtf(r2));
+                    if (conv_s || bad_s || it + 1 == a.max_iter) claim_next();  // the last product follows
                 }
                 gemm(kpad, s.n, 2, zx, zy, zn, 1.0f);  // X' = X Y
             }
@@ -1356,6 +1361,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         }
         }  // streamed form
         if (*abortp) break;
+        if (warp == 11 && lane == 0 && !claimed_s) claim_next();
         if (tid == 0) {
             a.iters[j] = done;
             atomicAdd(a.work_n3, static_cast<unsigned long long>(s.n) * s.n * s.n * done);
