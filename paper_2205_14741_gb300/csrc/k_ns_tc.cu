@@ -31,8 +31,14 @@
 //   warps 4..11  epilogue: tcgen05.ld, Y = 3/2 I - 1/2 acc (or X' = acc),
 //                residual ||X^2 - I||_F^2 in FP32, split to hi/lo, 16-byte
 //                stores to the slot (L2-resident)
+// Large submatrices are shared by clusters of four CTAs (k_ns_tc<., true>, see share()): each product's
+// tiles, the prologue and the bound's passes are dealt out to the CTAs, which meet at a cluster barrier
+// after every product; the slot, in global memory, is the cluster's.  343 submatrices of n = 943 .. 1196
+// (split FP16): 55.0 -> 38.1 ms.
 // On-chip form (up to 192): all 12 warps share the tensor-memory passes; one
 // lane of warp 1 issues the MMAs (of warp 10 the next iteration's in two-tile form).
+#include <climits>
+
 #include "smx_finish.cuh"
 #include "smx_kernels.h"
 #include "smx_tc_common.cuh"
@@ -40,7 +46,8 @@
 namespace smx {
 
 
-template <int PREC>
+// SHARED: clusters of kTcCluster CTAs work on one submatrix in the streamed form (launch_prec).
+template <int PREC, bool SHARED>
 __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_constant__ CUtensorMap tmap) {
     using C = TcCfg<PREC>;
     constexpr int NB = C::kNb, S = C::kStages, NT = C::kNmax;
@@ -118,7 +125,30 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
     uint32_t e_nb = 0;                  // epilogue: the buffer of the next single-chain tile
     const int64_t buf = static_cast<int64_t>(a.ld) * a.ld;
     uint16_t* ws = static_cast<uint16_t*>(a.ws);
-    const int slot_z = blockIdx.x * 6;
+    constexpr int kRanks = SHARED ? kTcCluster : 1;
+    const int rank = SHARED ? cluster_rank() : 0;
+    const int slot_z = static_cast<int>(blockIdx.x) / kRanks * 6;
+    float* const xch = a.exchange + (blockIdx.x / kRanks) * kTcExchange;  // of the cluster
+    // the end of a phase whose global writes the cluster's CTAs read
+    auto sync_all = [&] {
+        if constexpr (SHARED) phase_sync_copies();
+        else __syncthreads();
+    };
+    // The tiles of a product go to the CTA with the least columns so far (each role of each CTA keeps the
+    // same count): load counts columns, and 64 for what a tile costs besides.
+    auto take = [&](int (&load)[kRanks], int columns) -> bool {
+        if constexpr (!SHARED) return true;
+        int to = 0, least = load[0];
+#pragma unroll
+        for (int r = 1; r < kRanks; ++r)
+            if (load[r] < least) {
+                least = load[r];
+                to = r;
+            }
+#pragma unroll
+        for (int r = 0; r < kRanks; ++r) load[r] += r == to ? columns + 64 : 0;
+        return to == rank;
+    };
     uint32_t mma_ph = 0, mma_ph2 = 0;  // completed phases of mma_bar, mma_bar2 (uniform over the CTA)
     const uint32_t idesc_b_mn = 1u << 16;  // B operand MN-major
 
@@ -145,9 +175,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         auto ntiles_of = [&](int mt) { return (kpad - 128 * mt + NT - 1) / NT; };
         if (warp == 0) {
             if (elect_one()) {
+                int load[kRanks] = {};
                 for (int mt = 0; mt < mtiles && !*abortp; ++mt)
                     for (int nt = 0; nt < ntiles_of(mt) && !*abortp; ++nt) {
                         const int n0 = 128 * mt + NT * nt, nn = min(NT, kpad - n0);
+                        if (!take(load, nn)) continue;
                         for (int kc = 0; kc < kchunks; ++kc) {
                             const int stage = p_it % S;
                             const uint32_t round = p_it / S;
@@ -171,9 +203,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             __syncwarp();
         } else if (warp == 1) {
             if (elect_one()) {
+                int load[kRanks] = {};
                 for (int mt = 0; mt < mtiles && !*abortp; ++mt)
                     for (int nt = 0; nt < ntiles_of(mt) && !*abortp; ++nt) {
                         const int nn = min(NT, kpad - 128 * mt - NT * nt);
+                        if (!take(load, nn)) continue;
                         // the buffer(s) of this tile, released by the epilogue of their previous tiles
                         const uint32_t abuf = split ? 0u : m_nb;
                         if (!split) m_nb ^= 1u;
@@ -227,9 +261,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             // (conflict-free 16-byte row writes, 2-byte column reads)
             uint16_t* xs = reinterpret_cast<uint16_t*>(smem + C::kXposeOff + (warp - 4) * C::kXposeWarp);
             float r2 = 0.0f;
+            int load[kRanks] = {};
             for (int mt = 0; mt < mtiles; ++mt)
                 for (int nt = 0; nt < ntiles_of(mt); ++nt) {
                     const int n0 = 128 * mt + NT * nt, nn = min(NT, kpad - n0);
+                    if (!take(load, nn)) continue;
                     const uint32_t abuf = split ? 0u : e_nb;
                     if (!split) e_nb ^= 1u;
                     const uint32_t ph = (abuf ? e_full1++ : e_full0++) & 1u;
@@ -356,9 +392,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
             if (lane == 0) resid_s[warp - 4] = r2;
+            if (SHARED && lane == 0 && mode == 1) __stcg(xch + rank * kEpiWarps + warp - 4, r2);
             fence_proxy_async_global();
         }
-        __syncthreads();
+        sync_all();
     };
 
     // A job's successor is claimed when the job nears its end (kNearEnd), and its staged T_j is then
@@ -379,8 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
     // FP64 pipe).  Run by one thread: thread 0 for the first job and in the streamed form, warp 11's
     // first lane while a product is multiplied in the on-chip form, so that no CTA barrier waits
     // for its memory round trips; the loop head takes the results from shared memory.
-    auto claim_next = [&]() {
-        const int nx = atomicAdd(a.work_counter, 1);
+    auto describe = [&](int nx) {
         next_s = nx;
         claimed_s = 1;
         if (nx < a.n_subs) {
@@ -391,7 +427,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             const float g = static_cast<float>(a.gersh[jj]);
             const uint64_t bytes = static_cast<uint64_t>(sn.n) * sn.ld * sizeof(float);
             const uint32_t len = static_cast<uint32_t>(bytes < (4u << 20) ? bytes : (4u << 20)) & ~15u;
-            if (len) prefetch_l2_bulk(a.T + sn.t_off, len);
+            if (len && !SHARED) prefetch_l2_bulk(a.T + sn.t_off, len);
             const float bf = static_cast<float>(b);
             next_b_s = b;
             next_inv_b_s = 1.0f / bf;
@@ -399,9 +435,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             next_dhat_s = a.pred ? pr * (g / bf) : -1.0f;
         }
     };
-    if (tid == 0) claim_next();
+    auto claim_next = [&]() { describe(atomicAdd(a.work_counter, 1)); };
+    if (!SHARED && tid == 0) claim_next();
     __syncthreads();
     for (;;) {
+        if constexpr (SHARED) {  // the first CTA claims; all have left the submatrix before
+            if (tid == 0 && rank == 0) __stcg(reinterpret_cast<int*>(xch) + kTcExchangeJob, atomicAdd(a.work_counter, 1));
+            sync_all();
+            if (tid == 0) describe(__ldcg(reinterpret_cast<int*>(xch) + kTcExchangeJob));
+        }
         if (tid == 0) {
             job_s = next_s;
             claimed_s = 0;
@@ -426,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         const int zx0 = slot_z + 0, zx1 = slot_z + 2, zy = slot_z + 4;
 
         // on-chip form: the image of X (hi boxes, then lo boxes) at the start of the stage area
-        const bool resident = kpad <= kResKpad;
+        const bool resident = !SHARED && kpad <= kResKpad;
         const int RB = (kpad + 63) >> 6;
         const uint32_t img_bytes = static_cast<uint32_t>(RB * RB) * 8192u;
         const uint32_t hi_off = 0u, lo_off = img_bytes;  // hi image, lo image (split form)
@@ -497,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             uint16_t* xl = xh + buf;
             const int per_row = kpad / 8, total = kpad * per_row;
             constexpr int kU = 4;  // loads in flight per thread
-            for (int e0 = tid; e0 < total; e0 += kU * kThreads) {
+            for (int e0 = tid + rank * kU * kThreads; e0 < total; e0 += kRanks * kU * kThreads) {
                 float4 v[kU][2];
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
@@ -528,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             }
             fence_proxy_async_global();
             if (tid == 0) { conv_s = 0; bad_s = 0; plain_s = 0; rprev_s = INFINITY; }
-            __syncthreads();
+            sync_all();
         }
 
         // The factor c of the first step X1 = p(c X0), p(x) = x (3 - x^2) / 2, from the guaranteed
@@ -552,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     } else {
                         c = fmaxf(1.0f, c);
                     }
-                } else if (tid == 0) {
+                } else if (tid == 0 && rank == 0) {
                     atomicAdd(a.fallbacks, 1);
                 }
             }
@@ -1254,7 +1296,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     const uint16_t* zl = zh + buf;
                     // row sums of |Z|, eight rows per warp at a time, 8 columns per lane and load
                     constexpr int kR = 8;
-                    for (int r0 = warp * kR; r0 < kpad; r0 += kR * (kThreads / 32)) {
+                    for (int r0 = (warp + rank * (kThreads / 32)) * kR; r0 < kpad; r0 += kRanks * kR * (kThreads / 32)) {
                         float acc[kR];
 #pragma unroll
                         for (int u = 0; u < kR; ++u) acc[u] = 0.0f;
@@ -1275,7 +1317,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                         }
                     }
                 }
-                __syncthreads();
+                sync_all();
                 float rmax = 0.0f;
                 for (int r = tid; r < s.n; r += kThreads) rmax = fmaxf(rmax, wv[r]);
                 rmax = block_max2(rmax, 0.0f).x;
@@ -1283,20 +1325,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                 uint16_t* zh = ws + static_cast<int64_t>(zy) * buf;
                 uint16_t* zl = zh + buf;
                 if (rmax > 0.0f) {  // (a pass over Z is cheap next to the products at these sizes)
-                    // w > 0: rows that are zero in Z get a tiny positive weight
-                    for (int c = tid; c < s.n; c += kThreads) wv[c] = fmaxf(wv[c], 1e-12f * rmax);
-                    __syncthreads();
+                    const float wmin = 1e-12f * rmax;  // w > 0: rows that are zero in Z get a tiny positive weight
                     float q = 0.0f;
                     // (|Z| w)_r for eight rows per warp at a time, 8 columns per lane and load
                     constexpr int kR = 8;
-                    for (int r0 = warp * kR; r0 < s.n; r0 += kR * (kThreads / 32)) {
+                    for (int r0 = (warp + rank * (kThreads / 32)) * kR; r0 < s.n; r0 += kRanks * kR * (kThreads / 32)) {
                         float acc[kR];
 #pragma unroll
                         for (int u = 0; u < kR; ++u) acc[u] = 0.0f;
                         for (int c = 8 * lane; c < kpad; c += 256) {
                             const float4 w0 = *reinterpret_cast<const float4*>(wv + c);
                             const float4 w1 = *reinterpret_cast<const float4*>(wv + c + 4);
-                            const float wc[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+                            const float wc[8] = {fmaxf(w0.x, wmin), fmaxf(w0.y, wmin), fmaxf(w0.z, wmin), fmaxf(w0.w, wmin),
+                                                 fmaxf(w1.x, wmin), fmaxf(w1.y, wmin), fmaxf(w1.z, wmin), fmaxf(w1.w, wmin)};
                             float zr[kR][8];
 #pragma unroll
                             for (int u = 0; u < kR; ++u) {
@@ -1311,16 +1352,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
 #pragma unroll
                         for (int u = 0; u < kR; ++u) {
                             const float v = warp_sum_f(acc[u]);
-                            if (r0 + u < s.n) q = fmaxf(q, v / wv[r0 + u]);
+                            if (r0 + u < s.n) q = fmaxf(q, v / fmaxf(wv[r0 + u], wmin));
                         }
                     }
-                    best = fminf(best, block_max2(q, 0.0f).x);
+                    q = block_max2(q, 0.0f).x;
+                    if constexpr (SHARED) {
+                        if (tid == 0) __stcg(xch + kTcExchangeMax + rank, q);
+                        sync_all();
+                        for (int r = 0; r < kRanks; ++r) q = fmaxf(q, __ldcg(xch + kTcExchangeMax + r));
+                    }
+                    best = fminf(best, q);
                 }
                 const float smax = sqrtf(best * (1.0f + 1e-4f));  // margin for FP32 summation
                 const float scale = start_factor(smax);
                 // Z_rr -= 3 / c^2 (in place, the split re-done)
                 const float shift = 3.0f / (scale * scale);
-                for (int r = tid; r < s.n; r += kThreads) {
+                for (int r = tid + rank * kThreads; r < s.n; r += kRanks * kThreads) {
                     const int64_t o = static_cast<int64_t>(r) * a.ld + r;
                     float z = from16<PREC>(zh[o]);
                     if constexpr (NB == 2) z += from16<PREC>(zl[o]);
@@ -1334,13 +1381,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                     }
                 }
                 fence_proxy_async_global();
-                if (tid == 0) {
+                if (tid == 0 && rank == 0) {
                     // feature of the next snapshot: the Gershgorin bound of A^2, over G; and the
                     // effective scaling b_j / c of X0'
                     a.sq_ratio[j] = sqrtf(rmax * (1.0f + 1e-5f)) * bg_s;
                     a.bound[j] = b_s * static_cast<double>(1.0f / scale);
                 }
-                __syncthreads();
+                sync_all();
                 gemm(kpad, s.n, 2, zx, zy, zn, -0.5f * scale * scale * scale);  // X1 = -c^3/2 X0 (Z - 3/c^2 I)
             } else {
                 float shift = 3.0f, alpha = -0.5f;
@@ -1349,9 +1396,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
                 gemm(kpad, s.n, 1, zx, zx, zy, alpha, -alpha * shift);  // Y = 3/2 I - 1/2 X^2 when plain
                 if (tid == 0) {
                     float r2 = 0.0f;
-                    for (int w = 0; w < kEpiWarps; ++w) r2 += resid_s[w];
+                    if constexpr (SHARED) {
+                        for (int w = 0; w < kRanks * kEpiWarps; ++w) r2 += __ldcg(xch + w);
+                    } else {
+                        for (int w = 0; w < kEpiWarps; ++w) r2 += resid_s[w];
+                    }
                     check_stop(sqrtf(r2));
-                    if (conv_s || bad_s || it + 1 == a.max_iter) claim_next();  // the last product follows
+                    if (!SHARED && (conv_s || bad_s || it + 1 == a.max_iter)) claim_next();  // the last product follows
                 }
                 gemm(kpad, s.n, 2, zx, zy, zn, 1.0f);  // X' = X Y
             }
@@ -1361,8 +1412,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         }
         }  // streamed form
         if (*abortp) break;
-        if (warp == 11 && lane == 0 && !claimed_s) claim_next();
-        if (tid == 0) {
+        if (!SHARED && warp == 11 && lane == 0 && !claimed_s) claim_next();
+        if (tid == 0 && rank == 0) {
             a.iters[j] = done;
             atomicAdd(a.work_n3, static_cast<unsigned long long>(s.n) * s.n * s.n * done);
             if (bad_s) atomicCAS(a.status, kOk, kErrNonfinite);
@@ -1371,7 +1422,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         // the whole final X for FP64 finishing steps
         if (a.xfull) {
             double* xf = a.xfull + s.t_off;
-            for (int e = tid; e < s.n * s.n; e += blockDim.x) {
+            for (int e = tid + rank * kThreads; e < s.n * s.n; e += kRanks * kThreads) {
                 const int r = e / s.n, c = e - r * s.n;
                 float x;
                 if (resident) {
@@ -1402,7 +1453,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
             } else {
                 const uint16_t* fh = ws + static_cast<int64_t>(cur ? zx1 : zx0) * buf;
                 const uint16_t* fl = fh + buf;
-                for (int e = tid; e < s.n * s.bown; e += blockDim.x) {
+                for (int e = tid + rank * kThreads; e < s.n * s.bown; e += kRanks * kThreads) {
                     const int q = e / s.n, i = e - q * s.n;
                     const int64_t o = static_cast<int64_t>(i) * a.ld + s.own + q;
                     float x = from16<PREC>(fh[o]);
@@ -1413,6 +1464,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_ns_tc(NsTcArgs a, const __grid_
         }
         __syncthreads();
     }
+
+    // (a first CTA that gave up leaves its cluster no job to find)
+    if (SHARED && tid == 0 && rank == 0) __stcg(reinterpret_cast<int*>(xch) + kTcExchangeJob, INT_MAX);
 
     // teardown: on a timeout, let copies and MMAs in flight finish (bounded) before freeing TMEM
     __syncthreads();
@@ -1440,21 +1494,70 @@ size_t ns_tc_smem_bytes(int precision) {
     }
 }
 
-template <int PREC>
-static cudaError_t launch_prec(const NsTcArgs& a, const CUtensorMap& tmap, int max_nblk, cudaStream_t st) {
-    (void)max_nblk;
-    const size_t smem = TcCfg<PREC>::kDynSmem;
-    cudaError_t e = cudaFuncSetAttribute(k_ns_tc<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    k_ns_tc<PREC><<<a.n_slots, kThreads, smem, st>>>(a, tmap);
-    return cudaGetLastError();
+template <int PREC, bool SHARED>
+static cudaLaunchConfig_t tc_config(int ctas, cudaStream_t st, cudaLaunchAttribute* attr) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = kTcCluster;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(ctas));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = TcCfg<PREC>::kDynSmem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = SHARED ? 1 : 0;
+    return cfg;
 }
 
-cudaError_t launch_ns_tc(const NsTcArgs& a, int precision, const CUtensorMap& tmap, int max_nblk, cudaStream_t st) {
+template <int PREC, bool SHARED>
+static cudaError_t launch_prec(const NsTcArgs& a, const CUtensorMap& tmap, int ctas, cudaStream_t st) {
+    auto kernel = k_ns_tc<PREC, SHARED>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(TcCfg<PREC>::kDynSmem));
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = tc_config<PREC, SHARED>(ctas, st, &attr);
+    return cudaLaunchKernelEx(&cfg, kernel, a, tmap);
+}
+
+template <int PREC>
+static cudaError_t clusters_prec(int* room) {
+    auto kernel = k_ns_tc<PREC, true>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(TcCfg<PREC>::kDynSmem));
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = tc_config<PREC, true>(kTcCluster, nullptr, &attr);
+    return cudaOccupancyMaxActiveClusters(room, kernel, &cfg);
+}
+
+cudaError_t ns_tc_clusters(int precision, int* room) {
     switch (precision) {
-        case 1: return launch_prec<1>(a, tmap, max_nblk, st);
-        case 2: return launch_prec<2>(a, tmap, max_nblk, st);
-        case 3: return launch_prec<3>(a, tmap, max_nblk, st);
+        case 1: return clusters_prec<1>(room);
+        case 2: return clusters_prec<2>(room);
+        case 3: return clusters_prec<3>(room);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// Whether clusters of four CTAs share the submatrices (all of them streamed).  With one CTA each, a wave of
+// 152 submatrices works on 152 (hi, lo) sets of X, Y and X', far more than L2 holds, and every tile's
+// panels come from HBM; 36 clusters keep a quarter of it alive, read a submatrix's panels at about the same time
+// and leave a shorter last wave, but wait for one another at every product.  Builds with one CTA / a cluster
+// per submatrix: split FP16, 304 of n = 304 1.48 / 2.43 ms, 456 of n = 456 5.48 / 5.86, 304 of n = 608
+// 5.95 / 5.44, of n = 800 13.3 / 10.6 ms; FP16 n = 608 2.69 / 2.91, n = 800 5.87 / 5.23 ms.  So the line
+// lies at three operands of 3.3 MB.  Where all find room as clusters, they share at any size.
+static bool share(int precision, int n_subs, int min_n, int room) {
+    if (room < 1 || min_n <= kResKpad) return false;
+    const int64_t bytes = int64_t(3) * 2 * (precision == 1 ? 2 : 1) * min_n * min_n;
+    return n_subs <= room || bytes > 3300000;
+}
+
+cudaError_t launch_ns_tc(const NsTcArgs& a, int precision, const CUtensorMap& tmap, int min_n, int room, cudaStream_t st) {
+    const bool s = share(precision, a.n_subs, min_n, room);
+    const int ctas = s ? (a.n_slots < room ? a.n_slots : room) * kTcCluster : a.n_slots;
+    switch (precision) {
+        case 1: return s ? launch_prec<1, true>(a, tmap, ctas, st) : launch_prec<1, false>(a, tmap, ctas, st);
+        case 2: return s ? launch_prec<2, true>(a, tmap, ctas, st) : launch_prec<2, false>(a, tmap, ctas, st);
+        case 3: return s ? launch_prec<3, true>(a, tmap, ctas, st) : launch_prec<3, false>(a, tmap, ctas, st);
         default: return cudaErrorInvalidValue;
     }
 }

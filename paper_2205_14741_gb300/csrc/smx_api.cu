@@ -63,6 +63,7 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 struct smx_ctx {
     int device = 0;
     int num_sms = 0;
+    int tc_clusters = 0;             // ns_tc_clusters of the precision the workspace is for
     int clusters[4] = {0, 0, 0, 0};  // device_clusters, asked on the first 64-bit build
     cudaStream_t stream = nullptr;
 
@@ -92,7 +93,7 @@ struct smx_ctx {
     std::vector<int32_t> maps;     // block maps of the submatrices (empty: built by the gather)
     std::vector<int64_t> map_off;
     std::vector<SubDesc> subs;
-    int max_nblk = 0, max_n = 0;
+    int max_nblk = 0, max_n = 0, min_n = 0;
     int64_t t_elems = 0, x_elems = 0;
 
     // device buffers
@@ -102,7 +103,7 @@ struct smx_ctx {
     DevBuf d_sc;                      // DevScalars: status, flags, bracket, trace and energy
     DevScalars* h_sc = nullptr;       // pinned copy, filled by fetch()
     DevBuf d_fcol_ptr, d_frow_idx, d_fvoff, d_lstart, d_subs, d_order, d_maps, d_map_off;
-    DevBuf d_T, d_W1, d_ws, d_ws64, d_D, d_xown;
+    DevBuf d_T, d_W1, d_ws, d_tc_exchange, d_ws64, d_D, d_xown;
     DevBuf d_bound, d_iters, d_partial, d_work_n3;
     uint8_t* h_keep_pinned = nullptr;
 
@@ -350,6 +351,7 @@ static smx_status compact(smx_ctx* c) {
     c->subs.assign(B, SubDesc{});
     c->max_nblk = 0;
     c->max_n = 0;
+    c->min_n = INT32_MAX;
     int64_t t_off = 0, x_off = 0;
     const int64_t chunk_elems = std::max<int64_t>(1, staging_chunk_elems(c));
     const int32_t lo = c->col_lo, hi = c->col_hi < 0 ? B : c->col_hi;
@@ -387,6 +389,7 @@ static smx_status compact(smx_ctx* c) {
         x_off += round_up(static_cast<int64_t>(s.n) * s.bown, 32);
         c->max_nblk = std::max(c->max_nblk, s.nblk);
         c->max_n = std::max(c->max_n, s.n);
+        c->min_n = std::min(c->min_n, s.n);
     }
     c->chunk_start.push_back(hi);
     c->t_elems = c->t_chunk_max;
@@ -446,8 +449,10 @@ static smx_status prepare_tc_workspace(smx_ctx* c) {
     const int slots = std::max(1, std::min(c->num_sms, c->B));
     if (c->ws_prec == c->precision && c->ws_ld >= ld && c->ws_slots == slots) return SMX_OK;
     SMX_TRY(get_encoder(c));
+    SMX_CUDA(ns_tc_clusters(c->precision, &c->tc_clusters));
     const size_t bytes = static_cast<size_t>(slots) * 6 * ld * ld * 2;
     SMX_TRY(ensure(c->d_ws, bytes));
+    SMX_TRY(ensure(c->d_tc_exchange, static_cast<size_t>(slots) * kTcExchange * sizeof(float)));
     SMX_CUDA(cudaMemsetAsync(c->d_ws.p, 0, bytes, c->stream));
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(ld), static_cast<cuuint64_t>(ld), static_cast<cuuint64_t>(slots) * 6};
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * 2, static_cast<cuuint64_t>(ld) * ld * 2};
@@ -692,6 +697,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
             a.bound = dp<double>(c->d_bound);
             a.ws = c->d_ws.p;
             a.ld = c->ws_ld;
+            a.exchange = dp<float>(c->d_tc_exchange);
             a.n_slots = std::min(c->ws_slots, m);
             a.tau = static_cast<float>(tau_for(c->precision));
             a.stall_level = (c->precision == SMX_FP16 || c->precision == SMX_BF16) ? kStallLevel : 0.0f;
@@ -712,7 +718,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
             a.xown = dp<float>(c->d_xown);
             if (finish) a.xfull = dp<double>(c->d_W1);
             SMX_CUDA(cudaEventRecord(ns0, st));
-            SMX_CUDA(launch_ns_tc(a, c->precision, c->tmap, c->max_nblk, st));
+            SMX_CUDA(launch_ns_tc(a, c->precision, c->tmap, c->min_n, c->tc_clusters, st));
             if (finish) {
                 // FP64 finishing steps on the bulk phase's last iterate, then the scatter (the
                 // tensor-core scatter, which also resets the job counter, is not run)
@@ -1486,7 +1492,7 @@ void smx_destroy(smx_ctx* c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     DevBuf* bufs[] = {&c->d_H, &c->d_H32, &c->d_voff, &c->d_row_idx, &c->d_col_ptr, &c->d_bs, &c->d_keep_prev, &c->d_sc, &c->d_keep, &c->d_fcol_ptr,
                       &c->d_frow_idx, &c->d_fvoff, &c->d_lstart, &c->d_subs, &c->d_order, &c->d_T, &c->d_W1,
-                      &c->d_ws, &c->d_ws64, &c->d_maps, &c->d_map_off, &c->d_pairs, &c->d_D, &c->d_xown, &c->d_bound, &c->d_iters, &c->d_partial,
+                      &c->d_ws, &c->d_tc_exchange, &c->d_ws64, &c->d_maps, &c->d_map_off, &c->d_pairs, &c->d_D, &c->d_xown, &c->d_bound, &c->d_iters, &c->d_partial,
                       &c->d_work_n3,
                       &c->d_params, &c->d_mst, &c->d_vst, &c->d_partial_mlp, &c->d_feat, &c->d_pred, &c->d_labels,
                       &c->d_gersh, &c->d_prev_ratio, &c->d_sq_ratio, &c->d_tridiag, &c->d_loss, &c->d_sx, &c->d_st,

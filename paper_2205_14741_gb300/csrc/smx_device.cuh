@@ -134,6 +134,35 @@ __device__ __forceinline__ void fence_proxy_async_global() {
     asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// The CTA's place in its cluster, and the cluster's size (1 without a cluster launch).
+__device__ __forceinline__ int cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return static_cast<int>(r);
+}
+__device__ __forceinline__ int cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return static_cast<int>(r);
+}
+
+// The end of a phase: what the cluster's threads wrote to global memory is seen by the others' loads
+// (which bypass L1: __ldcg) after it.  The cluster's barrier does not wait for threads that have exited,
+// so a CTA that gave up after a timeout holds no other one back.
+__device__ __forceinline__ void phase_sync() {
+    if (cluster_size() == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+    }
+}
+// The same where bulk copies read it.
+__device__ __forceinline__ void phase_sync_copies() {
+    fence_proxy_async_global();
+    phase_sync();
+    if (cluster_size() > 1) fence_proxy_async_global();
+}
+
 // Orders this thread's generic-proxy shared-memory writes before later
 // async-proxy reads of them (tensor-core operands, bulk copies) issued after a
 // barrier.

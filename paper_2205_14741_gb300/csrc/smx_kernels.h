@@ -166,6 +166,10 @@ struct NonorthSetupArgs {
 cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, int max_n, const int* room, cudaStream_t st);
 
 // a5 (tcgen05 tensor cores) + a7.
+// CTAs that share a submatrix in the streamed form; what a cluster exchanges in global memory: the
+// residual's parts (8 warps of each CTA), a maximum of each CTA, the claimed job.
+constexpr int kTcCluster = 4;
+constexpr int kTcExchange = 64, kTcExchangeMax = 48, kTcExchangeJob = 56;
 struct NsTcArgs {
     const SubDesc* subs;
     const int32_t* order;  // processing order (largest first)
@@ -176,6 +180,7 @@ struct NsTcArgs {
     void* ws;              // 16-bit workspace: n_slots * 6 buffers of ld x ld
     int ld;                // multiple of 64, >= every padded n_j
     int n_slots;           // persistent CTAs (one per SM)
+    float* exchange;       // kTcExchange floats per slot
     float tau;
     // single-pass forms: also stop after a step whose residual lies below this level but is
     // more than half the previous one (the rounding floor; 0 = off)
@@ -203,7 +208,9 @@ struct NsTcArgs {
     const int* skip = nullptr;  // when set and non-zero at launch, the kernel does nothing
 };
 // precision: 1 = FP16 split hi/lo (3 products), 2 = FP16, 3 = BF16 (values of smx_precision)
-cudaError_t launch_ns_tc(const NsTcArgs& a, int precision, const CUtensorMap& tmap, int max_nblk, cudaStream_t st);
+// min_n: no submatrix has fewer rows; room: how many clusters of kTcCluster CTAs the device holds at once (ns_tc_clusters).
+cudaError_t launch_ns_tc(const NsTcArgs& a, int precision, const CUtensorMap& tmap, int min_n, int room, cudaStream_t st);
+cudaError_t ns_tc_clusters(int precision, int* room);
 
 // a7 + a8 for the tensor-core path: D[R_j, j] = 1/2 (E_j - X[:, own]) from the
 // saved owner columns, with the per-column trace (FP64) and energy (FP32 terms

@@ -124,35 +124,6 @@ __device__ __forceinline__ int acc_steps(uint32_t v) {
     return 4 * (__float_as_int(t) - 0x4C400000) + acc_small(__float_as_uint(__fsub_rn(x, __fsub_rn(t, 50331648.0f))));
 }
 
-// The CTA's place in its cluster, and the cluster's size (1 without a cluster launch).
-__device__ __forceinline__ int cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return static_cast<int>(r);
-}
-__device__ __forceinline__ int cluster_size() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return static_cast<int>(r);
-}
-
-// The end of a phase: what the cluster's threads wrote to global memory is seen by the others' loads
-// (which bypass L1: __ldcg) after it.  The cluster's barrier does not wait for threads that have exited,
-// so a CTA that gave up after a timeout holds no other one back.
-__device__ __forceinline__ void phase_sync() {
-    if (cluster_size() == 1) {
-        __syncthreads();
-    } else {
-        asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
-    }
-}
-// The same where bulk copies read it.
-__device__ __forceinline__ void phase_sync_copies() {
-    fence_proxy_async_global();
-    phase_sync();
-    if (cluster_size() > 1) fence_proxy_async_global();
-}
-
 // Entries (r, c .. c + 7) of a matrix with k rows (c even).
 __device__ __forceinline__ int64_t mat_at(int k, int r, int c) {
     return ((static_cast<int64_t>(c >> 1) * k + r) << 1) + (c & 1);
