@@ -172,6 +172,10 @@ __global__ void __launch_bounds__(8 * kFilterGroups) k_filter(const double* __re
     sc->filter_done = 0u;
 }
 
+// Dynamic shared memory above which a launch opts in: 48 KB hold a kernel's static arrays too (a few KB here;
+// measured against 48 KB alone, 19 blocks of 6 x 6 in FP64 were refused).
+constexpr size_t kPlainSmem = 32u << 10;
+
 cudaError_t launch_filter_gershgorin(const double* H, const int64_t* col_ptr, const int32_t* row_idx, const int64_t* voff,
                                      const int32_t* bsize, int n_cols, int bmax, int max_col_blocks, double eps,
                                      uint8_t* keep, const uint8_t* keep_prev, float* H32, DevScalars* sc, cudaStream_t st) {
@@ -181,7 +185,7 @@ cudaError_t launch_filter_gershgorin(const double* H, const int64_t* col_ptr, co
     int groups = kFilterGroups;
     while (groups > 1 && sizeof(double) * static_cast<size_t>(2 * groups + 1) * bmax + meta > (48u << 10)) groups >>= 1;
     const size_t smem = sizeof(double) * static_cast<size_t>(2 * groups + 1) * bmax + meta;
-    if (smem > (48u << 10)) {
+    if (smem > kPlainSmem) {
         cudaError_t e = cudaFuncSetAttribute(k_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }
@@ -686,7 +690,7 @@ template <class R, int BS>
 static cudaError_t launch_staged(const SubDesc* subs, int n_subs, int max_nblk, int stage_elems, size_t smem,
                                  const PatternView& pv, const R* H, double mu, R* T, double* bound, const GatherExtras& ex,
                                  cudaStream_t st) {
-    if (smem > (48u << 10)) {
+    if (smem > kPlainSmem) {
         cudaError_t e = cudaFuncSetAttribute(k_gather_staged<R, BS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
         if (e != cudaSuccess) return e;
@@ -713,7 +717,7 @@ static cudaError_t launch_gather(const SubDesc* subs, int n_subs, int max_nblk, 
     // per-warp block tables, R_j, local starts and the local block of every column
     const size_t smem = static_cast<size_t>(8) * max_nblk * sizeof(int64_t) +
                         (static_cast<size_t>(2 * max_nblk + 1) + static_cast<size_t>(max_n)) * sizeof(int);
-    if (smem > (48u << 10)) {
+    if (smem > kPlainSmem) {
         cudaError_t e = cudaFuncSetAttribute(k_gather_bound<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }
@@ -892,7 +896,7 @@ cudaError_t launch_scatter_owner(const SubDesc* subs, int n_subs, int max_nblk, 
     }
     const size_t smem = sizeof(int64_t) * static_cast<size_t>(max_nblk) +
                         sizeof(int) * (static_cast<size_t>(max_nblk) + 1 + static_cast<size_t>(max_n));
-    if (smem > (48u << 10)) {
+    if (smem > kPlainSmem) {
         cudaError_t e = cudaFuncSetAttribute(k_scatter_owner<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
     }

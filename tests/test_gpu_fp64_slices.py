@@ -149,3 +149,22 @@ def test_clusters_change_no_bit(m, b, f):
             c.set_column_range(j0, j1)
             c.build_density()
             assert np.array_equal(c.get_density().reshape(m, -1)[j0:j1], full[j0:j1]), (j0, j1)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp16x3"])
+def test_staged_gather_around_48_kb(precision):
+    # row stages just below and above 48 KB of dynamic shared memory, beside the kernel's static arrays
+    from paper_2205_14741_gb300 import SubmatrixDensity
+
+    for blocks in list(range(15, 24)) + [30, 34, 38, 42]:
+        s = make_mixed_block_system([6] * blocks, r_c=np.inf, ell=1.5, seed=blocks)
+        h = O.to_dense(s.block_size, s.col_ptr, s.row_idx, s.values)
+        lam, v = np.linalg.eigh(h)
+        k = int(np.argmax(np.diff(lam)))  # mu in the middle of the widest gap
+        with SubmatrixDensity.from_system(s) as c:
+            c.set_precision(precision)
+            c.set_mu(0.5 * float(lam[k] + lam[k + 1]))
+            c.build_density()
+            got = O.to_dense(s.block_size, s.col_ptr, s.row_idx, c.get_density())
+        tol = 1e-10 if precision == "fp64" else 1e-5  # the parity bounds of the two forms
+        assert float(np.max(np.abs(got - v[:, :k + 1] @ v[:, :k + 1].T))) <= tol, blocks
