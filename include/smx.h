@@ -169,9 +169,10 @@ smx_status smx_set_filter_threshold(smx_ctx* ctx, double eps);
 /* Upper bound (bytes, >= 1 MiB) on the device staging of the gathered
  * submatrices T_j - mu I (counted as FP64).  Block columns are processed in
  * consecutive chunks whose staging fits; one chunk when everything fits.
- * Default (no call): automatic, a tenth of the device memory for each FP64
- * staging buffer of the plain form (which keeps up to five of that size) and
- * half of it for the FP32 staging of the tensor-core forms (which keep one).
+ * Default (no call): automatic, a tenth of the device memory for the FP64
+ * staging of the plain form (whose work slots take up to twice that, four times
+ * for the function and non-orthogonal forms) and half of it for the FP32
+ * staging of the tensor-core forms (which keep one).
  * Results do not depend on the chunking.  Errors: SMX_ERR_ARG. */
 smx_status smx_set_staging_limit(smx_ctx* ctx, uint64_t bytes);
 
@@ -428,7 +429,7 @@ smx_status smx_get_submatrix_info(smx_ctx* ctx, int32_t* dims, int32_t* iters, d
  * device).
  * Computes D = 1/2 (I - sign(H - mu I)) of one dense symmetric H by FP64
  * Newton-Schulz iteration (Eq. 13 and Eq. 14 with S = I on a single dense
- * matrix; one CTA; the same iteration as the FP64 form of smx_build_density).
+ * matrix; one cluster of up to eight CTAs; the same iteration as the FP64 form of smx_build_density).
  *  h_dev       : device double[n*n], row-major, symmetric (read only).
  *  n           : 1 <= n <= 256; larger n returns SMX_ERR_ARG.
  *  mu          : finite chemical potential.

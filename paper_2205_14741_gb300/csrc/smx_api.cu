@@ -311,10 +311,12 @@ static smx_status analyse(smx_ctx* c) {
 // Bytes per staged element: FP64 for the plain form, FP32 for the tensor-core forms.
 static size_t staging_elem(const smx_ctx* c) { return c->precision == SMX_FP64 ? sizeof(double) : sizeof(float); }
 
+static size_t device_memory(const smx_ctx* c) { return c->mem_total ? c->mem_total : (size_t(24) << 30) * 4; }
+
 // Elements of staging per chunk.  An explicit limit counts bytes as FP64 elements.  The
-// automatic one takes a tenth of the device memory for each FP64 staging buffer (the plain form
-// keeps up to five of that size) and half of it for the FP32 staging of the tensor-core forms,
-// which keep one; it follows the precision (the chunks are laid out again when it changes).
+// automatic one takes a tenth of the device memory for the FP64 staging (the slots of the plain
+// form take up to two or four times as much: prepare_fp64_slots) and half of it for the FP32 staging
+// of the tensor-core forms; it follows the precision (the chunks are laid out again when it changes).
 static int64_t staging_chunk_elems(smx_ctx* c) {
     if (c->staging_limit) {
         c->chunk_elem = 0;
@@ -322,7 +324,7 @@ static int64_t staging_chunk_elems(smx_ctx* c) {
     }
     const size_t elem = staging_elem(c);
     c->chunk_elem = elem;
-    const size_t mem = c->mem_total ? c->mem_total : (size_t(24) << 30) * 4;
+    const size_t mem = device_memory(c);
     return static_cast<int64_t>((elem == sizeof(double) ? mem / 10 : mem / 2) / elem);
 }
 
@@ -526,11 +528,15 @@ static smx_status gather_chunk(smx_ctx* c, int j0, int m, double mu, const Gathe
 
 static smx_status read_status(smx_ctx* c);
 
-// Slots of the 64-bit kernels for m submatrices: one per persistent CTA (at most one per SM).
+// Slots of the 64-bit kernels for m submatrices: one per persistent CTA or cluster, at most one per SM, and
+// together at most two staging buffers (the density matrix) or four (the other forms) large.
 static smx_status prepare_fp64_slots(smx_ctx* c, int m, int mats, int planes, int* slots, size_t* slot_bytes) {
     if (!c->clusters[0]) SMX_CUDA(device_clusters(c->clusters));
     *slots = std::max(1, std::min(c->num_sms, m));
     *slot_bytes = fp64_slot_bytes(c->max_n, mats, planes);
+    const size_t staging = c->staging_limit ? c->staging_limit : device_memory(c) / 10;
+    const size_t fit = (mats == 2 && planes == 2 ? 2 : 4) * staging / *slot_bytes;
+    if (fit < static_cast<size_t>(*slots)) *slots = std::max<int>(1, static_cast<int>(fit));
     return ensure(c->d_ws64, *slot_bytes * static_cast<size_t>(*slots));
 }
 
