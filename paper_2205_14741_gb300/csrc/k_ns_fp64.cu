@@ -118,6 +118,30 @@ __device__ __noinline__ bool pass_source(const double* __restrict__ src, int ld,
     return bad;
 }
 
+// The mean of an n x n matrix X and its transpose into M and the planes: a bulk phase's last iterate, which is
+// symmetric up to that phase's rounding only (about 1e-7), while the products here take their factors
+// for symmetric.
+__device__ __noinline__ bool pass_iterate(const double* __restrict__ src, int ld, int64_t* M, uint8_t* planes, int n, int k) {
+    bool bad = false;
+    slice_pass<2>(k, k, planes,
+                  [&](int r, int c, int64_t (&v)[2][8]) {
+                      load_bits(src, ld, n, r, c, v[0]);
+#pragma unroll
+                      for (int i = 0; i < 8; ++i)
+                          v[1][i] = r < n && c + i < n ? __double_as_longlong(src[static_cast<int64_t>(r) * ld + c + i]) : 0;
+                  },
+                  [&](int r, int c, const int64_t (&v)[2][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i) {
+                          const int64_t x = to_fixed(__longlong_as_double(v[0][i]), 0, 0, bad);
+                          const int64_t y = to_fixed(__longlong_as_double(v[1][i]), 0, 0, bad);
+                          q[i] = (x >> 1) + (y >> 1);
+                      }
+                      st8(M, k, r, c, q);
+                  });
+    return bad;
+}
+
 // W = I - f S 2^up (f = 0: 1) to its digits; returns this thread's share of ||I - S 2^up||_F^2 in units of 2^-76.
 __device__ __noinline__ float pass_residual(const int64_t* S, uint8_t* planes, int n, int k, int up, uint64_t f) {
     float r2 = 0.0f;
@@ -212,10 +236,10 @@ __device__ __noinline__ void pass_transposed(const int64_t* A, const int64_t* B,
 
 // The symmetric source matrix A = src - mu I (n x n, leading dimension ld) in fixed point, A 2^-e, into M and
 // the planes P.  The power of two brings the largest 2-norm of a row into (1/2, 1] (so that the
-// products are exact and use all digits); without_scale keeps e = 0.  bound: no entry is larger (0:
+// products are exact and use all digits); iterate: src is a bulk phase's iterate, made symmetric, e = 0.  bound: no entry is larger (0:
 // not known).  Returns e; a value that is not finite sets ss->bad.
 __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, double mu, double bound, const SliceJob& jb, int64_t* M, uint8_t* P,
-                          bool without_scale, SliceShared* sh, SliceScalars* ss) {
+                          bool iterate, SliceShared* sh, SliceScalars* ss) {
     const int n = jb.n, k = jb.k, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto entry = [&](int r, int c) -> double {
         const double v = src[static_cast<int64_t>(r) * ld + c];
@@ -224,7 +248,7 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
     const int ranks = cluster_size(), rank = cluster_rank();
     int e = 0;
     if (threadIdx.x == 0) ss->bad = 0;
-    if (!without_scale) {
+    if (!iterate) {
         uint32_t top = static_cast<uint32_t>(__double2hiint(bound)) & 0x7fffffffu;
         if (top == 0) {  // high words order like the magnitudes
             for (int r = warp + rank * kSliceWarps; r < n; r += ranks * kSliceWarps)
@@ -265,7 +289,8 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
         e = e0 + (worst > 0.0f ? static_cast<int>(ceilf(0.5f * log2f(worst * 1.001f))) : 0);
     }
     __syncthreads();
-    const bool bad = cluster_sum(pass_source(src, ld, mu, e, 0, M, P, n, k) ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f;
+    const bool own_bad = iterate ? pass_iterate(src, ld, M, P, n, k) : pass_source(src, ld, mu, e, 0, M, P, n, k);
+    const bool bad = cluster_sum(own_bad ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f;
     if (bad) ss->bad = 1;
     __syncthreads();
     return e;

@@ -168,3 +168,18 @@ def test_staged_gather_around_48_kb(precision):
             got = O.to_dense(s.block_size, s.col_ptr, s.row_idx, c.get_density())
         tol = 1e-10 if precision == "fp64" else 1e-5  # the parity bounds of the two forms
         assert float(np.max(np.abs(got - v[:, :k + 1] @ v[:, :k + 1].T))) <= tol, blocks
+
+
+@pytest.mark.parametrize("n", [64, 160, 192])
+def test_finishing_steps_start_from_a_symmetric_iterate(n):
+    # every submatrix of a full pattern has the same iterate, so D's asymmetry is that iterate's; the bulk phase's
+    # is about 1e-7, and what the mean with the transpose leaves is the rounding of the last product
+    from paper_2205_14741_gb300 import SubmatrixDensity
+
+    s = make_mixed_block_system([1] * n, r_c=np.inf, ell=1.5, seed=6)
+    with SubmatrixDensity.from_system(s) as c:
+        c.set_precision("fp16x3", 1)
+        c.set_mu(0.02)
+        c.build_density()
+        d = O.to_dense(s.block_size, s.col_ptr, s.row_idx, c.get_density())
+    assert float(np.max(np.abs(d - d.T))) <= 1e-14
