@@ -399,7 +399,7 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
             best = pass == 0 ? q : fmin(best, q);
         }
     }
-    __syncthreads();
+    phase_sync();              // `exchange` is the caller's again: no CTA of the cluster still reads it
     fence_proxy_async_smem();  // the stages are the copies' again
 }
 

@@ -1,0 +1,40 @@
+"""What orders the accesses of a cluster's CTAs, and of a CTA's roles, in the 64-bit kernels, read from the source.
+
+A missing barrier shows in a run only when one CTA falls behind another in a window of a few hundred cycles, so
+these tests check that the ordering statement is where the shared memory is reused.
+"""
+
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2205_14741_gb300", "csrc")
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())  # without comments
+
+
+def body(text, name):
+    """The text of the function `name`, from its opening brace to the matching one."""
+    for m in re.finditer(r"\b%s\(" % name, text):
+        i, depth = m.end(), 1
+        while depth:  # past the parameters
+            depth += {"(": 1, ")": -1}.get(text[i], 0)
+            i += 1
+        if text[i:].lstrip().startswith("{"):
+            start = i = text.index("{", i)
+            while True:
+                depth += {"{": 1, "}": -1}.get(text[i], 0)
+                i += 1
+                if not depth:
+                    return text[start:i]
+    raise AssertionError(f"no function {name}")
+
+
+def test_bound_exchange_is_read_before_its_memory_is_reused():
+    # the exchanged row sums lie where the caller's next pass writes digits: every CTA's last read of them comes
+    # before a barrier of the cluster
+    b = body(source("k_ns_fp64.cu"), "first_bound")
+    last = b.rindex("share(")
+    assert "phase_sync()" in b[last:]
