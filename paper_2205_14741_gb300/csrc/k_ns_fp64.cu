@@ -493,11 +493,13 @@ __device__ int sign_steps(SliceShared* sh, const SliceJob& jb, int e, int max_it
     return done;
 }
 
-// Largest 2-norm of a column of M, squared.
+// Largest 2-norm of a column of M, squared.  The CTAs of a cluster take the columns in turn; the barrier of
+// their maximum also orders every read of M before what follows (the callers change M in place).
 __device__ __noinline__ float column_norm2(const SliceJob& jb, const int64_t* M, SliceShared* sh) {
     const int n = jb.n, k = jb.k, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ranks = cluster_size(), rank = cluster_rank();
     float worst = 0.0f;
-    for (int c = 2 * warp; c < n; c += 2 * kSliceWarps) {
+    for (int c = 2 * (warp + rank * kSliceWarps); c < n; c += 2 * ranks * kSliceWarps) {
         const longlong2* m = reinterpret_cast<const longlong2*>(M) + static_cast<int64_t>(c >> 1) * k;
         float a0 = 0.0f, a1 = 0.0f;
 #pragma unroll 4
@@ -514,7 +516,8 @@ __device__ __noinline__ float column_norm2(const SliceJob& jb, const int64_t* M,
         }
         worst = fmaxf(worst, fmaxf(a0, a1));
     }
-    return cta_max(worst, sh) * 0x1p-60f;
+    worst = cta_max(worst, sh);
+    return __uint_as_float(cluster_max(__float_as_uint(worst), reinterpret_cast<uint32_t*>(jb.scratch) + 32)) * 0x1p-60f;
 }
 
 // The sign iteration of the Eq. 12 block matrix [[0, A], [I, 0]] written per block (the coupled

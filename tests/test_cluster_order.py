@@ -38,3 +38,11 @@ def test_bound_exchange_is_read_before_its_memory_is_reused():
     b = body(source("k_ns_fp64.cu"), "first_bound")
     last = b.rindex("share(")
     assert "phase_sync()" in b[last:]
+
+
+def test_column_norms_are_read_before_the_matrix_changes():
+    # the coupled iteration halves Z in place after its column norms: the norms end in a barrier of the cluster
+    text = source("k_ns_fp64.cu")
+    assert "cluster_max(" in body(text, "column_norm2") and "phase_sync()" in body(source("smx_slices.cuh"), "cluster_max")
+    b = body(text, "coupled_steps")
+    assert b.index("column_norm2(") < b.index("pass_affine(Z, shift ? Z")
