@@ -716,14 +716,17 @@ __device__ double2 gershgorin_interval(const double* M, int n, int ld, double* s
 // The next submatrix of the CTA or cluster (largest first; every thread gets its place in the order): its
 // own place first, then whichever is next when it is free.  (Claimed one ahead, 256 submatrices on 152
 // SMs took 8 % longer: some SMs held two of the largest.)  Meanwhile the source of the submatrix that
-// the launch is likely to reach next comes into L2.
-__device__ __forceinline__ int claim_job(int* counter, SliceScalars* ss, SubDesc* cur, int* shared_job, bool first, int n_subs,
+// the launch is likely to reach next comes into L2.  shared_jobs: two words of the cluster, taken in turn: a
+// submatrix may pass without a barrier of the cluster (one that is not finite), and then a CTA may still
+// have to read its word when the first CTA writes the next one.
+__device__ __forceinline__ int claim_job(int* counter, SliceScalars* ss, SubDesc* cur, int* shared_jobs, int round, int n_subs,
                                          const int32_t* order, const SubDesc* subs, const double* src) {
     __syncthreads();
     const int ranks = cluster_size(), clusters = gridDim.x / ranks;
     const bool leader = cluster_rank() == 0;
+    int* const shared_job = shared_jobs + (round & 1);
     if (threadIdx.x == 0 && leader) {
-        const int job = first ? blockIdx.x / ranks : clusters + atomicAdd(counter, 1);
+        const int job = round == 0 ? blockIdx.x / ranks : clusters + atomicAdd(counter, 1);
         if (ranks > 1) __stcg(shared_job, job);
         ss->job = job;
         if (job + clusters < n_subs) {
@@ -745,9 +748,10 @@ __device__ __forceinline__ int claim_job(int* counter, SliceScalars* ss, SubDesc
 
 // The last cluster to run out of work resets the job counter for the next launch.
 // A leader that gave up leaves its cluster no job to find.
-__device__ __forceinline__ void release_jobs(int* counter, unsigned int* ticket, int* shared_job) {
+__device__ __forceinline__ void release_jobs(int* counter, unsigned int* ticket, int* shared_jobs) {
     if (threadIdx.x == 0 && cluster_rank() == 0) {
-        __stcg(shared_job, INT_MAX);
+        __stcg(shared_jobs, INT_MAX);
+        __stcg(shared_jobs + 1, INT_MAX);
         __threadfence();
         if (atomicAdd(ticket, 1u) == gridDim.x / cluster_size() - 1) {
             *counter = 0;
@@ -781,8 +785,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
     slices_begin(sh, slice_stages(), a.status);
     uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x / cluster_size()) * a.slot_bytes;
     const bool lead = cluster_rank() == 0;  // writes the results
-    for (bool first = true;; first = false) {
-        const int job = claim_job(a.work_counter, &ss, &s, reinterpret_cast<int*>(slot + 64), first, a.n_subs, a.order, a.subs, a.Mc ? a.Mc : a.T);
+    for (int round = 0;; ++round) {
+        const int job = claim_job(a.work_counter, &ss, &s, reinterpret_cast<int*>(slot + 64), round, a.n_subs, a.order, a.subs, a.Mc ? a.Mc : a.T);
         if (job >= a.n_subs || sh->abort) break;
         const int j = s.col;
         if (threadIdx.x == 0) {
@@ -928,8 +932,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid
     SliceShared* const sh = &shared;
     slices_begin(sh, slice_stages(), a.status);
     uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x / cluster_size()) * a.slot_bytes;
-    for (bool first = true;; first = false) {
-        const int job = claim_job(a.work_counter, &ss, &s, reinterpret_cast<int*>(slot + 64), first, a.n_subs, a.order, a.subs, a.Lc);
+    for (int round = 0;; ++round) {
+        const int job = claim_job(a.work_counter, &ss, &s, reinterpret_cast<int*>(slot + 64), round, a.n_subs, a.order, a.subs, a.Lc);
         if (job >= a.n_subs || sh->abort) break;
         if (threadIdx.x == 0) {
             slice_job(jb, slot + kSlotHead, s.n, a.kmax, a.mats);

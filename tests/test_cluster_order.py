@@ -46,3 +46,11 @@ def test_column_norms_are_read_before_the_matrix_changes():
     assert "cluster_max(" in body(text, "column_norm2") and "phase_sync()" in body(source("smx_slices.cuh"), "cluster_max")
     b = body(text, "coupled_steps")
     assert b.index("column_norm2(") < b.index("pass_affine(Z, shift ? Z")
+
+
+def test_a_claimed_job_is_read_before_its_word_is_written_again():
+    # between two claims there may be no barrier of the cluster: two words in turn, so that the write of one is
+    # ordered after its last read by the claim between them
+    b = body(source("k_ns_fp64.cu"), "claim_job")
+    word = re.search(r"(\w+) \+ \(round & 1\)", b)
+    assert word and b.index(word.group(0)) < b.index("__stcg(") < b.index("phase_sync()") < b.index("__ldcg(")
