@@ -65,6 +65,7 @@ struct SliceShared {
     int* status;
     uint32_t tmem;
     int abort;
+    int gave_up[2];  // abort as the readers of an accumulation all see it (by its number modulo 2)
     int kpart;       // chunks of one exact accumulation (fewer than kSliceK / 16 where an operand's rows are longer)
     int tile;        // columns of a tile: kSliceTile, or half of it to have tiles for all CTAs of a larger cluster
     int weights;     // 7: the pairs of weights 2 .. 8; 8: of weight 9 too (kpart at most 10)
@@ -327,14 +328,16 @@ __device__ __noinline__ void slice_product(SliceShared* sh, const uint8_t* __res
                 int64_t sum[kTurns][4];
                 for (int p = 0; p < parts; ++p) {
                     // one lane polls; the other warps wait at a barrier without touching shared memory, whose
-                    // bandwidth the products need
-                    if (warp == 2 && lane == 0) mbar_wait(&sh->tfull, use & 1, ab, status);
-                    asm volatile("bar.sync 1, 448;" ::: "memory");
-                    ++use;
-                    if (*ab) {
-                        alive = false;
-                        break;
+                    // bandwidth the products need.  That lane's one look at the abort flag decides for all: each
+                    // looking for itself, a flag raised in between would leave some of them at this barrier for good.
+                    if (warp == 2 && lane == 0) {
+                        mbar_wait(&sh->tfull, use & 1, ab, status);
+                        sh->gave_up[use & 1] = *ab;
                     }
+                    asm volatile("bar.sync 1, 448;" ::: "memory");
+                    alive = !sh->gave_up[use & 1];
+                    ++use;
+                    if (!alive) break;
                     tc_fence_after();
 #pragma unroll
                     for (int h = 0; h < kTurns; ++h) {

@@ -54,3 +54,13 @@ def test_a_claimed_job_is_read_before_its_word_is_written_again():
     b = body(source("k_ns_fp64.cu"), "claim_job")
     word = re.search(r"(\w+) \+ \(round & 1\)", b)
     assert word and b.index(word.group(0)) < b.index("__stcg(") < b.index("phase_sync()") < b.index("__ldcg(")
+
+
+def test_readers_of_an_accumulation_give_up_together():
+    # the 14 reading warps meet at barrier 1 once per accumulation: one decision, published before the barrier
+    b = body(source("smx_slices.cuh"), "slice_product")
+    readers = b[b.index("bar.sync 1, 448") - 300:]
+    assert readers.index("sh->gave_up[use & 1] = *ab") < readers.index("bar.sync 1, 448")
+    after = readers[readers.index("bar.sync 1, 448"):]
+    assert after.index("alive = !sh->gave_up[use & 1]") < after.index("++use")
+    assert "*ab" not in after  # no warp looks at the flag for itself
