@@ -310,13 +310,21 @@ struct SignBound {
 
 // For the symmetric non-negative-bounded Y = S: the largest row sum of |Y| (every thread), and the smaller
 // max_r (|Y| w)_r / w_r of two power steps from the row sums (thread 0; 0 without any).  The CTAs of a
-// cluster take 32 rows each in turn and exchange the sums at `exchange` (3 k values).
+// cluster take 32 rows each in turn and exchange the sums at `exchange`.  Memory there: 3 k values for that, and past
+// kBoundSharedRows rows two vectors of k values for each CTA, which lie in the stage area below.
+// (Held there for any k, they ran past its end from k = 13,472 on.)
+constexpr int kBoundSharedRows = 2048;
+static_assert(2 * 8 * kBoundSharedRows <= kSliceStages * kSliceStageBytes, "the two vectors fit the stage area");
+static_assert((3 + 2 * 8) * 8 * kBoundSharedRows <= slice_bytes(kBoundSharedRows), "a matrix's planes hold the vectors of eight CTAs");
 __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceShared* sh, SliceScalars* ss, unsigned long long* exchange,
                                          double& row_max, double& best) {
     const int ranks = cluster_size(), rank = cluster_rank();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    unsigned long long* wv = reinterpret_cast<unsigned long long*>(sh->smem);  // row sums, then weights
+    unsigned long long* wv = k <= kBoundSharedRows ? reinterpret_cast<unsigned long long*>(sh->smem)
+                                                   : exchange + static_cast<int64_t>(3 + 2 * rank) * k;  // row sums, then weights
     unsigned long long* av = wv + k;
+    // entries are at most 1 (2^62): the sums of k of them, below in units of up to 2^-51, stay below 2^64
+    const int cut = k <= 4096 ? 12 : 16;
     // v complete in every CTA of the cluster; the maximum (m: of the CTA's own rows)
     auto share = [&](unsigned long long* v, unsigned long long m) {
         if (ranks > 1) {
@@ -333,7 +341,7 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
         }
         return cta_max_u64(m, ss);
     };
-    // row sums of |Y| in units of 2^-50
+    // row sums of |Y| in units of 2^(cut - 62)
     unsigned long long m = 0;
     for (int r = 2 * (warp + rank * kSliceWarps); r < n; r += 2 * ranks * kSliceWarps) {  // Y is symmetric: two columns at a time
         const longlong2* y = reinterpret_cast<const longlong2*>(S) + static_cast<int64_t>(r >> 1) * k;
@@ -341,8 +349,8 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
 #pragma unroll 4
         for (int c = lane; c < k; c += 32) {
             const longlong2 v = __ldcg(y + c);
-            a0 += abs_fixed(v.x) >> 12;
-            a1 += abs_fixed(v.y) >> 12;
+            a0 += abs_fixed(v.x) >> cut;
+            a1 += abs_fixed(v.y) >> cut;
         }
         a0 = warp_sum_u64(a0);
         a1 = warp_sum_u64(a1);
@@ -353,7 +361,7 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
         m = max(m, max(a0, a1));
     }
     m = share(wv, m);
-    row_max = static_cast<double>(m) * 0x1p-50;
+    row_max = ldexp(static_cast<double>(m), cut - 62);
     best = 0.0;  // of the power steps (every row's quotient; 0: none)
     for (int pass = 0; pass < 2 && m > 0; ++pass) {
         // weights: any multiple of w serves; the largest into [2^62, 2^63), at least one unit
@@ -366,13 +374,13 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
         m = 0;
         for (int r = 2 * (warp + rank * kSliceWarps); r < n; r += 2 * ranks * kSliceWarps) {
             const longlong2* y = reinterpret_cast<const longlong2*>(S) + static_cast<int64_t>(r >> 1) * k;
-            unsigned long long a0 = 0, a1 = 0;  // (|Y| w)_r, w in units of 2^-63, in units of 2^-51
+            unsigned long long a0 = 0, a1 = 0;  // (|Y| w)_r, w in units of 2^-63, in units of 2^(cut - 63)
 #pragma unroll 4
             for (int c = lane; c < k; c += 32) {  // (zero past n)
                 const longlong2 v = __ldcg(y + c);
                 const unsigned long long w = wv[c] << 1;
-                a0 += __umul64hi(abs_fixed(v.x) << 1, w) >> 12;
-                a1 += __umul64hi(abs_fixed(v.y) << 1, w) >> 12;
+                a0 += __umul64hi(abs_fixed(v.x) << 1, w) >> cut;
+                a1 += __umul64hi(abs_fixed(v.y) << 1, w) >> cut;
             }
             a0 = warp_sum_u64(a0);
             a1 = warp_sum_u64(a1);
@@ -395,7 +403,7 @@ __device__ __noinline__ void first_bound(const int64_t* S, int n, int k, SliceSh
         if (tid == 0) {
             for (int w = 1; w < kSliceWarps; ++w)
                 if (ss->d[w] > q) q = ss->d[w];
-            q *= 0x1p12;
+            q = ldexp(q, cut);
             best = pass == 0 ? q : fmin(best, q);
         }
     }

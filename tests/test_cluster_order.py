@@ -64,3 +64,12 @@ def test_readers_of_an_accumulation_give_up_together():
     after = readers[readers.index("bar.sync 1, 448"):]
     assert after.index("alive = !sh->gave_up[use & 1]") < after.index("++use")
     assert "*ab" not in after  # no warp looks at the flag for itself
+
+
+def test_bound_vectors_leave_the_stage_area_before_it_ends():
+    # two vectors of 64-bit words per row in shared memory; past a size they lie in the slot
+    text, slices = source("k_ns_fp64.cu"), source("smx_slices.cuh")
+    rows = int(re.search(r"kBoundSharedRows = (\d+)", text).group(1))
+    planes, tile, stages = (int(re.search(r"%s = (\d+)" % c, slices).group(1)) for c in ("kSlicePlanes", "kSliceTile", "kSliceStages"))
+    assert 16 * rows <= stages * planes * 32 * (128 + tile)
+    assert "k <= kBoundSharedRows ?" in body(text, "first_bound")

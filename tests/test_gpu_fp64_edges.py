@@ -1,0 +1,42 @@
+"""The 64-bit forms where their fixed-point arithmetic, their memory or their claims end: sizes, magnitudes and
+submatrices that fail."""
+
+import numpy as np
+import pytest
+
+import oracle as O
+from synth import make_mixed_block_system
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+@pytest.mark.parametrize("columns", [3, 131])
+def test_fp64_past_the_rows_whose_bound_fits_shared_memory(columns):
+    # n = 2081: the vectors of the first bound lie in global memory; a submatrix to a cluster, and one to a CTA.
+    # D is known: a reflection I - 2 V V^T with 5 columns V, scaled by 1/2.
+    from paper_2205_14741_gb300 import SubmatrixDensity
+
+    s = make_mixed_block_system([16] * 130 + [1], r_c=np.inf, ell=1.5, seed=1)
+    v = np.linalg.qr(np.random.default_rng(2).standard_normal((s.n, 5)))[0]
+    h = 0.5 * np.eye(s.n) - v @ v.T
+    first = np.concatenate([[0], np.cumsum(s.block_size)])
+    vals = np.empty_like(s.values)
+    off = O.block_value_offsets(s.block_size, s.col_ptr, s.row_idx)
+    for j in range(131):
+        for k in range(s.col_ptr[j], s.col_ptr[j + 1]):
+            r = s.row_idx[k]
+            vals[off[k]:off[k + 1]] = h[first[r]:first[r + 1], first[j]:first[j + 1]].T.ravel()
+    with SubmatrixDensity.from_system(s) as c:
+        c.set_values(vals)
+        c.set_column_range(0, columns)
+        c.build_density()
+        got = O.to_dense(s.block_size, s.col_ptr, s.row_idx, c.get_density())[:, : first[columns]]
+    # a product's error is below 3.4e-17 sqrt(2081 / 158) per entry; 30 of them with factors of up to 2.5
+    assert float(np.max(np.abs(got - (v @ v.T)[:, : first[columns]]))) <= 30 * 2.5 * 3.4e-17 * np.sqrt(2081 / 158) + 2e-14
