@@ -208,6 +208,16 @@ __device__ __noinline__ void pass_affine(const int64_t* S, int64_t* out, uint8_t
                   });
 }
 
+// M <- 0.
+__device__ __noinline__ void pass_zero(int64_t* M, int k) {
+    slice_pass<1>(k, k, nullptr, [](int, int, int64_t (&)[1][8]) {},
+                  [&](int r, int c, const int64_t (&)[1][8], int64_t (&q)[8]) {
+#pragma unroll
+                      for (int i = 0; i < 8; ++i) q[i] = 0;
+                      st8(M, k, r, c, q);
+                  });
+}
+
 // T <- (a T + b S) 2^up (a = 0: 1), and its digits.
 __device__ __noinline__ void pass_mix(int64_t* T, const int64_t* S, uint8_t* planes, int k, uint64_t a, uint64_t b, int up) {
     slice_pass<2>(k, k, planes,
@@ -634,7 +644,10 @@ __device__ int fermi_tanh(SliceShared* sh, const SliceJob& jb, const double* __r
         bad = true;
         return 0;
     }
-    if (zero) return 0;  // T = 0
+    if (zero) {  // (the slot holds what the submatrix before left)
+        pass_zero(T, k);
+        return 0;
+    }
     int nprod = 0;
     // wide: with the digit pairs of weight 9 (an error in T may double at every doubling; the products of
     // K enter it with factors of 1/9 and less)

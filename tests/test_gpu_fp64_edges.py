@@ -40,3 +40,24 @@ def test_fp64_past_the_rows_whose_bound_fits_shared_memory(columns):
         got = O.to_dense(s.block_size, s.col_ptr, s.row_idx, c.get_density())[:, : first[columns]]
     # a product's error is below 3.4e-17 sqrt(2081 / 158) per entry; 30 of them with factors of up to 2.5
     assert float(np.max(np.abs(got - (v @ v.T)[:, : first[columns]]))) <= 30 * 2.5 * 3.4e-17 * np.sqrt(2081 / 158) + 2e-14
+
+
+@pytest.mark.parametrize("first", ["density", "fermi", "inv_sqrt"])
+@pytest.mark.parametrize("m", [9, 200])
+def test_fermi_at_infinite_temperature_after_another_build(m, first):
+    # F = I/2 whatever the work memory held before: an iterate of another function, or T at another temperature
+    from paper_2205_14741_gb300 import SubmatrixDensity
+
+    s = make_mixed_block_system([3] * m, r_c=6.0, ell=1.5, seed=8)
+    lam = np.linalg.eigvalsh(O.to_dense(s.block_size, s.col_ptr, s.row_idx, s.values))
+    with SubmatrixDensity.from_system(s) as c:
+        c.set_function(first)
+        c.set_fermi_beta(12.0)
+        c.set_mu(float(lam[0]) - 0.5 if first == "inv_sqrt" else 0.02)
+        c.build_density()
+        c.get_trace()
+        c.set_function("fermi")
+        c.set_fermi_beta(0.0)
+        c.build_density()
+        got = O.to_dense(s.block_size, s.col_ptr, s.row_idx, c.get_density())
+    assert np.array_equal(got, 0.5 * np.eye(s.n))
