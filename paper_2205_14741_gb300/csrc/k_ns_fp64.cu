@@ -35,6 +35,7 @@ struct SliceJob {
     int64_t* M[kFp64Mats];
     uint8_t* P[kFp64Planes];
     float* scratch;  // of the cluster (the first kSlotHead bytes of its slot): sums, maxima, the claimed job, maxima
+    unsigned long long* sums;  // of the cluster: three squared lengths per row (coupled_steps)
 };
 
 // Scalars that one thread forms in FP64 for the CTA.
@@ -56,8 +57,29 @@ __device__ __forceinline__ void slice_job(SliceJob& jb, uint8_t* slot, int n, in
     for (int i = 0; i < kFp64Mats; ++i) jb.M[i] = reinterpret_cast<int64_t*>(slot + i * mb);
     for (int i = 0; i < kFp64Planes; ++i) jb.P[i] = slot + mats * mb + i * slice_bytes(kmax);
 }
-// The first bytes of a slot serve the cluster (kSlotHead); slice_job gets what follows.
+// The first bytes of a slot serve the cluster (kSlotHead); slice_job gets what follows.  The last hold the rows'
+// squared lengths.
 constexpr int64_t kSlotHead = 256;
+constexpr int64_t sums_bytes(int64_t k) { return 3 * 8 * k; }
+
+// Adds the squared length of sixteen neighbouring entries of row r, half each of a lane pair (s: this lane's in units
+// of 2^-24, the squares of at most eight entries of magnitude 2), to the row's sum: in integers, so that
+// the sum is the same in every order.
+__device__ __forceinline__ void add_length(unsigned long long* sums, int r, float s) {
+    const unsigned int u = __float2uint_rn(s);
+    const unsigned int both = u + __shfl_xor_sync(0xffffffffu, u, 1);
+    if ((threadIdx.x & 1) == 0) atomicAdd(sums + r, static_cast<unsigned long long>(both));
+}
+// The squared length of eight fixed-point values in units of 2^-24 (their upper halves: units of 2^-30).
+__device__ __forceinline__ float length8(const int64_t (&q)[8]) {
+    float s = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float x = static_cast<float>(static_cast<int>(q[i] >> 32));
+        s = fmaf(x, x, s);
+    }
+    return s * 0x1p-36f;
+}
 
 __device__ __forceinline__ int64_t ld1(const int64_t* p) { return __ldcg(reinterpret_cast<const long long*>(p)); }
 
@@ -144,23 +166,32 @@ __device__ __noinline__ bool pass_iterate(const double* __restrict__ src, int ld
 }
 
 // W = I - f S 2^up (f = 0: 1) to its digits; returns this thread's share of ||I - S 2^up||_F^2 in units of 2^-76.
-__device__ __noinline__ float pass_residual(const int64_t* S, uint8_t* planes, int n, int k, int up, uint64_t f) {
+// sums (with f = 0): the rows' squared lengths are added to it, far too long where an entry of S 2^up is above 1 (by
+// more than rounding), of which the difference may not fit.
+__device__ __noinline__ float pass_residual(const int64_t* S, uint8_t* planes, int n, int k, int up, uint64_t f,
+                                            unsigned long long* sums = nullptr) {
     float r2 = 0.0f;
+    const uint32_t most = 0x40400000u >> up;  // 1 + 2^-8 in units of 2^-30 (2^-up)
     slice_pass<1>(k, k, planes, [&](int r, int c, int64_t (&v)[1][8]) { ld8(S, k, r, c, v[0]); },
                   [&](int r, int c, const int64_t (&v)[1][8], int64_t (&q)[8]) {
+                      float row = 0.0f;
+                      uint32_t top = 0;
 #pragma unroll
                       for (int i = 0; i < 8; ++i) {
                           const int64_t one = r == c + i && r < n ? kFixedOne : 0, s = v[0][i] << up;
                           const float d = fixed_float(one - s);
                           r2 = fmaf(d, d, r2);
+                          row = fmaf(d, d, row);
+                          top = max(top, static_cast<uint32_t>(abs_fixed(v[0][i]) >> 32));
                           q[i] = one - (f ? fixed_mul(s, f) : s);
                       }
+                      if (sums) add_length(sums, r, top > most ? 0x1p28f : fminf(row * 0x1p-52f, 0x1p28f));
                   });
     return r2;
 }
 
-// X <- f (X + 1/2 S) (f = 0: 1), and its digits.
-__device__ __noinline__ void pass_update(int64_t* X, const int64_t* S, uint8_t* planes, int k, uint64_t f) {
+// X <- f (X + 1/2 S) (f = 0: 1), and its digits; the rows' squared lengths are added to sums.
+__device__ __noinline__ void pass_update(int64_t* X, const int64_t* S, uint8_t* planes, int k, uint64_t f, unsigned long long* sums = nullptr) {
     slice_pass<2>(k, k, planes,
                   [&](int r, int c, int64_t (&v)[2][8]) {
                       ld8(X, k, r, c, v[0]);
@@ -173,11 +204,12 @@ __device__ __noinline__ void pass_update(int64_t* X, const int64_t* S, uint8_t* 
                           if (f) q[i] = fixed_mul(q[i], f);
                       }
                       st8(X, k, r, c, q);
+                      if (sums) add_length(sums, r, length8(q));
                   });
 }
 
-// Z <- 3/2 I - 1/2 (Y - 1/2 S)
-__device__ __noinline__ void pass_first_root(const int64_t* Y, const int64_t* S, int64_t* Z, int n, int k) {
+// Z <- 3/2 I - 1/2 (Y - 1/2 S); the rows' squared lengths are added to sums.
+__device__ __noinline__ void pass_first_root(const int64_t* Y, const int64_t* S, int64_t* Z, int n, int k, unsigned long long* sums) {
     slice_pass<2>(k, k, nullptr,
                   [&](int r, int c, int64_t (&v)[2][8]) {
                       ld8(Y, k, r, c, v[0]);
@@ -188,6 +220,7 @@ __device__ __noinline__ void pass_first_root(const int64_t* Y, const int64_t* S,
                       for (int i = 0; i < 8; ++i)
                           q[i] = (r == c + i && r < n ? kFixedOne + (kFixedOne >> 1) : 0) - ((v[0][i] - (v[1][i] >> 1)) >> 1);
                       st8(Z, k, r, c, q);
+                      add_length(sums, r, length8(q));
                   });
 }
 
@@ -545,12 +578,30 @@ __device__ __noinline__ float column_norm2(const SliceJob& jb, const int64_t* M,
 // largest eigenvalue.  Y ends in M[0] (digits P[0]), Z in M[1] (digits P[1]) in units of 2^(ez - 62); M[2]
 // takes the products, P[2] the digits of R.  Every matrix is a polynomial of A, so the products are
 // symmetric.  The first step needs one product (Z = I), the last only that of the wanted root.
-// Y and R have 2-norms of at most 1; Z's rows are kept below 1 by its exponent (a step multiplies its
-// 2-norm by at most 1.5).  ||R||_F^2 > 1.5 n or a vanishing Z means that A is not positive definite.
+//
+// Positive definiteness.  For a positive definite A the eigenvalues of Y and R lie in [0, 1], so no row of them is
+// longer than 1 and no entry of Z Y is larger, and a step lengthens no row of Z by more than 3/2 (Z's are kept
+// below 1 by its exponent).  The integers would wrap where floating point overflows, and the iteration could then
+// converge to a root of another matrix.  So the passes add up the rows' squared lengths, and a matrix whose
+// rows are too long enters no product: with rows of at most 1 in both factors no entry of a product leaves
+// the integers' range, nor does X + 1/2 X R, and nothing wraps before it is seen.  A negative eigenvalue -t of Z Y
+// grows from step to step (t (3 + t)^2 / 4 > 2.25 t) until the rows of R, which hold its 1 + t, are too long.
 __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* __restrict__ src, int ld, double b, int max_iter, float tau,
                              bool want_y, bool want_z, int& ez, SliceScalars* ss, bool& conv, bool& bad) {
     const int n = jb.n, k = jb.k;
     int64_t *Y = jb.M[0], *Z = jb.M[1], *S = jb.M[2];
+    unsigned long long *row_r = jb.sums, *row_y = row_r + k, *row_z = row_y + k;  // squared lengths in units of 2^-24
+    // (cleared one phase or more after every CTA of the cluster has read them, and before they are added to)
+    auto clear = [&](unsigned long long* sums, int count) {
+        for (int r = cluster_rank() * kSliceThreads + threadIdx.x; r < count; r += cluster_size() * kSliceThreads) __stcg(sums + r, 0ull);
+    };
+    auto longest = [&](const unsigned long long* sums) {
+        unsigned long long m = 0;
+        for (int r = threadIdx.x; r < n; r += kSliceThreads) m = max(m, __ldcg(sums + r));
+        return static_cast<float>(cta_max_u64(m, ss)) * 0x1p-24f;
+    };
+    constexpr float kLongest = 1.002f;  // of a length squared that is at most 1 (its squares are rounded)
+    clear(row_r, 3 * k);
     conv = bad = false;
     ez = 0;
     int done = 0;
@@ -570,10 +621,11 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
             slice_product(sh, jb.P[1], jb.P[0], k, k, S, true);  // Z Y
             if (*static_cast<volatile int*>(&sh->abort)) break;
         }
-        float r2 = pass_residual(it > 0 ? S : Y, jb.P[2], n, k, ez, 0);
+        clear(row_y, 2 * k);
+        float r2 = pass_residual(it > 0 ? S : Y, jb.P[2], n, k, ez, 0, row_r);
         r2 = cluster_sum(r2 * 0x1p-76f, sh, jb.scratch);
         done = it + 1;
-        if (!isfinite(r2) || r2 > 1.5f * static_cast<float>(n) || ez > 40) {
+        if (longest(row_r) > kLongest) {
             bad = true;
             break;
         }
@@ -581,7 +633,8 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
         if (!conv || want_y) {
             slice_product(sh, jb.P[0], jb.P[2], k, k, S, true);  // Y R
             if (*static_cast<volatile int*>(&sh->abort)) break;
-            pass_update(Y, S, jb.P[0], k, 0);
+            clear(row_r, k);
+            pass_update(Y, S, jb.P[0], k, 0, row_y);
         }
         if (!conv || want_z) {
             if (it > 0) {
@@ -589,10 +642,16 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
                 if (*static_cast<volatile int*>(&sh->abort)) break;
             }
             // Z' = Z + 1/2 R Z; from Z = I: I + 1/2 R = 3/2 I - 1/2 Y0, where Y now holds Y0 + 1/2 Y0 R and S = Y0 R
-            if (it > 0) pass_update(Z, S, nullptr, k, 0);
-            else pass_first_root(Y, S, Z, n, k);
-            const int shift = column_norm2(jb, Z, sh) > 1.0f ? 1 : 0;
+            if (it > 0) pass_update(Z, S, nullptr, k, 0, row_z);
+            else pass_first_root(Y, S, Z, n, k, row_z);
+            const float z = longest(row_z);
+            const int shift = z > 1.0f ? 1 : 0;
             ez += shift;
+            if (z > 2.25f * kLongest || longest(row_y) > kLongest || ez > 30) {
+                bad = true;
+                conv = false;
+                break;
+            }
             pass_affine(Z, shift ? Z : nullptr, jb.P[1], n, k, 0, false, -shift, 0);
         }
         if (conv) break;
@@ -813,6 +872,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
         if (threadIdx.x == 0) {
             slice_job(jb, slot + kSlotHead, s.n, a.kmax, a.mats);
             jb.scratch = reinterpret_cast<float*>(slot);
+            jb.sums = reinterpret_cast<unsigned long long*>(slot + a.slot_bytes - sums_bytes(a.kmax));
         }
         __syncthreads();
         const int n = s.n, k = jb.k;
@@ -959,6 +1019,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid
         if (threadIdx.x == 0) {
             slice_job(jb, slot + kSlotHead, s.n, a.kmax, a.mats);
             jb.scratch = reinterpret_cast<float*>(slot);
+            jb.sums = reinterpret_cast<unsigned long long*>(slot + a.slot_bytes - sums_bytes(a.kmax));
         }
         __syncthreads();
         set_accumulation(sh, 7, kSliceK / 16);
@@ -1012,7 +1073,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid
 
 size_t fp64_slot_bytes(int max_n, int mats, int planes) {
     const int64_t k = (static_cast<int64_t>(max_n) + 31) & ~int64_t(31);
-    return static_cast<size_t>(kSlotHead + mats * k * k * 8 + planes * slice_bytes(k));
+    return static_cast<size_t>(kSlotHead + mats * k * k * 8 + planes * slice_bytes(k) + sums_bytes(k));
 }
 
 // n_clusters clusters of `size` CTAs.

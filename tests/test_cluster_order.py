@@ -41,11 +41,19 @@ def test_bound_exchange_is_read_before_its_memory_is_reused():
 
 
 def test_column_norms_are_read_before_the_matrix_changes():
-    # the coupled iteration halves Z in place after its column norms: the norms end in a barrier of the cluster
+    # the maximum over the cluster's CTAs ends in a barrier, so the callers may change the matrix in place
     text = source("k_ns_fp64.cu")
     assert "cluster_max(" in body(text, "column_norm2") and "phase_sync()" in body(source("smx_slices.cuh"), "cluster_max")
-    b = body(text, "coupled_steps")
-    assert b.index("column_norm2(") < b.index("pass_affine(Z, shift ? Z")
+
+
+def test_row_lengths_are_read_before_they_are_cleared():
+    # the coupled iteration's sums: added to in a pass, read after its barrier, cleared after one more barrier
+    b = body(source("k_ns_fp64.cu"), "coupled_steps")
+    b = b[b.index("for (int it"):]
+    at = [b.index(x) for x in ("clear(row_y, 2 * k)", "pass_residual(", "longest(row_r)", "slice_product(sh, jb.P[0], jb.P[2]", "clear(row_r, k)",
+                               "pass_update(Y", "slice_product(sh, jb.P[2], jb.P[1]", "pass_update(Z", "longest(row_z)", "longest(row_y)",
+                               "pass_affine(Z, shift ? Z")]
+    assert at == sorted(at)
 
 
 def test_a_claimed_job_is_read_before_its_word_is_written_again():

@@ -61,3 +61,53 @@ def test_fermi_at_infinite_temperature_after_another_build(m, first):
         c.build_density()
         got = O.to_dense(s.block_size, s.col_ptr, s.row_idx, c.get_density())
     assert np.array_equal(got, 0.5 * np.eye(s.n))
+
+
+def _full(h, block=None):
+    """The matrix h on a complete pattern of blocks of at most 64 rows."""
+    n = h.shape[0]
+    block = block or min(n, 50)
+    s = make_mixed_block_system([block] * (n // block) + ([n % block] if n % block else []), r_c=np.inf, ell=1.5, seed=1)
+    first = np.concatenate([[0], np.cumsum(s.block_size)])
+    off = O.block_value_offsets(s.block_size, s.col_ptr, s.row_idx)
+    vals = np.empty_like(s.values)
+    for j in range(s.n_blocks):
+        for k in range(s.col_ptr[j], s.col_ptr[j + 1]):
+            r = s.row_idx[k]
+            vals[off[k]:off[k + 1]] = h[first[r]:first[r + 1], first[j]:first[j + 1]].T.ravel()
+    s.values[:] = vals
+    return s
+
+
+@pytest.mark.parametrize("coupling", [0.0, 0.005, 0.05, "rotated"])
+@pytest.mark.parametrize("n", [2, 6, 48, 200])
+@pytest.mark.parametrize("f", ["inv_sqrt", "sqrt", "inv", "overlap"])
+def test_one_negative_eigenvalue_is_not_positive_definite(f, n, coupling):
+    # a negative eigenvalue of any size, on one row, weakly coupled or spread over all: no root, so no result
+    from paper_2205_14741_gb300 import SmxError, SubmatrixDensity, _lib
+
+    rng = np.random.default_rng(n)
+    accepted = []
+    for x in list(np.linspace(0.1, 1.0, 10)) + [0.137, 0.333, 0.777, 0.9999, 1e-3]:
+        if coupling == "rotated":
+            v = rng.standard_normal(n)
+            h = np.eye(n) - (1.0 + x) * np.outer(v, v) / (v @ v)
+        else:
+            h = np.eye(n) + coupling * np.triu(rng.standard_normal((n, n)), 1) / np.sqrt(n)
+            h = np.triu(h) + np.triu(h, 1).T
+            p = int(rng.integers(n))
+            h[p, p] = -x
+        s = _full(h)
+        with SubmatrixDensity.from_system(s) as c:
+            if f == "overlap":
+                c.set_values(_full(np.diag(np.where(np.arange(n) % 2, 0.5, -0.5))).values)
+                c.set_overlap(s.values)
+            else:
+                c.set_function(f)
+            try:
+                c.build_density()
+                c.get_trace()
+                accepted.append(float(x))
+            except SmxError as e:
+                assert e.status in (_lib.ERR_NOCONV, _lib.ERR_NONFINITE)
+    assert accepted == []
