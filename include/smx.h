@@ -65,9 +65,11 @@ typedef enum {
 } smx_status;
 
 /* Arithmetic of the Newton-Schulz bulk phase (Eq. 13 iteration).
- *  SMX_FP64   : 64-bit arithmetic ("plain" form): products by error-free slices of eight bits on
- *               the tensor cores (the sums are exact, the result as accurate as FP64
- *               multiply-adds), 64-bit integers between them.
+ *  SMX_FP64   : 64-bit arithmetic ("plain" form).  A submatrix whose shortest row (2-norm) is at
+ *               least an eighth of its longest: products by error-free slices of eight bits on the
+ *               tensor cores, 64-bit integers between them, in units of the longest row; such a
+ *               result is as accurate as with FP64 multiply-adds.  The others, whose small rows
+ *               would lose digits there: FP64 multiply-adds (about 25 times slower).
  *  SMX_FP16X3 : tcgen05 tensor cores, FP16 operands split as hi + lo with three
  *               products (hi*hi + hi*lo + lo*hi) per step and FP32 accumulation
  *               in tensor memory; about 22 significant bits per operand.

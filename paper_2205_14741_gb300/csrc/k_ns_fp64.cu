@@ -43,6 +43,7 @@ struct SliceScalars {
     int job;
     int e;
     int bad;
+    int graded;        // the rows of the matrix looked at last are of very different size (kGraded)
     int stop;          // the schedule's factor allows this step to be the last
     uint64_t f1, f2;   // the step's factor a and a^2 (fixed_factor), 0 for a plain step
     double lsch;       // lower end of the interval the scaled schedule assumes (1: plain steps)
@@ -59,7 +60,6 @@ __device__ __forceinline__ void slice_job(SliceJob& jb, uint8_t* slot, int n, in
 }
 // The first bytes of a slot serve the cluster (kSlotHead); slice_job gets what follows.  The last hold the rows'
 // squared lengths.
-constexpr int64_t kSlotHead = 256;
 constexpr int64_t sums_bytes(int64_t k) { return 3 * 8 * k; }
 
 // Adds the squared length of sixteen neighbouring entries of row r, half each of a lane pair (s: this lane's in units
@@ -115,6 +115,35 @@ __device__ __forceinline__ void set_accumulation(SliceShared* sh, int weights, i
     __syncthreads();
 }
 
+// Submatrices whose shortest row (2-norm) is below kGraded times the longest go to the FP64 kernels (k_ns_graded.cu).
+// The fixed point here holds an entry to 2^-57 of the longest row, floating point to 2^-53 of itself: for A = D S0 D, S0
+// well conditioned, the relative error of the roots and of the sign grows as 1 / d^2 in the one (d the smallest entry
+// of D) and not at all in the other.  An emulation of both (n = 16): at a ratio of the rows of 1, 1/5, 1/10, 1/20 and
+// 1/100 the roots' error is 5e-17, 1e-16, 2e-16, 3e-16 and 2e-15 in fixed point, 2e-16 .. 6e-16 in FP64; the sign's
+// 6e-17, 1e-16, 3e-16, 1e-15 and 2e-14, 3e-16 .. 1e-15 in FP64.  They cross between 1/10 and 1/20, so
+// from 1/8 on none is further off than in FP64.  (The water-like systems' rows: 0.6 and more.)
+constexpr float kGraded = 1.0f / 8.0f;
+
+// Puts block column j on the list; one thread of a cluster calls it.
+__device__ __forceinline__ void list_graded(GradedList* list, int j) { list->column[atomicAdd(&list->count, 1)] = j; }
+
+// The cluster's sums of squared lengths (SliceJob::sums): cleared a phase before they are added to and a phase after
+// every CTA has read them; the largest and the smallest of n of them.
+__device__ __forceinline__ void clear_sums(unsigned long long* sums, int count) {
+    for (int r = cluster_rank() * kSliceThreads + threadIdx.x; r < count; r += cluster_size() * kSliceThreads) __stcg(sums + r, 0ull);
+}
+__device__ __forceinline__ unsigned long long largest_sum(const unsigned long long* sums, int n, SliceScalars* ss) {
+    unsigned long long m = 0;
+    for (int r = threadIdx.x; r < n; r += kSliceThreads) m = max(m, __ldcg(sums + r));
+    return cta_max_u64(m, ss);
+}
+__device__ __noinline__ bool sums_graded(const unsigned long long* sums, int n, SliceScalars* ss) {
+    const unsigned long long most = largest_sum(sums, n, ss);
+    unsigned long long m = 0;
+    for (int r = threadIdx.x; r < n; r += kSliceThreads) m = max(m, ~__ldcg(sums + r));
+    return static_cast<float>(~cta_max_u64(m, ss)) < kGraded * kGraded * static_cast<float>(most);
+}
+
 // The bits of entries (r, c .. c + 7) of a symmetric matrix of doubles (read along its rows), zero past n.
 __device__ __forceinline__ void load_bits(const double* __restrict__ src, int ld, int n, int r, int c, int64_t (&v)[8]) {
 #pragma unroll
@@ -124,9 +153,10 @@ __device__ __forceinline__ void load_bits(const double* __restrict__ src, int ld
 // The elementwise passes between products (each a function of its own, so that its registers are
 // its own: what the callers keep across it lies on the stack, not what its loop works on).
 
-// The symmetric n x n matrix src - mu I, times f 2^-e, into M and the planes (see to_fixed).
+// The symmetric n x n matrix src - mu I, times f 2^-e, into M and the planes (see to_fixed).  The rows' squared
+// lengths are added to sums, in units of 2^-48 (they may all be short: f 2^-e brings a bound of the eigenvalues to 1).
 __device__ __noinline__ bool pass_source(const double* __restrict__ src, int ld, double mu, int e, uint64_t f, int64_t* M, uint8_t* planes, int n,
-                                         int k) {
+                                         int k, unsigned long long* sums = nullptr) {
     bool bad = false;
     slice_pass<1>(k, k, planes, [&](int r, int c, int64_t (&v)[1][8]) { load_bits(src, ld, n, r, c, v[0]); },
                   [&](int r, int c, const int64_t (&v)[1][8], int64_t (&q)[8]) {
@@ -137,6 +167,11 @@ __device__ __noinline__ bool pass_source(const double* __restrict__ src, int ld,
                           q[i] = to_fixed(x, e, f, bad);
                       }
                       st8(M, k, r, c, q);
+                      if (sums) {
+                          float s = length8(q);
+                          s += __shfl_xor_sync(0xffffffffu, s, 1);
+                          if ((threadIdx.x & 1) == 0) atomicAdd(sums + r, static_cast<unsigned long long>(s * 0x1p24f));
+                      }
                   });
     return bad;
 }
@@ -281,7 +316,8 @@ __device__ __noinline__ void pass_transposed(const int64_t* A, const int64_t* B,
 // The symmetric source matrix A = src - mu I (n x n, leading dimension ld) in fixed point, A 2^-e, into M and
 // the planes P.  The power of two brings the largest 2-norm of a row into (1/2, 1] (so that the
 // products are exact and use all digits); iterate: src is a bulk phase's iterate, made symmetric, e = 0.  bound: no entry is larger (0:
-// not known).  Returns e; a value that is not finite sets ss->bad.
+// not known).  Returns e; a value that is not finite sets ss->bad, rows of very different size ss->graded: nothing is
+// loaded then.
 __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, double mu, double bound, const SliceJob& jb, int64_t* M, uint8_t* P,
                           bool iterate, SliceShared* sh, SliceScalars* ss) {
     const int n = jb.n, k = jb.k, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -291,7 +327,8 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
     };
     const int ranks = cluster_size(), rank = cluster_rank();
     int e = 0;
-    if (threadIdx.x == 0) ss->bad = 0;
+    bool graded = false;
+    if (threadIdx.x == 0) ss->bad = ss->graded = 0;
     if (!iterate) {
         uint32_t top = static_cast<uint32_t>(__double2hiint(bound)) & 0x7fffffffu;
         if (top == 0) {  // high words order like the magnitudes
@@ -309,10 +346,10 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
         }
         const int e0 = ex - 1022;  // |A| < 2^e0
         auto scaled = [&](double v) -> float {  // v 2^-e0, 0 below 2^-122
-            const int hi = __double2hiint(v), ef = ((hi >> 20) & 0x7ff) - e0;
-            return ef > 900 ? d2f_rn(__hiloint2double((hi & 0x800fffff) | (ef << 20), __double2loint(v))) : 0.0f;
+            const int hi = __double2hiint(v), ev = (hi >> 20) & 0x7ff, ef = ev - e0;
+            return ev > 0 && ef > 900 ? d2f_rn(__hiloint2double((hi & 0x800fffff) | (ef << 20), __double2loint(v))) : 0.0f;
         };
-        float worst = 0.0f;
+        float worst = 0.0f, least = INFINITY;
         for (int r = 2 * (warp + rank * kSliceWarps); r < n; r += 2 * ranks * kSliceWarps) {
             const int r1 = min(r + 1, n - 1);
             float a0 = 0.0f, a1 = 0.0f;
@@ -328,11 +365,32 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
                 a1 += __shfl_xor_sync(0xffffffffu, a1, o);
             }
             worst = fmaxf(worst, fmaxf(a0, a1));
+            least = fminf(least, fminf(a0, a1));
         }
-        worst = __uint_as_float(cluster_max(__float_as_uint(cta_max(worst, sh)), reinterpret_cast<uint32_t*>(jb.scratch) + 8));
+        // the largest, and the smallest by the largest complement (non-negative floats order like their bits)
+        worst = cta_max(worst, sh);
+        uint32_t rest = static_cast<uint32_t>(cta_max_u64(~__float_as_uint(least), ss));
+        if (ranks > 1) {
+            uint32_t* const ex = reinterpret_cast<uint32_t*>(jb.scratch);
+            if (threadIdx.x == 0) {
+                __stcg(ex + 8 + rank, __float_as_uint(worst));
+                __stcg(ex + 56 + rank, rest);
+            }
+            phase_sync();
+            for (int r = 0; r < ranks; ++r) {
+                worst = fmaxf(worst, __uint_as_float(__ldcg(ex + 8 + r)));
+                rest = max(rest, __ldcg(ex + 56 + r));
+            }
+        }
+        graded = __uint_as_float(~rest) < kGraded * kGraded * worst;
         e = e0 + (worst > 0.0f ? static_cast<int>(ceilf(0.5f * log2f(worst * 1.001f))) : 0);
     }
     __syncthreads();
+    if (graded) {
+        if (threadIdx.x == 0) ss->graded = 1;
+        __syncthreads();
+        return e;
+    }
     const bool own_bad = iterate ? pass_iterate(src, ld, M, P, n, k) : pass_source(src, ld, mu, e, 0, M, P, n, k);
     const bool bad = cluster_sum(own_bad ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f;
     if (bad) ss->bad = 1;
@@ -586,22 +644,17 @@ __device__ __noinline__ float column_norm2(const SliceJob& jb, const int64_t* M,
 // rows are too long enters no product: with rows of at most 1 in both factors no entry of a product leaves
 // the integers' range, nor does X + 1/2 X R, and nothing wraps before it is seen.  A negative eigenvalue -t of Z Y
 // grows from step to step (t (3 + t)^2 / 4 > 2.25 t) until the rows of R, which hold its 1 + t, are too long.
+//
+// Returns the number of steps, -1 for rows of very different size (kGraded); with want_z ss->graded tells whether Z's are.
 __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* __restrict__ src, int ld, double b, int max_iter, float tau,
                              bool want_y, bool want_z, int& ez, SliceScalars* ss, bool& conv, bool& bad) {
     const int n = jb.n, k = jb.k;
     int64_t *Y = jb.M[0], *Z = jb.M[1], *S = jb.M[2];
     unsigned long long *row_r = jb.sums, *row_y = row_r + k, *row_z = row_y + k;  // squared lengths in units of 2^-24
-    // (cleared one phase or more after every CTA of the cluster has read them, and before they are added to)
-    auto clear = [&](unsigned long long* sums, int count) {
-        for (int r = cluster_rank() * kSliceThreads + threadIdx.x; r < count; r += cluster_size() * kSliceThreads) __stcg(sums + r, 0ull);
-    };
-    auto longest = [&](const unsigned long long* sums) {
-        unsigned long long m = 0;
-        for (int r = threadIdx.x; r < n; r += kSliceThreads) m = max(m, __ldcg(sums + r));
-        return static_cast<float>(cta_max_u64(m, ss)) * 0x1p-24f;
-    };
+    auto longest = [&](const unsigned long long* sums) { return static_cast<float>(largest_sum(sums, n, ss)) * 0x1p-24f; };
     constexpr float kLongest = 1.002f;  // of a length squared that is at most 1 (its squares are rounded)
-    clear(row_r, 3 * k);
+    clear_sums(row_r, 3 * k);
+    phase_sync();
     conv = bad = false;
     ez = 0;
     int done = 0;
@@ -611,17 +664,19 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
     const uint64_t f = ((ib & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
     const int e = 1022 - static_cast<int>((ib >> 52) & 0x7ff);
     bool off = !(b > 0.0) || !isfinite(inv) || inv == 0.0;
-    off |= pass_source(src, ld, 0.0, e, f, Y, jb.P[0], n, k);
+    off |= pass_source(src, ld, 0.0, e, f, Y, jb.P[0], n, k, row_z);
+    const bool graded = sums_graded(row_z, n, ss);
     if (cluster_sum(off ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f) {
         bad = true;
         return 0;
     }
+    if (graded) return -1;
     for (int it = 0; it < max_iter; ++it) {
         if (it > 0) {
             slice_product(sh, jb.P[1], jb.P[0], k, k, S, true);  // Z Y
             if (*static_cast<volatile int*>(&sh->abort)) break;
         }
-        clear(row_y, 2 * k);
+        clear_sums(row_y, 2 * k);
         float r2 = pass_residual(it > 0 ? S : Y, jb.P[2], n, k, ez, 0, row_r);
         r2 = cluster_sum(r2 * 0x1p-76f, sh, jb.scratch);
         done = it + 1;
@@ -633,7 +688,7 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
         if (!conv || want_y) {
             slice_product(sh, jb.P[0], jb.P[2], k, k, S, true);  // Y R
             if (*static_cast<volatile int*>(&sh->abort)) break;
-            clear(row_r, k);
+            clear_sums(row_r, k);
             pass_update(Y, S, jb.P[0], k, 0, row_y);
         }
         if (!conv || want_z) {
@@ -656,6 +711,11 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
         }
         if (conv) break;
     }
+    if (conv && want_z) {
+        const bool z_graded = sums_graded(row_z, n, ss);
+        if (threadIdx.x == 0) ss->graded = z_graded;
+        __syncthreads();
+    }
     return done;
 }
 
@@ -670,7 +730,8 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
 //   F = 1/2 (I - T).
 // A doubling at most doubles an error in T (m = 11 at beta g = 150).  T is kept as T 2^t with the
 // largest t for which its norm bound min(1, 2^doublings / 16) stays below 1.  The result's T 2^t is in
-// M[0] (units of 2^-62), t in ss->e; M[1] takes the products.  Returns the number of products.
+// M[0] (units of 2^-62), t in ss->e; M[1] takes the products.  Returns the number of products, -1 for rows
+// of very different size (kGraded).
 __device__ int fermi_tanh(SliceShared* sh, const SliceJob& jb, const double* __restrict__ src, int ld, double g, double beta, SliceScalars* ss,
                           bool& bad) {
     const int n = jb.n, k = jb.k;
@@ -698,7 +759,13 @@ __device__ int fermi_tanh(SliceShared* sh, const SliceJob& jb, const double* __r
     const int e = 1022 - static_cast<int>((ib >> 52) & 0x7ff);
     const bool zero = !(fac > 0.0);
     bool off = !isfinite(fac);
-    if (!zero && !off) off = pass_source(src, ld, 0.0, e, f, T, PT, n, k);
+    bool graded = false;
+    if (!zero && !off) {
+        clear_sums(jb.sums, k);
+        phase_sync();
+        off = pass_source(src, ld, 0.0, e, f, T, PT, n, k, jb.sums);
+        graded = sums_graded(jb.sums, n, ss);
+    }
     if (cluster_sum(off ? 1.0f : 0.0f, sh, jb.scratch) > 0.0f) {
         bad = true;
         return 0;
@@ -707,6 +774,7 @@ __device__ int fermi_tanh(SliceShared* sh, const SliceJob& jb, const double* __r
         pass_zero(T, k);
         return 0;
     }
+    if (graded) return -1;
     int nprod = 0;
     // wide: with the digit pairs of weight 9 (an error in T may double at every doubling; the products of
     // K enter it with factors of 1/9 and less)
@@ -882,6 +950,10 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
         if constexpr (FORM == kFormFermi) {
             done = fermi_tanh(sh, jb, T, s.ld, a.bound[j], a.beta, &ss, bad);
             if (sh->abort) break;
+            if (done < 0) {
+                if (threadIdx.x == 0 && lead) list_graded(a.graded, j);
+                continue;
+            }
             if (threadIdx.x == 0 && lead) {
                 a.iters[j] = done;
                 atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
@@ -900,6 +972,10 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
             done = coupled_steps(sh, jb, T, s.ld, b, a.max_iter, static_cast<float>(a.tau), a.function == kFnSqrt, a.function != kFnSqrt, ez,
                                  &ss, conv, bad);
             if (sh->abort) break;
+            if (done < 0) {
+                if (threadIdx.x == 0 && lead) list_graded(a.graded, j);
+                continue;
+            }
             if (threadIdx.x == 0 && lead) {
                 a.iters[j] = done;
                 atomicAdd(a.work_n3, static_cast<unsigned long long>(n) * n * n * done);
@@ -947,6 +1023,10 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
         SignModel model{a.bound[j], a.pred ? static_cast<double>(a.pred[2 * j + 1]) * gersh / a.bound[j] : -1.0, a.fallbacks};
         const int e = load_fixed(src, s.ld, a.Mc ? a.mu : 0.0, gersh, jb, jb.M[0], jb.P[0], finish, sh, &ss);
         bad = ss.bad != 0;
+        if (!bad && (ss.graded || (a.Mc && a.root_graded[j]))) {  // (L is a factor of the result)
+            if (threadIdx.x == 0 && lead) list_graded(a.graded, j);
+            continue;
+        }
         // with the learned bound W reaches a norm of 2, with a bulk phase's iterate X one of about 1.2
         set_accumulation(sh, 7, a.use_model || finish ? 160 / 16 : kSliceK / 16);
         if (!bad)
@@ -1027,7 +1107,12 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid
         int ez = 0;
         const int done = coupled_steps(sh, jb, a.Lc + s.t_off, s.ld, a.bound_s[s.col], a.max_iter, static_cast<float>(a.tau), false, true, ez, &ss, conv, bad);
         if (sh->abort) break;
+        if (done < 0) {
+            if (threadIdx.x == 0 && cluster_rank() == 0) list_graded(a.graded, s.col);
+            continue;
+        }
         if (threadIdx.x == 0 && cluster_rank() == 0) {
+            a.root_graded[s.col] = ss.graded;
             a.iters[s.col] = done;
             if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
             else if (!conv) atomicCAS(a.status, kOk, kErrNoconv);
@@ -1044,6 +1129,10 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid
                 atomicCAS(a.status, kOk, kErrNonfinite);
                 a.lohi[2 * s.col] = a.lohi[2 * s.col + 1] = 0.0;
             }
+            continue;
+        }
+        if (ss.graded) {
+            if (threadIdx.x == 0 && cluster_rank() == 0) list_graded(a.graded, s.col);
             continue;
         }
         set_accumulation(sh, 8, 160 / 16);
@@ -1136,15 +1225,19 @@ cudaError_t device_clusters(int* room) {
 
 cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_n, int max_nblk, const int* room, cudaStream_t st) {
     if (sizeof(int) * (static_cast<size_t>(max_nblk) + 1) > kSliceSmem - 1024) return cudaErrorInvalidValue;
+    cudaError_t e;
     switch (a.function) {
-        case kFnDensity: return launch_form(k_ns_fp64<kFormSign>, a, slots, max_n, room, st);
-        case kFnFermi: return launch_form(k_ns_fp64<kFormFermi>, a, slots, max_n, room, st);
-        default: return launch_form(k_ns_fp64<kFormRoots>, a, slots, max_n, room, st);
+        case kFnDensity: e = launch_form(k_ns_fp64<kFormSign>, a, slots, max_n, room, st); break;
+        case kFnFermi: e = launch_form(k_ns_fp64<kFormFermi>, a, slots, max_n, room, st); break;
+        default: e = launch_form(k_ns_fp64<kFormRoots>, a, slots, max_n, room, st);
     }
+    if (e != cudaSuccess || a.finish_iters > 0) return e;
+    return launch_ns_graded(a, slots, max_nblk, st);
 }
 
 cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, int max_n, const int* room, cudaStream_t st) {
-    return launch_form(k_nonorth_setup, a, slots, max_n, room, st);
+    const cudaError_t e = launch_form(k_nonorth_setup, a, slots, max_n, room, st);
+    return e != cudaSuccess ? e : launch_graded_setup(a, slots, st);
 }
 
 }  // namespace smx
@@ -1177,7 +1270,8 @@ constexpr int kNoAllocMaxDevices = 64;
 }  // namespace
 
 // The slot of one CTA (two matrices of 64-bit integers and the digits of two operands) for n = 256,
-// followed by a small header: [0] status, [1] iterations.  About 2.8 MiB.
+// followed by a small header: [0] status, [1] iterations, [2] rows of very different size (for k_dense_graded, with a bound
+// of their length at [4]).  About 2.8 MiB.
 constexpr int64_t kNoAllocBytes = kSlotHead + 2 * kNoAllocMat * 8 + 2 * slice_bytes(kNoAllocMaxN);
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes + 32];
 
@@ -1189,7 +1283,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(cons
     __shared__ SliceScalars ss;
     __shared__ SignBound sb;
     int* hdr = reinterpret_cast<int*>(scratch + kNoAllocBytes);
-    if (threadIdx.x == 0 && cluster_rank() == 0) hdr[0] = kOk;
+    if (threadIdx.x == 0 && cluster_rank() == 0) hdr[0] = kOk, hdr[2] = 0;
     SliceShared* const sh = &shared;
     slices_begin(sh, slice_stages(), hdr);
     // every call overwrites the work matrices in full; nothing is carried over
@@ -1202,9 +1296,10 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(cons
     const int e = load_fixed(H, n, mu, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
     bool conv = false, bad = ss.bad != 0;
     int done = 0;
-    if (!bad) done = sign_steps(sh, jb, e, max_iter, tau, 0, nullptr, &sb, &ss, conv, bad);
+    const bool graded = !bad && ss.graded;
+    if (!bad && !graded) done = sign_steps(sh, jb, e, max_iter, tau, 0, nullptr, &sb, &ss, conv, bad);
     const bool aborted = *static_cast<volatile int*>(&sh->abort) != 0;
-    if (!aborted) {
+    if (!aborted && !graded) {
         const int64_t* X = jb.M[0];
         for (int r = cluster_rank() * kSliceWarps + (threadIdx.x >> 5); r < n; r += cluster_size() * kSliceWarps)
             for (int c = threadIdx.x & 31; c < n; c += 32) {  // 1/2 (I - X) in units of 2^-63: up to 2^63
@@ -1216,7 +1311,11 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(cons
     }
     slices_end(sh);
     if (threadIdx.x == 0 && cluster_rank() == 0) {
-        if (!aborted) atomicCAS(hdr, kOk, bad ? kErrNonfinite : (conv ? kOk : kErrNoconv));
+        if (graded) {
+            hdr[2] = 1;
+            *reinterpret_cast<double*>(hdr + 4) = ldexp(1.0, e);
+        }
+        if (!aborted && !graded) atomicCAS(hdr, kOk, bad ? kErrNonfinite : (conv ? kOk : kErrNoconv));
         hdr[1] = done;
     }
 }
@@ -1280,6 +1379,10 @@ extern "C" smx_status smx_dense_density_noalloc(const double* h_dev, int32_t n, 
         if (e != cudaSuccess) cudaGetLastError();
     }
     if (e != cudaSuccess) return SMX_ERR_CUDA;
+    int* const head = reinterpret_cast<int*>(scratch + smx::kNoAllocBytes);
+    if (smx::launch_dense_graded(h_dev, static_cast<int>(n), mu, d_dev, scratch, 1e-7, 100, head + 2, reinterpret_cast<double*>(head + 4), head, st) !=
+        cudaSuccess)
+        return SMX_ERR_CUDA;
     int hdr[2] = {0, 0};
     if (cudaMemcpyAsync(hdr, scratch + smx::kNoAllocBytes, sizeof(hdr), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return SMX_ERR_CUDA;

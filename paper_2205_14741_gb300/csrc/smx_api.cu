@@ -103,7 +103,7 @@ struct smx_ctx {
     DevBuf d_sc;                      // DevScalars: status, flags, bracket, trace and energy
     DevScalars* h_sc = nullptr;       // pinned copy, filled by fetch()
     DevBuf d_fcol_ptr, d_frow_idx, d_fvoff, d_lstart, d_subs, d_order, d_maps, d_map_off;
-    DevBuf d_T, d_W1, d_ws, d_tc_exchange, d_ws64, d_D, d_xown;
+    DevBuf d_T, d_W1, d_ws, d_tc_exchange, d_ws64, d_graded, d_D, d_xown;
     DevBuf d_bound, d_iters, d_partial, d_work_n3;
     uint8_t* h_keep_pinned = nullptr;
 
@@ -134,7 +134,7 @@ struct smx_ctx {
 
     // non-orthogonal form (Eq. 14 with an overlap S on the pattern of H)
     bool have_S = false, nonorth_ready = false;
-    DevBuf d_S, d_Lc, d_Mc, d_nlohi, d_setup_iters;
+    DevBuf d_S, d_Lc, d_Mc, d_nlohi, d_setup_iters, d_root_graded;
     double nbr_lo = 0.0, nbr_hi = 0.0;  // bracket: the Gershgorin intervals of all M_j
 
     // learned spectral bound
@@ -537,6 +537,10 @@ static smx_status prepare_fp64_slots(smx_ctx* c, int m, int mats, int planes, in
     const size_t staging = c->staging_limit ? c->staging_limit : device_memory(c) / 10;
     const size_t fit = (mats == 2 && planes == 2 ? 2 : 4) * staging / *slot_bytes;
     if (fit < static_cast<size_t>(*slots)) *slots = std::max<int>(1, static_cast<int>(fit));
+    if (!c->d_graded.p) {
+        SMX_TRY(ensure(c->d_graded, graded_list_bytes(c->B)));
+        SMX_CUDA(cudaMemsetAsync(c->d_graded.p, 0, sizeof(GradedList), c->stream));
+    }
     return ensure(c->d_ws64, *slot_bytes * static_cast<size_t>(*slots));
 }
 
@@ -552,6 +556,7 @@ static smx_status nonorth_setup(smx_ctx* c) {
     SMX_TRY(ensure(c->d_Mc, tb));
     SMX_TRY(ensure(c->d_nlohi, sizeof(double) * 2 * c->B));
     SMX_TRY(ensure(c->d_setup_iters, sizeof(int32_t) * c->B));
+    SMX_TRY(ensure(c->d_root_graded, sizeof(int32_t) * c->B));
     const int j0 = c->chunk_start[0], m = c->chunk_start[1] - j0;
     int slots = 0;
     size_t slot_bytes = 0;
@@ -580,9 +585,11 @@ static smx_status nonorth_setup(smx_ctx* c) {
     a.max_iter = 100;
     a.iters = dp<int32_t>(c->d_setup_iters);
     a.lohi = dp<double>(c->d_nlohi);
+    a.root_graded = dp<int32_t>(c->d_root_graded);
+    a.graded = dp<GradedList>(c->d_graded);
     a.status = &scalars(c)->status;
     SMX_CUDA(launch_nonorth_setup(a, slots, c->max_n, c->clusters, st));
-    c->kernel_launches += 3;
+    c->kernel_launches += 4;
     std::vector<double> lohi(2 * static_cast<size_t>(m));
     SMX_CUDA(cudaMemcpyAsync(lohi.data(), dp<double>(c->d_nlohi) + 2 * j0, sizeof(double) * lohi.size(), cudaMemcpyDeviceToHost, st));
     const smx_status ds = read_status(c);  // synchronises
@@ -657,6 +664,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
         a.H = dp<double>(c->d_H);
         a.D = dp<double>(c->d_D);
         a.partial = dp<double2>(c->d_partial);
+        a.graded = dp<GradedList>(c->d_graded);
         a.skip = skip;
         return a;
     };
@@ -688,10 +696,12 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
                 a.Mc = dp<double>(c->d_Mc);
                 a.Lc = dp<double>(c->d_Lc);
                 a.Sv = dp<double>(c->d_S);
+                a.root_graded = dp<int32_t>(c->d_root_graded);
                 a.mu = mu;
             }
             SMX_CUDA(cudaEventRecord(ns0, st));
             SMX_CUDA(launch_ns_fp64(a, std::min(slots, m), c->max_n, c->max_nblk, c->clusters, st));
+            c->kernel_launches += 1;  // (and the kernel of the listed submatrices)
             SMX_CUDA(cudaEventRecord(ns1, st));
         } else {
             NsTcArgs a;
@@ -1503,7 +1513,7 @@ void smx_destroy(smx_ctx* c) {
                       &c->d_params, &c->d_mst, &c->d_vst, &c->d_partial_mlp, &c->d_feat, &c->d_pred, &c->d_labels,
                       &c->d_gersh, &c->d_prev_ratio, &c->d_sq_ratio, &c->d_tridiag, &c->d_loss, &c->d_sx, &c->d_st,
                       &c->d_fit_x, &c->d_fit_t, &c->d_grad, &c->d_S, &c->d_Lc, &c->d_Mc, &c->d_nlohi,
-                      &c->d_setup_iters};
+                      &c->d_setup_iters, &c->d_root_graded, &c->d_graded};
     for (DevBuf* b : bufs) release(*b);
     for (auto& pr : c->ns_events) {
         cudaEventDestroy(pr.first);

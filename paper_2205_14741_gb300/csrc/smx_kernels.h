@@ -92,8 +92,18 @@ enum : int { kFnDensity = 0, kFnInvSqrt = 1, kFnSqrt = 2, kFnInv = 3, kFnFermi =
 // A CTA (or cluster) of the 64-bit kernels works in a slot of global memory: up to three k x k matrices of 64-bit
 // integers and the digits of up to three operands (smx_slices.cuh).
 constexpr int kFp64Mats = 3, kFp64Planes = 3;
-// Bytes of a slot for submatrices of up to max_n rows.
+// Bytes of a slot for submatrices of up to max_n rows (at least five n x n matrices of doubles after its head).
 size_t fp64_slot_bytes(int max_n, int mats, int planes);
+// The first bytes of a slot serve the CTAs that share it.
+constexpr int64_t kSlotHead = 256;
+
+// Block columns whose submatrices a 64-bit kernel leaves to the FP64 kernels (k_ns_graded.cu), which follow it on the
+// stream and empty the list.
+struct GradedList {
+    int count, next, done, unused;
+    int32_t column[1];  // count of them
+};
+inline size_t graded_list_bytes(int n_cols) { return sizeof(GradedList) + sizeof(int32_t) * static_cast<size_t>(n_cols); }
 
 struct NsFp64Args {
     const SubDesc* subs;
@@ -127,7 +137,9 @@ struct NsFp64Args {
     const double* Mc = nullptr;  // M_j = L_j A_H L_j, laid out like T
     const double* Lc = nullptr;  // L_j = A_S^-1/2, laid out like T
     const double* Sv = nullptr;  // S in the input value layout
+    const int32_t* root_graded = nullptr;  // per block column: L_j's rows are of very different size
     double mu = 0.0;
+    GradedList* graded;  // empty at launch and afterwards
     // learned bound: predictions per block column ([2 j + 1] = delta_hat / G_j); see NsTcArgs::pred
     const float* pred = nullptr;
     // FP64 finishing steps after a low-precision bulk phase (> 0): T holds the bulk phase's last
@@ -161,9 +173,17 @@ struct NonorthSetupArgs {
     int max_iter;
     int32_t* iters;         // out: steps of the coupled iteration per block column
     double* lohi;           // out: [2 * B] Gershgorin interval of M_j
+    int32_t* root_graded;   // out: per block column: L_j's rows are of very different size
+    GradedList* graded;     // empty at launch and afterwards
     int* status;
 };
 cudaError_t launch_nonorth_setup(const NonorthSetupArgs& a, int slots, int max_n, const int* room, cudaStream_t st);
+// Both launch a second kernel for the listed submatrices (a build's finishing steps do not):
+cudaError_t launch_ns_graded(const NsFp64Args& a, int slots, int max_nblk, cudaStream_t st);
+cudaError_t launch_graded_setup(const NonorthSetupArgs& a, int slots, cudaStream_t st);
+// ... and the dense entry point: D of H when *graded is not 0 (see k_dense_graded).
+cudaError_t launch_dense_graded(const double* H, int n, double mu, double* D, uint8_t* slot, double tau, int max_iter, int* graded, const double* b,
+                                int* status, cudaStream_t st);
 
 // a5 (tcgen05 tensor cores) + a7.
 // CTAs that share a submatrix in the streamed form; what a cluster exchanges in global memory: the

@@ -50,7 +50,7 @@ def test_row_lengths_are_read_before_they_are_cleared():
     # the coupled iteration's sums: added to in a pass, read after its barrier, cleared after one more barrier
     b = body(source("k_ns_fp64.cu"), "coupled_steps")
     b = b[b.index("for (int it"):]
-    at = [b.index(x) for x in ("clear(row_y, 2 * k)", "pass_residual(", "longest(row_r)", "slice_product(sh, jb.P[0], jb.P[2]", "clear(row_r, k)",
+    at = [b.index(x) for x in ("clear_sums(row_y, 2 * k)", "pass_residual(", "longest(row_r)", "slice_product(sh, jb.P[0], jb.P[2]", "clear_sums(row_r, k)",
                                "pass_update(Y", "slice_product(sh, jb.P[2], jb.P[1]", "pass_update(Z", "longest(row_z)", "longest(row_y)",
                                "pass_affine(Z, shift ? Z")]
     assert at == sorted(at)
