@@ -315,11 +315,13 @@ __device__ __noinline__ void pass_transposed(const int64_t* A, const int64_t* B,
 
 // The symmetric source matrix A = src - mu I (n x n, leading dimension ld) in fixed point, A 2^-e, into M and
 // the planes P.  The power of two brings the largest 2-norm of a row into (1/2, 1] (so that the
-// products are exact and use all digits); iterate: src is a bulk phase's iterate, made symmetric, e = 0.  bound: no entry is larger (0:
-// not known).  Returns e; a value that is not finite sets ss->bad, rows of very different size ss->graded: nothing is
-// loaded then.
+// products are exact and use all digits); kIterate: src is a bulk phase's iterate, made symmetric, e = 0.  bound: no entry is larger (0:
+// not known).  Returns e; a value that is not finite sets ss->bad, and rows of very different size set ss->graded (but
+// for kFactor, whose rows have been looked at): nothing is loaded then.
+enum { kSource, kIterate, kFactor };
 __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, double mu, double bound, const SliceJob& jb, int64_t* M, uint8_t* P,
-                          bool iterate, SliceShared* sh, SliceScalars* ss) {
+                          int kind, SliceShared* sh, SliceScalars* ss) {
+    const bool iterate = kind == kIterate;
     const int n = jb.n, k = jb.k, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto entry = [&](int r, int c) -> double {
         const double v = src[static_cast<int64_t>(r) * ld + c];
@@ -382,7 +384,7 @@ __device__ __noinline__ int load_fixed(const double* __restrict__ src, int ld, d
                 rest = max(rest, __ldcg(ex + 56 + r));
             }
         }
-        graded = __uint_as_float(~rest) < kGraded * kGraded * worst;
+        graded = kind == kSource && __uint_as_float(~rest) < kGraded * kGraded * worst;
         e = e0 + (worst > 0.0f ? static_cast<int>(ceilf(0.5f * log2f(worst * 1.001f))) : 0);
     }
     __syncthreads();
@@ -1021,7 +1023,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
         const bool finish = a.finish_iters > 0;
         const double gersh = a.Mc ? scratch[32] : a.gersh[j];
         SignModel model{a.bound[j], a.pred ? static_cast<double>(a.pred[2 * j + 1]) * gersh / a.bound[j] : -1.0, a.fallbacks};
-        const int e = load_fixed(src, s.ld, a.Mc ? a.mu : 0.0, gersh, jb, jb.M[0], jb.P[0], finish, sh, &ss);
+        const int e = load_fixed(src, s.ld, a.Mc ? a.mu : 0.0, gersh, jb, jb.M[0], jb.P[0], finish ? kIterate : kSource, sh, &ss);
         bad = ss.bad != 0;
         if (!bad && (ss.graded || (a.Mc && a.root_graded[j]))) {  // (L is a factor of the result)
             if (threadIdx.x == 0 && lead) list_graded(a.graded, j);
@@ -1058,7 +1060,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
             set_accumulation(sh, 8, 160 / 16);
             pass_affine(X, nullptr, jb.P[0], n, k, 0, false, 0, 0);
             int64_t *L = jb.M[0], *U = jb.M[1];
-            const int el = load_fixed(a.Lc + s.t_off, s.ld, 0.0, 0.0, jb, L, jb.P[1], false, sh, &ss);
+            const int el = load_fixed(a.Lc + s.t_off, s.ld, 0.0, 0.0, jb, L, jb.P[1], kFactor, sh, &ss);
             const int w = s.bown <= 16 ? 16 : (s.bown + 31) & ~31;
             pass_transposed(L, nullptr, s.own, s.bown, jb.P[2], w, k, 0);
             slice_product(sh, jb.P[0], jb.P[2], k, w, U, false);
@@ -1123,7 +1125,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_nonorth_setup(const __grid
         }
         // A_H 2^-eh with rows of at most 1; Q = A_H L, then M = L Q = L A_H L: the right factor's digits
         // are those of Q^T, whose rows are Q's columns
-        const int eh = load_fixed(a.Mc + s.t_off, s.ld, 0.0, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
+        const int eh = load_fixed(a.Mc + s.t_off, s.ld, 0.0, 0.0, jb, jb.M[0], jb.P[0], kSource, sh, &ss);
         if (ss.bad) {
             if (threadIdx.x == 0 && cluster_rank() == 0) {
                 atomicCAS(a.status, kOk, kErrNonfinite);
@@ -1293,7 +1295,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(cons
         jb.scratch = reinterpret_cast<float*>(scratch);
     }
     __syncthreads();
-    const int e = load_fixed(H, n, mu, 0.0, jb, jb.M[0], jb.P[0], false, sh, &ss);
+    const int e = load_fixed(H, n, mu, 0.0, jb, jb.M[0], jb.P[0], kSource, sh, &ss);
     bool conv = false, bad = ss.bad != 0;
     int done = 0;
     const bool graded = !bad && ss.graded;

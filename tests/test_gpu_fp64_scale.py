@@ -229,3 +229,24 @@ def test_graded_and_other_submatrices_in_one_build():
         host = c.get_density(), c.get_trace()
         c.solve_mu_device()
         assert np.array_equal(c.get_density(), host[0]) and c.get_trace() == host[1]
+
+
+@pytest.mark.parametrize("f", ["inv_sqrt", "density", "overlap"])
+def test_rows_at_the_line_between_the_forms(f):
+    # a ratio of the rows at 1/8 and within a few roundings of it, and roots of such an overlap: whichever form takes them
+    for step in range(-4, 5):
+        d = np.full(N, 1.0)
+        d[5::3] = 0.125 * (1.0 + step * 2.0 ** -23)
+        s = np.diag(d)
+        h = np.diag(np.where(np.arange(N) % 2, d, -d))
+        with _context(h if f in ("density", "overlap") else s, 2) as c:
+            if f == "overlap":
+                c.set_overlap(_full(s, 2))
+            elif f != "density":
+                c.set_function(f)
+            c.build_density()
+            c.get_trace()
+            got = _dense(c.get_density(), N, 2)
+        below = np.diag(np.where(np.arange(N) % 2, 0.0, 1.0))
+        ref = {"inv_sqrt": np.diag(d ** -0.5), "density": below, "overlap": below / d}[f]
+        assert _error(got, ref) <= TOL, step
