@@ -962,7 +962,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
                 if (bad) atomicCAS(a.status, kOk, kErrNonfinite);
             }
             const int64_t* F = jb.M[0];
-            const double fs = ldexp(1.0, -ss.e);
+            const double fs = bad ? NAN : ldexp(1.0, -ss.e);
             auto frow = [&](int q, int i) -> double { return fs * from_fixed(ld1(F + mat_at(k, i, s.own + q))); };
             if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch);  // 1/2 (I - T)
             fence_proxy_async_smem();
@@ -994,6 +994,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
                 F = jb.M[2];
                 fs = ldexp(1.0 / b, 2 * ez);
             }
+            if (bad) fs = NAN;
             auto frow = [&](int q, int i) -> double { return fs * from_fixed(ld1(F + mat_at(k, i, s.own + q))); };
             if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, frow, ls_smem, scratch, false);
             fence_proxy_async_smem();
@@ -1068,13 +1069,15 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_ns_fp64(const __grid_const
             pass_transposed(L, U, s.own, s.bown, jb.P[2], w, k, 1);
             slice_product(sh, jb.P[1], jb.P[2], k, w, U, false);
             if (sh->abort) break;
-            const double fs = ldexp(1.0, 2 * el);
+            const double fs = bad ? NAN : ldexp(1.0, 2 * el);
             auto prow = [&](int q, int i) -> double { return fs * from_fixed(ld1(U + mat_at(k, i, q))); };
             if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, prow, ls_smem, scratch, false, a.Sv);
             fence_proxy_async_smem();
             continue;
         }
-        auto xrow = [&](int q, int i) -> double { return from_fixed(ld1(X + mat_at(k, i, s.own + q))); };
+        // (a submatrix that failed: NaN, not what the slot holds)
+        const double fs = bad ? NAN : 0x1p-62;
+        auto xrow = [&](int q, int i) -> double { return fs * static_cast<double>(ld1(X + mat_at(k, i, s.own + q))); };
         if (lead) finish_column(s, a.pv, a.H, a.D, a.partial, xrow, ls_smem, scratch);
         fence_proxy_async_smem();
         }
@@ -1306,6 +1309,10 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_dense_density_noalloc(cons
         for (int r = cluster_rank() * kSliceWarps + (threadIdx.x >> 5); r < n; r += cluster_size() * kSliceWarps)
             for (int c = threadIdx.x & 31; c < n; c += 32) {  // 1/2 (I - X) in units of 2^-63: up to 2^63
                 const int64_t x = ld1(X + mat_at(jb.k, c, r)), one = r == c ? kFixedOne : 0;
+                if (bad) {  // (no iterate: the array holds the last call's)
+                    Dout[static_cast<int64_t>(r) * n + c] = NAN;
+                    continue;
+                }
                 const bool negative = x > one;
                 const uint64_t d = static_cast<uint64_t>(one) - static_cast<uint64_t>(x);
                 Dout[static_cast<int64_t>(r) * n + c] = fixed_to_double(negative ? 0 - d : d, negative, -63);

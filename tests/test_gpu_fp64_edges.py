@@ -111,3 +111,64 @@ def test_one_negative_eigenvalue_is_not_positive_definite(f, n, coupling):
             except SmxError as e:
                 assert e.status in (_lib.ERR_NOCONV, _lib.ERR_NONFINITE)
     assert accepted == []
+
+
+def test_a_failed_submatrix_leaves_no_numbers():
+    # D of a submatrix that failed is NaN, not what the work memory held; the others' columns stand
+    from paper_2205_14741_gb300 import SmxError, SubmatrixDensity, _lib, dense_density_noalloc
+
+    s = make_mixed_block_system([4] * 90, r_c=5.0, ell=1.5, seed=3)
+    off = O.block_value_offsets(s.block_size, s.col_ptr, s.row_idx)
+    diag = [int(k) for j in range(90) for k in range(s.col_ptr[j], s.col_ptr[j + 1]) if s.row_idx[k] == j]
+    vals = s.values * 0.05
+    for k in diag:
+        vals[off[k]:off[k + 1]] = np.eye(4).ravel()
+    bad = vals.copy()
+    bad[off[diag[7]]] = -0.8  # the submatrices that hold block 7 are not positive definite
+    hit = {j for j in range(90) if 7 in s.row_idx[s.col_ptr[j]:s.col_ptr[j + 1]]}
+    assert 0 < len(hit) < 90
+    out = torch.empty(vals.size, dtype=torch.float64, device="cuda")
+    with SubmatrixDensity.from_system(s) as c:
+        c.set_function("inv_sqrt")
+        c.set_values(vals)
+        c.build_density()
+        good = c.get_density()
+        c.set_values(bad)
+        with pytest.raises(SmxError) as e:
+            c.build_density()
+            c.get_trace()
+        assert e.value.status == _lib.ERR_NONFINITE
+        got = c.get_density(out).cpu().numpy()  # (a device copy reports no status)
+    for j in range(90):
+        part = slice(int(off[s.col_ptr[j]]), int(off[s.col_ptr[j + 1]]))
+        assert np.all(np.isnan(got[part])) if j in hit else np.array_equal(got[part], good[part])
+
+    h = torch.eye(40, dtype=torch.float64, device="cuda")
+    d = torch.zeros_like(h)
+    dense_density_noalloc(h, 40, 0.0, d)
+    h[3, 5] = h[5, 3] = float("inf")
+    with pytest.raises(SmxError) as e:
+        dense_density_noalloc(h, 40, 0.0, d)
+    assert e.value.status == _lib.ERR_NONFINITE
+    assert bool(torch.isnan(d).all())
+
+
+def test_a_nonfinite_snapshot_leaves_no_numbers():
+    from paper_2205_14741_gb300 import SmxError, SubmatrixDensity, _lib
+
+    s = make_mixed_block_system([4] * 90, r_c=5.0, ell=1.5, seed=3)
+    off = O.block_value_offsets(s.block_size, s.col_ptr, s.row_idx)
+    with SubmatrixDensity.from_system(s) as c:
+        c.set_electron_count(180.0, max_steps=3, tol=1e-9)
+        c.solve_mu()
+        bad = s.values.copy()
+        k = next(k for k in range(s.col_ptr[11], s.col_ptr[12]) if s.row_idx[k] == 11)
+        bad[off[k]] = np.nan
+        c.set_values(torch.from_numpy(bad).cuda(), on_device=True)
+        with pytest.raises(SmxError) as e:
+            c.solve_mu()
+        assert e.value.status == _lib.ERR_NONFINITE
+        got = c.get_density(torch.empty(bad.size, dtype=torch.float64, device="cuda")).cpu().numpy()
+    for j in range(90):
+        if 11 in s.row_idx[s.col_ptr[j]:s.col_ptr[j + 1]]:
+            assert np.all(np.isnan(got[off[s.col_ptr[j]]:off[s.col_ptr[j + 1]]])), j
