@@ -1210,8 +1210,10 @@ static cudaError_t launch_form(K kernel, const A& a, int slots, int max_n, const
     return launch_clusters(kernel, slots, 1 << i, st, a);
 }
 
-cudaError_t device_clusters(int* room) {
-    cudaError_t e = cudaFuncSetAttribute(k_ns_fp64<kFormSign>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSliceSmem));
+// room[i]: how many clusters of 2^i CTAs of the kernel the device holds at once, i = 0 .. 3.
+template <class K>
+static cudaError_t kernel_clusters(K kernel, int* room) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSliceSmem));
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
@@ -1223,10 +1225,12 @@ cudaError_t device_clusters(int* room) {
         cfg.dynamicSmemBytes = kSliceSmem;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        e = cudaOccupancyMaxActiveClusters(&room[i], k_ns_fp64<kFormSign>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&room[i], kernel, &cfg);
     }
     return e;
 }
+
+cudaError_t device_clusters(int* room) { return kernel_clusters(k_ns_fp64<kFormSign>, room); }
 
 cudaError_t launch_ns_fp64(const NsFp64Args& a, int slots, int max_n, int max_nblk, const int* room, cudaStream_t st) {
     if (sizeof(int) * (static_cast<size_t>(max_nblk) + 1) > kSliceSmem - 1024) return cudaErrorInvalidValue;
@@ -1336,6 +1340,8 @@ std::mutex g_noalloc_mutex;
 // per device: the array's device address and the context it was looked up in
 uint8_t* g_noalloc_ptr[smx::kNoAllocMaxDevices] = {};
 CUcontext g_noalloc_ctx[smx::kNoAllocMaxDevices] = {};
+// the CTAs of the largest cluster it has room for there
+int g_noalloc_cluster[smx::kNoAllocMaxDevices] = {};
 
 // The current driver context, through the runtime's driver entry point (no link to libcuda).
 CUcontext current_context() {
@@ -1362,6 +1368,7 @@ extern "C" smx_status smx_dense_density_noalloc(const double* h_dev, int32_t n, 
     if (cudaGetDevice(&dev) != cudaSuccess) return SMX_ERR_CUDA;
     if (dev < 0 || dev >= smx::kNoAllocMaxDevices) return SMX_ERR_UNSUPPORTED;
     uint8_t* scratch = nullptr;
+    int largest = 1;
     {
         // set-up once per device, with that device current: the host-side name
         // of a __device__ array is not a device address, so look the address up.
@@ -1372,22 +1379,19 @@ extern "C" smx_status smx_dense_density_noalloc(const double* h_dev, int32_t n, 
         if (!g_noalloc_ptr[dev] || g_noalloc_ctx[dev] != cur) {
             void* p = nullptr;
             if (cudaGetSymbolAddress(&p, smx::g_noalloc_scratch) != cudaSuccess || !p) return SMX_ERR_CUDA;
-            if (cudaFuncSetAttribute(smx::k_dense_density_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smx::kSliceSmem)) != cudaSuccess)
-                return SMX_ERR_CUDA;
+            int room[4] = {0, 0, 0, 0};
+            if (smx::kernel_clusters(smx::k_dense_density_noalloc, room) != cudaSuccess) return SMX_ERR_CUDA;
+            g_noalloc_cluster[dev] = room[3] > 0 ? 8 : room[2] > 0 ? 4 : room[1] > 0 ? 2 : 1;
             g_noalloc_ptr[dev] = static_cast<uint8_t*>(p);
             g_noalloc_ctx[dev] = cur;
         }
         scratch = g_noalloc_ptr[dev];
+        largest = g_noalloc_cluster[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // (a device without room for the cluster takes a smaller one)
-    cudaError_t e = cudaErrorInvalidValue;
-    for (int size = smx::cluster_for(n); size >= 1 && e != cudaSuccess; size >>= 1) {
-        e = smx::launch_clusters(smx::k_dense_density_noalloc, 1, size, st, h_dev, static_cast<int>(n), mu, d_dev, scratch, 1e-7f, 100);
-        if (e != cudaSuccess) cudaGetLastError();
-    }
-    if (e != cudaSuccess) return SMX_ERR_CUDA;
+    const int size = smx::cluster_for(n) < largest ? smx::cluster_for(n) : largest;
+    if (smx::launch_clusters(smx::k_dense_density_noalloc, 1, size, st, h_dev, static_cast<int>(n), mu, d_dev, scratch, 1e-7f, 100) != cudaSuccess)
+        return SMX_ERR_CUDA;
     int* const head = reinterpret_cast<int*>(scratch + smx::kNoAllocBytes);
     if (smx::launch_dense_graded(h_dev, static_cast<int>(n), mu, d_dev, scratch, 1e-7, 100, head + 2, reinterpret_cast<double*>(head + 4), head, st) !=
         cudaSuccess)

@@ -519,8 +519,11 @@ cudaError_t launch_graded_setup(const NonorthSetupArgs& a, int slots, cudaStream
 
 cudaError_t launch_dense_graded(const double* H, int n, double mu, double* D, uint8_t* slot, double tau, int max_iter, int* graded, const double* b,
                                 int* status, cudaStream_t st) {
-    k_dense_graded<<<1, kThreads, 0, st>>>(H, n, mu, D, slot, tau, max_iter, graded, b, status);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};  // (an error of the caller's that is pending is neither taken for one of this launch nor cleared)
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, k_dense_graded, H, n, mu, D, slot, tau, max_iter, graded, b, status);
 }
 
 }  // namespace smx

@@ -17,7 +17,7 @@ def source(name):
 
 def body(text, name):
     """The text of the function `name`, from its opening brace to the matching one."""
-    for m in re.finditer(r"\b%s\(" % name, text):
+    for m in re.finditer(r"\b%s\(" % name, text):  # (its definition: followed by a brace)
         i, depth = m.end(), 1
         while depth:  # past the parameters
             depth += {"(": 1, ")": -1}.get(text[i], 0)
@@ -81,3 +81,12 @@ def test_bound_vectors_leave_the_stage_area_before_it_ends():
     planes, tile, stages = (int(re.search(r"%s = (\d+)" % c, slices).group(1)) for c in ("kSlicePlanes", "kSliceTile", "kSliceStages"))
     assert 16 * rows <= stages * planes * 32 * (128 + tile)
     assert "k <= kBoundSharedRows ?" in body(text, "first_bound")
+
+
+def test_dense_entry_point_keeps_a_pending_error():
+    # the runtime's last error is the caller's: it is not read (which clears it), and a launch is tried once, with a
+    # cluster that the device has been asked about
+    text = source("k_ns_fp64.cu")
+    b = body(text, "smx_dense_density_noalloc")
+    assert "cudaGetLastError" not in b and b.count("launch_clusters(") == 1 and "kernel_clusters(" in b
+    assert "cudaGetLastError" not in body(source("k_ns_graded.cu"), "launch_dense_graded")
