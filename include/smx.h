@@ -99,8 +99,8 @@ typedef enum {
  *                   the finite-temperature counterpart of Eq. 14 (beta from
  *                   smx_set_fermi_beta): per submatrix, tanh by a Taylor start at
  *                   a small argument and k doublings tanh(2x) = 2 tanh(x)/(1 + tanh^2 x),
- *                   each with a Newton-Schulz inverse of I + T^2 (products only;
- *                   about 7 + 11 k products, k = log2(8 beta G_j)). */
+ *                   each with an inverse of I + T^2 in products only (6 + 12 k
+ *                   products in all, k = log2(8 beta G_j)). */
 typedef enum {
     SMX_FN_DENSITY = 0,
     SMX_FN_INV_SQRT = 1,
@@ -268,7 +268,9 @@ smx_status smx_set_overlap(smx_ctx* ctx, const double* values, int32_t on_device
  * Newton-Schulz, scatter, trace and energy.  Asynchronous on the context
  * stream except for a small host round trip when the filtered pattern must
  * be recomputed.  Errors: SMX_ERR_NONFINITE (input), SMX_ERR_OOM, SMX_ERR_CUDA,
- * SMX_ERR_UNSUPPORTED (a submatrix larger than this build handles). */
+ * SMX_ERR_UNSUPPORTED (a submatrix larger than this build handles).  In the
+ * 64-bit forms the columns of a submatrix that ended in SMX_ERR_NONFINITE are
+ * NaN in D. */
 smx_status smx_build_density(smx_ctx* ctx);
 
 /* Finds Eq. 14's mu by bisection (see smx_set_electron_count) and leaves the
@@ -431,7 +433,8 @@ smx_status smx_get_submatrix_info(smx_ctx* ctx, int32_t* dims, int32_t* iters, d
  * device).
  * Computes D = 1/2 (I - sign(H - mu I)) of one dense symmetric H by FP64
  * Newton-Schulz iteration (Eq. 13 and Eq. 14 with S = I on a single dense
- * matrix; one cluster of up to eight CTAs; the same iteration as the FP64 form of smx_build_density).
+ * matrix; one cluster of up to eight CTAs; the same arithmetic and iteration as SMX_FP64 of
+ * smx_build_density).  D is NaN after SMX_ERR_NONFINITE.
  *  h_dev       : device double[n*n], row-major, symmetric (read only).
  *  n           : 1 <= n <= 256; larger n returns SMX_ERR_ARG.
  *  mu          : finite chemical potential.

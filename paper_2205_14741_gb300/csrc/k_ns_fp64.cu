@@ -1198,11 +1198,14 @@ static int cluster_for(int n) {
     return tiles >= 8 ? 8 : tiles >= 4 ? 4 : tiles >= 2 ? 2 : 1;
 }
 
-// CTAs per submatrix: as many as find room at once for all n_subs of them, at most cluster_for(max_n);
-// with more submatrices than SMs each keeps to one (two SMs that share a submatrix also share its
-// barriers, reductions and short products, so they finish fewer of them).  Builds measured with one CTA each and
-// with clusters: 32 submatrices of n = 66 .. 120 (four each) 595 and 301 us, one of n = 192 (eight) 944 and
-// 275 us.  room[i]: clusters of 2^i CTAs the device holds at once (device_clusters).
+// CTAs per submatrix: as many as find room at once for all n_subs of them, at most cluster_for(max_n); one each where
+// not even pairs do.  room[i]: clusters of 2^i CTAs the device holds at once (device_clusters; 76 pairs here, about 36
+// fours and 18 eights).  Density builds of n_subs submatrices of n = 120 .. 204 with one CTA, two and four each, us:
+//   8: 985 / 614 / 447 (eight: 331)   32: 1002 / 622 / 456    37: 1008 / 620 / 485    64: 1014 / 637 / 790
+//   75: 1027 / 652 / 960    96: 1046 / 961 / 1140    128: 1082 / 1092 / 1515    256: 2042 / 2034 / 2928    304: 2166 / 2327 / 3402
+// At the lines the larger cluster still wins where all fit, and four lose as soon as they do not.  Pairs past 76 gain
+// where one CTA each leaves a short last wave (152: 1958 / 1315, 200: 2007 / 1588) and lose from about 300 on;
+// telling those apart needs the submatrices' sizes, which the rule does not look at.
 template <class K, class A>
 static cudaError_t launch_form(K kernel, const A& a, int slots, int max_n, const int* room, cudaStream_t st) {
     int size = cluster_for(max_n), i = size == 8 ? 3 : size == 4 ? 2 : size == 2 ? 1 : 0;

@@ -235,11 +235,9 @@ __device__ __forceinline__ void tc_mma_f16(uint32_t d_tmem, uint64_t a_desc, uin
 }
 
 // One lane of a converged warp.  A loop that issues tcgen05.mma runs inside a branch on this
-// predicate, not on lane == 0: knowing that the branch holds one lane, the compiler moves the
-// descriptors to the uniform registers the instruction needs directly; else each instruction takes
-// a loop over the possible lanes, about 150 cycles whatever its size.  Measured (M = 128, K = 16,
-// one SM): 12 instructions of 192 columns on average in 2170 cycles with lane == 0, in 1154 with
-// this one (2 columns a cycle, the tensor cores' rate); N = 64 in 65 cycles instead of 177.
+// predicate, not on lane == 0.  Measured (M = 128, K = 16, one SM): 12 instructions of 192 columns on
+// average in 2170 cycles with lane == 0, in 1154 with this one (2 columns a cycle, the tensor
+// cores' rate); N = 64 in 65 cycles instead of 177.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));

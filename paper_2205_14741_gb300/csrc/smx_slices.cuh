@@ -14,7 +14,8 @@
 // an accumulator; g = 2 .. 8 (28 pairs) are kept.  The epilogue adds the seven accumulators as
 // integers with their weights, so the only errors of a product are the 2^-57 rounding of the
 // operands and the dropped weights g >= 9: about 3.4e-17 sqrt(K / 158) per entry, below the
-// rounding of a chain of K FP64 fused multiply-adds on entries of order 0.1 .. 1.
+// rounding of a chain of K FP64 fused multiply-adds on entries of order 0.1 .. 1.  (In units of the matrix's
+// longest row: rows much shorter than that would lose digits, and are not multiplied here; kGraded.)
 //
 // Exactness.  The rows of both operands have 2-norms of at most 1.05 (the callers scale by a
 // power of two where it takes one).  So |sum_k d_1 d_j| <= 256 * 1.05 * 128 sqrt(K) for j > 1, and
