@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kThreads) k_ns_graded(const __grid_constant__ 
             bool bad;
             const double* F = tanh_doublings(w, T, s.ld, a.bound[j], a.beta, products, bad);
             record(products, true, bad);
-            auto row = [&](int q, int i) -> double { return F[own + static_cast<int64_t>(q) * n + i]; };
+            auto row = [&](int q, int i) -> double { return bad ? NAN : F[own + static_cast<int64_t>(q) * n + i]; };
             finish_column(s, a.pv, a.H, a.D, a.partial, row, ls_smem, scratch);  // 1/2 (I - T)
         } else if (a.function != kFnDensity) {
             // A^-1/2 = Z / sqrt(b), A^1/2 = sqrt(b) Y, A^-1 = Z Z / b
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kThreads) k_ns_graded(const __grid_constant__ 
             const bool inv = a.function == kFnInv;
             if (inv) thin_product(n, r.Z, n, r.Z + own, n, 1, s.bown, r.T, false, 1.0 / b);
             const double* F = inv ? r.T : (a.function == kFnSqrt ? r.Y : r.Z) + own;
-            const double fs = inv ? 1.0 : a.function == kFnSqrt ? sqrt(b) : 1.0 / sqrt(b);
+            const double fs = r.bad ? NAN : inv ? 1.0 : a.function == kFnSqrt ? sqrt(b) : 1.0 / sqrt(b);
             const int64_t sq = inv ? 1 : n, si = inv ? s.bown : 1;
             auto row = [&](int q, int i) -> double { return fs * F[q * sq + i * si]; };
             finish_column(s, a.pv, a.H, a.D, a.partial, row, ls_smem, scratch, false);
@@ -415,10 +415,10 @@ __global__ void __launch_bounds__(kThreads) k_ns_graded(const __grid_constant__ 
                 const double* L = a.Lc + s.t_off;
                 thin_product(n, r.X, n, L + static_cast<int64_t>(s.own) * s.ld, s.ld, 1, s.bown, r.Y, true, 1.0);
                 thin_product(n, L, s.ld, r.Y, 1, s.bown, s.bown, r.Z, false, 0.5);
-                auto row = [&](int q, int i) -> double { return r.Z[static_cast<int64_t>(i) * s.bown + q]; };
+                auto row = [&](int q, int i) -> double { return r.bad ? NAN : r.Z[static_cast<int64_t>(i) * s.bown + q]; };
                 finish_column(s, a.pv, a.H, a.D, a.partial, row, ls_smem, scratch, false, a.Sv);
             } else {
-                auto row = [&](int q, int i) -> double { return r.X[own + static_cast<int64_t>(q) * n + i]; };
+                auto row = [&](int q, int i) -> double { return r.bad ? NAN : r.X[own + static_cast<int64_t>(q) * n + i]; };
                 finish_column(s, a.pv, a.H, a.D, a.partial, row, ls_smem, scratch);
             }
         }
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(kThreads) k_dense_graded(const double* __restr
     const Work w = slot_work(n, slot, As, Bs, scratch);
     const SignResult r = sign_iteration(w, H, n, mu, *b, false, -1.0, nullptr, max_iter, tau);
     each(n, [&](int i, int c) {
-        D[static_cast<int64_t>(i) * n + c] = 0.5 * ((i == c ? 1.0 : 0.0) - r.X[static_cast<int64_t>(i) * n + c]);
+        D[static_cast<int64_t>(i) * n + c] = r.bad ? NAN : 0.5 * ((i == c ? 1.0 : 0.0) - r.X[static_cast<int64_t>(i) * n + c]);
     });
     if (threadIdx.x == 0) {
         status[0] = r.bad ? kErrNonfinite : r.conv ? kOk : kErrNoconv;

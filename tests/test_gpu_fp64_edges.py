@@ -113,7 +113,8 @@ def test_one_negative_eigenvalue_is_not_positive_definite(f, n, coupling):
     assert accepted == []
 
 
-def test_a_failed_submatrix_leaves_no_numbers():
+@pytest.mark.parametrize("entry", [-0.8, -1e-3])  # rows of one size, and a small one (FP64 multiply-adds)
+def test_a_failed_submatrix_leaves_no_numbers(entry):
     # D of a submatrix that failed is NaN, not what the work memory held; the others' columns stand
     from paper_2205_14741_gb300 import SmxError, SubmatrixDensity, _lib, dense_density_noalloc
 
@@ -124,7 +125,9 @@ def test_a_failed_submatrix_leaves_no_numbers():
     for k in diag:
         vals[off[k]:off[k + 1]] = np.eye(4).ravel()
     bad = vals.copy()
-    bad[off[diag[7]]] = -0.8  # the submatrices that hold block 7 are not positive definite
+    k = diag[7]
+    bad[off[k]:off[k] + 4] *= 0.0
+    bad[off[k]] = entry  # the submatrices that hold block 7 are not positive definite
     hit = {j for j in range(90) if 7 in s.row_idx[s.col_ptr[j]:s.col_ptr[j + 1]]}
     assert 0 < len(hit) < 90
     out = torch.empty(vals.size, dtype=torch.float64, device="cuda")
