@@ -4,8 +4,8 @@
 // (smx_slices.cuh) holds every entry in units of the submatrix's largest row.  For A = D S0 D with a well-conditioned
 // S0 the relative error of A^-1/2 stays at some 1e-15 in the one and grows as 1 / d^2 in the other (d the smallest
 // entry of D).  So the kernels of k_ns_fp64.cu put such submatrices on a list (kGraded there says which) and leave
-// them to the kernels below, which follow every launch of those and return at once when the list is empty (1 .. 3 us of
-// a build: dense n = 192 275 -> 277 us).
+// them to the kernels below, which follow every launch of those and return at once when the list is empty (a build's
+// also forms the sums of its partials, which had a launch of their own; dense n = 192 275 -> 277 us).
 //
 // A persistent CTA takes one submatrix at a time and keeps its matrices in a slot of the other kernels' work memory.
 // Bound by the FP64 units, which take about 16 cycles per warp instruction and SM: products in 64 x 64 tiles from
@@ -340,9 +340,17 @@ __device__ __forceinline__ int next_listed(GradedList* list, int* job_s) {
     __syncthreads();
     return *job_s;
 }
-// The last CTA empties the list.
-__device__ __forceinline__ void release_list(GradedList* list) {
-    if (threadIdx.x == 0 && atomicAdd(&list->done, 1) == static_cast<int>(gridDim.x) - 1) list->count = list->next = list->done = 0;
+// The last CTA empties the list, and gets true (job_s: a word of shared memory).
+__device__ __forceinline__ bool release_list(GradedList* list, int* job_s) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        *job_s = atomicAdd(&list->done, 1) == static_cast<int>(gridDim.x) - 1;
+        if (*job_s) list->count = list->next = list->done = 0;
+    }
+    __syncthreads();
+    __threadfence();
+    return *job_s != 0;
 }
 
 __device__ __forceinline__ Work slot_work(int n, uint8_t* slot, double (*As)[kTile + 1], double (*Bs)[kTile + 1], double* scratch) {
@@ -357,7 +365,7 @@ __device__ __forceinline__ Work slot_work(int n, uint8_t* slot, double (*As)[kTi
 
 }  // namespace
 
-// The listed submatrices of a build.
+// The listed submatrices of a build, then (the last CTA; the first if none is listed) the sums of its partials.
 __global__ void __launch_bounds__(kThreads) k_ns_graded(const __grid_constant__ NsFp64Args a) {
     __shared__ double As[kKc][kTile + 1], Bs[kKc][kTile + 1], scratch[64];
     __shared__ SubDesc s;
@@ -365,7 +373,10 @@ __global__ void __launch_bounds__(kThreads) k_ns_graded(const __grid_constant__ 
     extern __shared__ int ls_smem[];
     if (a.skip && *a.skip) return;
     const int count = a.graded->count;
-    if (count == 0) return;
+    if (count == 0) {
+        if (a.sums && blockIdx.x == 0) sum_partials(a.partial, a.n_cols, &a.sums->trace, &a.sums->energy, scratch);
+        return;
+    }
     uint8_t* slot = a.ws + static_cast<int64_t>(blockIdx.x) * a.slot_bytes;
     for (;;) {
         const int job = next_listed(a.graded, &job_s);
@@ -423,7 +434,7 @@ __global__ void __launch_bounds__(kThreads) k_ns_graded(const __grid_constant__ 
             }
         }
     }
-    release_list(a.graded);
+    if (release_list(a.graded, &job_s) && a.sums) sum_partials(a.partial, a.n_cols, &a.sums->trace, &a.sums->energy, scratch);
 }
 
 // The listed submatrices of a non-orthogonal setup: L = A_S^-1/2 into Lc, M = L A_H L into Mc and its interval.
@@ -482,7 +493,7 @@ __global__ void __launch_bounds__(kThreads) k_graded_setup(const __grid_constant
             a.lohi[2 * s.col + 1] = r.bad ? 0.0 : hi;
         }
     }
-    release_list(a.graded);
+    release_list(a.graded, &job_s);
 }
 
 // The dense entry point's matrix, when *graded (cleared here) says that its rows are of very different size: D = 1/2 (I

@@ -737,23 +737,6 @@ cudaError_t launch_gather_bound_f32(const SubDesc* subs, int n_subs, int max_nbl
     return launch_gather<float>(subs, n_subs, max_nblk, max_n, bmax, uniform, pv, H32, mu, T32, bound, ex, st);
 }
 
-// Deterministic sums of partial[0, n_cols) by one block (each thread adds a fixed
-// strided subset in order, then a fixed tree) into sc->trace, sc->energy.
-__device__ void sum_partials(const double2* partial, int n_cols, DevScalars* sc, double* scratch) {
-    double tr = 0.0, en = 0.0;
-    for (int c = threadIdx.x; c < n_cols; c += blockDim.x) {
-        const double2 p = __ldcg(partial + c);
-        tr += p.x;
-        en += p.y;
-    }
-    tr = block_sum(tr, scratch);
-    en = block_sum(en, scratch);
-    if (threadIdx.x == 0) {
-        sc->trace = tr;
-        sc->energy = en;
-    }
-}
-
 // One CTA per submatrix: scatter of the saved owner columns (Fig. 2 step (iii);
 // Eq. 14: D[R_j, j] = 1/2 (E_j - X[:, own]), X symmetric, so the saved column q
 // is X's row own + q), then (the last CTA) the sums of a8.
@@ -879,7 +862,7 @@ __global__ void __launch_bounds__(256) k_scatter_owner(const SubDesc* __restrict
     __syncthreads();
     if (!last_s) return;
     __threadfence();
-    sum_partials(partial, n_cols, sc, scratch);
+    sum_partials(partial, n_cols, &sc->trace, &sc->energy, scratch);
     if (tid == 0) {
         sc->scatter_done = 0u;
         sc->ns_counter = 0;  // the Newton-Schulz launch before this one is complete
@@ -908,7 +891,7 @@ __global__ void __launch_bounds__(1024) k_reduce(const double2* __restrict__ par
                                                  const int* skip) {
     if (skip && *skip) return;
     __shared__ double scratch[32];
-    sum_partials(partial, n_cols, sc, scratch);
+    sum_partials(partial, n_cols, &sc->trace, &sc->energy, scratch);
 }
 
 cudaError_t launch_reduce(const double2* partial, int n_cols, DevScalars* sc, cudaStream_t st, const int* skip) {

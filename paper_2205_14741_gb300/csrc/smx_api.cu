@@ -692,6 +692,10 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
             a.max_iter = 100;
             a.use_model = model ? 1 : 0;
             if (model && c->model_gap) a.pred = dp<float>(c->d_pred);
+            if (k + 2 == c->chunk_start.size()) {
+                a.sums = sc;
+                a.n_cols = B;
+            }
             if (c->have_S) {
                 a.Mc = dp<double>(c->d_Mc);
                 a.Lc = dp<double>(c->d_Lc);
@@ -757,8 +761,7 @@ static smx_status build_at(smx_ctx* c, double mu, const double* mu_dev = nullptr
         c->kernel_launches += 1;
         c->ns_launches += 1;
     }
-    if (c->precision == SMX_FP64 || finish) {
-        // the tensor-core scatter sums the partials itself
+    if (finish) {  // (otherwise the tensor-core scatter or the listed submatrices' kernel sums the partials)
         SMX_CUDA(launch_reduce(dp<double2>(c->d_partial), B, sc, st, skip));
         c->kernel_launches += 1;
     }

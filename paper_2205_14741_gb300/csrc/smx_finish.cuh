@@ -54,4 +54,22 @@ __device__ void finish_column(const SubDesc& s, const PatternView& pv, const dou
     if (threadIdx.x == 0) partial[s.col] = make_double2(tr, en);
 }
 
+// Deterministic sums of partial[0, n_cols) by 256 threads of one block (each adds a fixed strided
+// subset in order, then a fixed tree), which all threads call.
+__device__ __forceinline__ void sum_partials(const double2* partial, int n_cols, double* trace, double* energy, double* scratch) {
+    double tr = 0.0, en = 0.0;
+    if (threadIdx.x < 256)
+        for (int c = threadIdx.x; c < n_cols; c += 256) {
+            const double2 p = __ldcg(partial + c);
+            tr += p.x;
+            en += p.y;
+        }
+    tr = block_sum(tr, scratch);
+    en = block_sum(en, scratch);
+    if (threadIdx.x == 0) {
+        *trace = tr;
+        *energy = en;
+    }
+}
+
 }  // namespace smx

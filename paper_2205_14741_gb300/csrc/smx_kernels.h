@@ -140,6 +140,8 @@ struct NsFp64Args {
     const int32_t* root_graded = nullptr;  // per block column: L_j's rows are of very different size
     double mu = 0.0;
     GradedList* graded;  // empty at launch and afterwards
+    DevScalars* sums = nullptr;  // the kernel of the listed submatrices forms the build's sums here (the last chunk's)
+    int n_cols = 0;              // ... over this many partials
     // learned bound: predictions per block column ([2 j + 1] = delta_hat / G_j); see NsTcArgs::pred
     const float* pred = nullptr;
     // FP64 finishing steps after a low-precision bulk phase (> 0): T holds the bulk phase's last

@@ -221,9 +221,10 @@ def test_graded_and_other_submatrices_in_one_build():
         ref = density_submatrix(s.block_size, s.col_ptr, s.row_idx, s.values, 0.0)
         # the oracle's eigendecomposition sees the small rows to 2^-53 of the large ones: to 1e-10 of their own size
         assert float(np.max(np.abs(whole - ref.values))) <= 1e-8
+        assert abs(trace - ref.trace) <= 1e-8 * s.n
         c.set_staging_limit(1 << 20)
         c.build_density()
-        assert np.array_equal(c.get_density(), whole)
+        assert np.array_equal(c.get_density(), whole) and c.get_trace()[0] == trace
         c.set_electron_count(trace - 3.0, max_steps=6, tol=1e-12)
         c.solve_mu()
         host = c.get_density(), c.get_trace()
