@@ -206,18 +206,18 @@ __device__ __noinline__ bool pass_iterate(const double* __restrict__ src, int ld
 __device__ __noinline__ float pass_residual(const int64_t* S, uint8_t* planes, int n, int k, int up, uint64_t f,
                                             unsigned long long* sums = nullptr) {
     float r2 = 0.0f;
-    const uint32_t most = 0x40400000u >> up;  // 1 + 2^-8 in units of 2^-30 (2^-up)
+    const uint64_t most = static_cast<uint64_t>(kFixedOne + (kFixedOne >> 8)) >> up;
     slice_pass<1>(k, k, planes, [&](int r, int c, int64_t (&v)[1][8]) { ld8(S, k, r, c, v[0]); },
                   [&](int r, int c, const int64_t (&v)[1][8], int64_t (&q)[8]) {
                       float row = 0.0f;
-                      uint32_t top = 0;
+                      uint64_t top = 0;
 #pragma unroll
                       for (int i = 0; i < 8; ++i) {
                           const int64_t one = r == c + i && r < n ? kFixedOne : 0, s = v[0][i] << up;
                           const float d = fixed_float(one - s);
                           r2 = fmaf(d, d, r2);
                           row = fmaf(d, d, row);
-                          top = max(top, static_cast<uint32_t>(abs_fixed(v[0][i]) >> 32));
+                          top = max(top, abs_fixed(v[0][i]));
                           q[i] = one - (f ? fixed_mul(s, f) : s);
                       }
                       if (sums) add_length(sums, r, top > most ? 0x1p28f : fminf(row * 0x1p-52f, 0x1p28f));
@@ -704,7 +704,7 @@ __device__ int coupled_steps(SliceShared* sh, const SliceJob& jb, const double* 
             const float z = longest(row_z);
             const int shift = z > 1.0f ? 1 : 0;
             ez += shift;
-            if (z > 2.25f * kLongest || longest(row_y) > kLongest || ez > 30) {
+            if (z > 2.25f * kLongest || longest(row_y) > kLongest || ez > 40) {
                 bad = true;
                 conv = false;
                 break;
